@@ -60,11 +60,11 @@ __global__ void k_gather_sum(const int* __restrict__ t0, const int* __restrict__
     out[i] = s;
 }
 
-std::vector<GTile> tiles64(const std::vector<GProb>& probs) {
+std::vector<GTile> square_tiles(const std::vector<GProb>& probs, int edge) {
     std::vector<GTile> t;
     for (int p = 0; p < (int)probs.size(); ++p)
-        for (int m0 = 0; m0 < probs[p].M; m0 += 64)
-            for (int n0 = 0; n0 < probs[p].N; n0 += 64) t.push_back({p, m0, n0, 0});
+        for (int m0 = 0; m0 < probs[p].M; m0 += edge)
+            for (int n0 = 0; n0 < probs[p].N; n0 += edge) t.push_back({p, m0, n0, 0});
     return t;
 }
 
@@ -73,11 +73,12 @@ void gemm64(const std::vector<GProb>& p, const std::vector<GSeg>& s, const doubl
             cudaStream_t st) {
     if (p.empty()) return;
     DBuf dp, ds, dt;
-    const std::vector<GTile> t = tiles64(p);
+    const F64Shape shape = f64_shape(p, s);
+    const std::vector<GTile> t = square_tiles(p, shape.tile);
     upload(dp, p, st);
     upload(ds, s, st);
     upload(dt, t, st);
-    launch_gemm_simt<double>(dp.as<GProb>(), ds.as<GSeg>(), dt.as<GTile>(), (int)t.size(), A, B, C, st);
+    launch_gemm_f64(dp.as<GProb>(), ds.as<GSeg>(), dt.as<GTile>(), (int)t.size(), shape.tile, shape, A, B, C, st);
 }
 
 GProb prob(int M, int N, long long c_off, int sam, int sak, int sbn, int sbk, int scm, int scn, int seg0, int nseg,

@@ -144,6 +144,14 @@ struct DiagTerm {
 template <class T>
 void launch_gemm_simt(const GProb* probs, const GSeg* segs, const GTile* tiles, int ntiles, const T* A, const T* B,
                       T* C, cudaStream_t st);
+// FP64 GEMM: `tile` = edge of a CTA's output tile, `ksplit` = warps that share it.  The tile list has
+// square tiles of `edge` (a multiple of shape.tile).
+struct F64Shape {
+    int tile, ksplit;
+};
+F64Shape f64_shape(const std::vector<GProb>& probs, const std::vector<GSeg>& segs);
+void launch_gemm_f64(const GProb* probs, const GSeg* segs, const GTile* tiles, int ntiles, int edge, F64Shape shape,
+                     const double* A, const double* B, double* C, cudaStream_t st);
 
 // Elementwise block kernels run one CTA per chunk of CHUNK elements of one job; `chunks`
 // lists (job, first element) for every chunk (built on the host, see make_chunks).

@@ -1,6 +1,6 @@
 // FP64 / memory-bound kernels of the two-site DMRG step.
 //
-//  * k_gemm64       grouped, strided FP64 GEMM (the parity-mode contractions of the projected
+//  * k_gemm_f64     grouped, strided FP64 GEMM (the parity-mode contractions of the projected
 //                   Hamiltonian and of the projected-operator updates, Sec. II)
 //  * k_copy/k_mix   block gathers, transposes, MPO channel mixing (memory-bound)
 //  * k_diag         diagonal of the projected Hamiltonian (Davidson preconditioner)
@@ -57,8 +57,178 @@ __device__ double block_sum(double v) {
 }
 
 // ------------------------------------------------------------------------------------------
-// Grouped SIMT GEMM (FP64 or FP32): 64x64 output tile per CTA, 256 threads, 4x4 per thread,
-// K chunks of 16.
+// Grouped FP64 GEMM.  This part issues 2 DFMA per clock and SM (one warp instruction every 64
+// clocks per scheduler), so the FP64 pipe is the bound and everything else is sized around it:
+//  * A warp owns a 16 x 16 output tile (a lane 2 rows x 4 columns) and skips the row octets and
+//    column quads outside the block, so small charge blocks pay for at most 8 x 4 padding.
+//    (64 x 64 CTA tiles computed their padding: a 15 x 15 block cost as much as a 64 x 64 one.)
+//  * Operands come straight from L1 / L2 into registers, four k at a time and one group ahead:
+//    a group is 32 DFMA = 2048 clocks of one scheduler, far above an L2 latency, and a 16-row
+//    K-contiguous panel re-reads its 128-byte lines from L1.  No shared memory, no barriers.
+//  * KS warps of a CTA share one tile with K (or the segments) split between them, summed in
+//    warp order at the end, so that a few tiles still reach every scheduler (see f64_shape).
+// FP64 matvec at the 24x8 cylinder's m = 500 bond, whole call: 3926 -> 1960 us; batches at f64_shape.
+// ------------------------------------------------------------------------------------------
+template <int MI, int NJ>
+__device__ __forceinline__ void f64_span(const double* pa0, const double* pa1, long long sak, const double* pb,
+                                         const int (&ob)[4], long long sbk, int n, double (&acc)[2][4]) {
+    constexpr int U = 4;
+    double a[U][MI], b[U][NJ];
+    int k = 0;
+    if (n >= U) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            a[u][0] = pa0[u * sak];
+            if (MI > 1) a[u][MI - 1] = pa1[u * sak];
+#pragma unroll
+            for (int j = 0; j < NJ; ++j) b[u][j] = pb[u * sbk + ob[j]];
+        }
+    }
+    for (; k + U <= n; k += U) {
+        double a2[U][MI], b2[U][NJ];
+        pa0 += U * sak;
+        pa1 += U * sak;
+        pb += U * sbk;
+        const bool more = k + 2 * U <= n;
+        if (more) {
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                a2[u][0] = pa0[u * sak];
+                if (MI > 1) a2[u][MI - 1] = pa1[u * sak];
+#pragma unroll
+                for (int j = 0; j < NJ; ++j) b2[u][j] = pb[u * sbk + ob[j]];
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+            for (int i = 0; i < MI; ++i)
+#pragma unroll
+                for (int j = 0; j < NJ; ++j) acc[i][j] = fma(a[u][i], b[u][j], acc[i][j]);
+        if (more) {
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+#pragma unroll
+                for (int i = 0; i < MI; ++i) a[u][i] = a2[u][i];
+#pragma unroll
+                for (int j = 0; j < NJ; ++j) b[u][j] = b2[u][j];
+            }
+        }
+    }
+    // the last n % U steps: loads first, then the products
+    const int rem = n - k;
+#pragma unroll
+    for (int u = 0; u < U - 1; ++u)
+        if (u < rem) {
+            a[u][0] = pa0[u * sak];
+            if (MI > 1) a[u][MI - 1] = pa1[u * sak];
+#pragma unroll
+            for (int j = 0; j < NJ; ++j) b[u][j] = pb[u * sbk + ob[j]];
+        }
+#pragma unroll
+    for (int u = 0; u < U - 1; ++u)
+        if (u < rem)
+#pragma unroll
+            for (int i = 0; i < MI; ++i)
+#pragma unroll
+                for (int j = 0; j < NJ; ++j) acc[i][j] = fma(a[u][i], b[u][j], acc[i][j]);
+}
+
+// One warp's part of a tile: all segments (KS = 1), or the segments ks, ks + KS, ... when there are
+// at least 4 KS of them, else the ks-th part of every segment's K.
+template <int MI, int NJ, int KS>
+__device__ __forceinline__ void f64_tile(const GProb& p, const GSeg* __restrict__ segs, const double* __restrict__ A,
+                                         const double* __restrict__ B, int m0, int n0, int ks, double (&acc)[2][4]) {
+    const int lane = threadIdx.x & 31, r = lane >> 2, c = lane & 3;
+    // rows and columns beyond the block read its last one; their results are not stored
+    const long long ra0 = (long long)min(m0 + r, p.M - 1) * p.sam, ra1 = (long long)min(m0 + 8 + r, p.M - 1) * p.sam;
+    const int nb = min(n0 + c, p.N - 1);
+    int ob[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) ob[j] = (min(n0 + c + 4 * j, p.N - 1) - nb) * p.sbn;
+    const bool whole = KS == 1 || p.nseg >= 4 * KS;
+    for (int s = (KS > 1 && whole) ? ks : 0; s < p.nseg; s += (KS > 1 && whole) ? KS : 1) {
+        const GSeg sg = segs[p.seg0 + s];
+        int k0 = 0, k1 = sg.K;
+        if (!whole) {
+            k0 = (int)((long long)sg.K * ks / KS);
+            k1 = (int)((long long)sg.K * (ks + 1) / KS);
+        }
+        const double* a = A + sg.a_off + (long long)k0 * p.sak;
+        const double* b = B + sg.b_off + (long long)k0 * p.sbk + (long long)nb * p.sbn;
+        f64_span<MI, NJ>(a + ra0, a + ra1, p.sak, b, ob, p.sbk, k1 - k0, acc);
+    }
+}
+
+// tiles[blockIdx.x / sub]: a tile of `sub` CTA tiles (row by row, edge / CT of them side by side).
+// KS = 1: CT = 32, four warps with a 16 x 16 tile each; KS > 1: CT = 16, KS warps on one tile.
+template <int KS>
+__global__ void __launch_bounds__(KS == 1 ? 128 : 32 * KS)
+    k_gemm_f64(const GProb* __restrict__ probs, const GSeg* __restrict__ segs, const GTile* __restrict__ tiles, int side,
+               const double* __restrict__ A, const double* __restrict__ B, double* __restrict__ C) {
+    constexpr int CT = KS == 1 ? 32 : 16;
+    __shared__ double part[KS > 1 ? KS - 1 : 1][KS > 1 ? 256 : 1];
+    const int sub = side * side, si = blockIdx.x % sub;
+    const GTile t = tiles[blockIdx.x / sub];
+    const GProb p = probs[t.prob];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    int m0 = t.m0 + (si / side) * CT, n0 = t.n0 + (si % side) * CT;
+    if (KS == 1) {
+        m0 += (warp >> 1) * 16;
+        n0 += (warp & 1) * 16;
+    }
+    if (m0 >= p.M || n0 >= p.N) return;              // whole warps (KS = 1), whole CTAs (KS > 1)
+    double acc[2][4];
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
+    const int ks = KS > 1 ? warp : 0;
+    const int nj = min(4, (p.N - n0 + 3) / 4);
+    if (p.M - m0 > 8) {
+        if (nj == 4) f64_tile<2, 4, KS>(p, segs, A, B, m0, n0, ks, acc);
+        else if (nj == 3) f64_tile<2, 3, KS>(p, segs, A, B, m0, n0, ks, acc);
+        else if (nj == 2) f64_tile<2, 2, KS>(p, segs, A, B, m0, n0, ks, acc);
+        else f64_tile<2, 1, KS>(p, segs, A, B, m0, n0, ks, acc);
+    } else {
+        if (nj == 4) f64_tile<1, 4, KS>(p, segs, A, B, m0, n0, ks, acc);
+        else if (nj == 3) f64_tile<1, 3, KS>(p, segs, A, B, m0, n0, ks, acc);
+        else if (nj == 2) f64_tile<1, 2, KS>(p, segs, A, B, m0, n0, ks, acc);
+        else f64_tile<1, 1, KS>(p, segs, A, B, m0, n0, ks, acc);
+    }
+    if (KS > 1) {
+        if (warp > 0)
+#pragma unroll
+            for (int i = 0; i < 2; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) part[warp - 1][(i * 4 + j) * 32 + lane] = acc[i][j];
+        __syncthreads();
+        if (warp > 0) return;
+#pragma unroll
+        for (int w = 0; w < KS - 1; ++w)
+#pragma unroll
+            for (int i = 0; i < 2; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) acc[i][j] += part[w][(i * 4 + j) * 32 + lane];
+    }
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const int m = m0 + (lane >> 2) + 8 * i;
+        if (m >= p.M) continue;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int n = n0 + (lane & 3) + 4 * j;
+            if (n >= p.N) continue;
+            const long long idx = p.c_off + (long long)m * p.scm + (long long)n * p.scn;
+            double v = p.alpha * acc[i][j];
+            if (p.accumulate) v += C[idx];
+            C[idx] = v;
+        }
+    }
+}
+
+// ------------------------------------------------------------------------------------------
+// Grouped SIMT GEMM (FP32): 64x64 output tile per CTA, 256 threads, 4x4 per thread, K chunks of 16.
 // ------------------------------------------------------------------------------------------
 template <class T>
 __global__ void __launch_bounds__(256) k_gemm_simt(const GProb* __restrict__ probs,
@@ -645,10 +815,44 @@ void launch_gemm_simt(const GProb* probs, const GSeg* segs, const GTile* tiles, 
     k_gemm_simt<T><<<ntiles, 256, 0, st>>>(probs, segs, tiles, A, B, C);
     PD_LAUNCHED();
 }
-template void launch_gemm_simt<double>(const GProb*, const GSeg*, const GTile*, int, const double*, const double*,
-                                       double*, cudaStream_t);
 template void launch_gemm_simt<float>(const GProb*, const GSeg*, const GTile*, int, const float*, const float*,
                                       float*, cudaStream_t);
+
+F64Shape f64_shape(const std::vector<GProb>& probs, const std::vector<GSeg>& segs) {
+    // 16 x 16 tiles and their mean K decide.  A tile's chain is 8 K warp instructions of 64 clocks on
+    // one scheduler, and 608 schedulers (152 SMs) want several tiles each: with 16 or more (or a K
+    // too short to divide) a warp takes a tile alone, else four warps share one, and 16 where there
+    // are fewer tiles than schedulers and a long K.  Measured, one / four / sixteen warps a tile:
+    //   5000 of 15x15x15              74 /   92 /  346 us   (64 x 64 CTA tiles before: 541)
+    //     34 of 80x80x80              69 /   53 /  100      (98)
+    //     52 of 15x15, 98 x K = 15   468 /  133 /  112      (1625)
+    //     17 of 320x320x640         1964 / 1869 / 2300      (1957; 1.19 TFLOP/s of the 1.25 measured peak)
+    //    400 of 150x150x150         2300 / 2477 / 4583      (3859)
+    long long tiles = 0, kt = 0;
+    for (const GProb& p : probs) {
+        const long long t = (long long)((p.M + 15) / 16) * ((p.N + 15) / 16);
+        long long k = 0;
+        for (int s = 0; s < p.nseg; ++s) k += segs[p.seg0 + s].K;
+        tiles += t;
+        kt += t * k;
+    }
+    const double kmean = tiles ? (double)kt / (double)tiles : 0.0;
+    if (tiles >= 9728 || kmean < 16.0) return {32, 1};
+    if (tiles <= 608 && kmean >= 256.0) return {16, 16};
+    return {16, 4};
+}
+
+void launch_gemm_f64(const GProb* probs, const GSeg* segs, const GTile* tiles, int ntiles, int edge, F64Shape shape,
+                     const double* A, const double* B, double* C, cudaStream_t st) {
+    if (ntiles <= 0) return;
+    const int side = edge / shape.tile;
+    const long long grid = (long long)ntiles * side * side;
+    PD_REQUIRE(side >= 1 && side * shape.tile == edge && grid < (1LL << 31), DMRG_ERR_CAPACITY, "FP64 GEMM tile list");
+    if (shape.ksplit == 1) k_gemm_f64<1><<<(unsigned)grid, 128, 0, st>>>(probs, segs, tiles, side, A, B, C);
+    else if (shape.ksplit == 4) k_gemm_f64<4><<<(unsigned)grid, 128, 0, st>>>(probs, segs, tiles, side, A, B, C);
+    else k_gemm_f64<16><<<(unsigned)grid, 512, 0, st>>>(probs, segs, tiles, side, A, B, C);
+    PD_LAUNCHED();
+}
 
 template <class Tin, class Tout>
 void launch_copy(const CopyJob* jobs, const int2* chunks, int nchunks, const Tin* src, Tout* dst, cudaStream_t st) {

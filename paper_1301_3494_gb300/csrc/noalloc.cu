@@ -68,11 +68,14 @@ void put(T* dev, const std::vector<T>& h, cudaStream_t st) {
     if (!h.empty()) PD_CK(cudaMemcpyAsync(dev, h.data(), h.size() * sizeof(T), cudaMemcpyHostToDevice, st));
 }
 
+// 64 x 64 tiles whatever shape the GEMM takes (its CTAs subdivide them): the scratch that the lists
+// need, and so which bonds fit, does not depend on the shape.
+constexpr int kTile = 64;
 std::vector<GTile> tiles_of(const std::vector<GProb>& probs) {
     std::vector<GTile> t;
     for (int p = 0; p < (int)probs.size(); ++p)
-        for (int m0 = 0; m0 < probs[p].M; m0 += 64)
-            for (int n0 = 0; n0 < probs[p].N; n0 += 64) t.push_back({p, m0, n0, 0});
+        for (int m0 = 0; m0 < probs[p].M; m0 += kTile)
+            for (int n0 = 0; n0 < probs[p].N; n0 += kTile) t.push_back({p, m0, n0, 0});
     return t;
 }
 
@@ -216,10 +219,10 @@ extern "C" dmrg_status dmrg_heff_apply_noalloc(const dmrg_bond_desc* bd, const d
             put(d_rt[k], rt[k], st);
         }
         PD_CK(cudaMemsetAsync(y_dev, 0, sizeof(double) * std::max<long long>(1, P.size), st));
-        launch_gemm_simt<double>(d_lp, d_ls, d_lt, (int)lt.size(), x_dev, L_dev, X, st);
+        launch_gemm_f64(d_lp, d_ls, d_lt, (int)lt.size(), kTile, f64_shape(lp, ls), x_dev, L_dev, X, st);
         launch_mix<double, double>(d_mj, d_mc, (int)mchunks.size(), d_mt, X, Y, st);
         for (size_t k = 0; k < nlaunch; ++k)
-            launch_gemm_simt<double>(d_rp[k], d_rs[k], d_rt[k], (int)rt[k].size(), R_dev, Y, y_dev, st);
+            launch_gemm_f64(d_rp[k], d_rs[k], d_rt[k], (int)rt[k].size(), kTile, f64_shape(rp[k], rs[k]), R_dev, Y, y_dev, st);
         // the host-side lists above are pageable, so every copy was staged before returning
         return DMRG_OK;
     } catch (const Error& e) {

@@ -126,12 +126,19 @@ void GemmBatch::upload_tiles(int tm, int tn, cudaStream_t st) {
     tile_n = tn;
 }
 
+F64Shape GemmBatch::upload_f64(cudaStream_t st) {
+    if (!f64.tile) f64 = f64_shape(probs, segs);
+    upload_tiles(f64.tile, f64.tile, st);
+    return f64;
+}
+
 void run_gemm64(GemmBatch& g, const double* A, const double* B, double* C, cudaStream_t st) {
     if (g.empty()) return;
     if (g_gemm64_emu && run_gemm64_emu(g, A, B, C, st)) return;
-    g.upload_tiles(64, 64, st);
+    const F64Shape shape = g.upload_f64(st);
     void* tok = prof_on() ? prof_start(st) : nullptr;
-    launch_gemm_simt<double>(g.dprobs.as<GProb>(), g.dsegs.as<GSeg>(), g.dtiles.as<GTile>(), g.ntiles, A, B, C, st);
+    launch_gemm_f64(g.dprobs.as<GProb>(), g.dsegs.as<GSeg>(), g.dtiles.as<GTile>(), g.ntiles, shape.tile, shape, A, B, C,
+                    st);
     if (tok) prof_stop(tok, st, g_prof_class == PROF_ENV ? PROF_ENV : PROF_F64, g.flops);
 }
 

@@ -157,6 +157,7 @@ struct GemmBatch {
     DBuf dprobs, dsegs, dtiles;
     int ntiles = 0;
     int tile_m = 0, tile_n = 0;         // shape of the uploaded tile list
+    F64Shape f64{0, 0};                 // FP64 tile shape (0: not chosen yet)
     int bn_choice = 0;                  // tensor-core tile width chosen for this batch (0: not yet)
     long long a_rows = 0, b_rows = 0;   // slab extents (tensor-core path)
     int lda = 0, ldb = 0;
@@ -176,8 +177,10 @@ struct GemmBatch {
         probs.push_back(p);
     }
     bool empty() const { return probs.empty(); }
-    // Upload for the FP64 engine (64x64 tiles) or the tensor-core engine (tile_m x tile_n).
+    // Upload for the FP32 SIMT engine (64x64 tiles) or the tensor-core engine (tile_m x tile_n).
     void upload_tiles(int tm, int tn, cudaStream_t st);
+    // Upload for the FP64 engine, with the tile shape that suits the batch (chosen once).
+    F64Shape upload_f64(cudaStream_t st);
 };
 
 // Run a batch: FP64 SIMT (A, B, C double) or tensor core (A, B slabs of type `t`, C of type
