@@ -461,9 +461,9 @@ __global__ void k_finite(const double* __restrict__ x, long long n, unsigned* er
     if (bad) atomicOr(err, ERRBIT_NONFINITE);
 }
 
-// Lowest eigenpair of a small symmetric matrix (k <= 32) by cyclic Jacobi, one thread.
-__global__ void k_small_eig(const double* __restrict__ G, int k, int ldg, double* __restrict__ yth) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
+// Lowest eigenpair of a small symmetric matrix (k <= 32) by cyclic Jacobi in FP64, one thread: the
+// general form, for matrices whose lowest eigenvalues the FP32 basis of k_small_eig cannot tell apart.
+__device__ __noinline__ void small_eig_serial(const double* __restrict__ G, int k, int ldg, double* __restrict__ yth) {
     double a[32][32], v[32][32];
     for (int i = 0; i < k; ++i)
         for (int j = 0; j < k; ++j) {
@@ -506,6 +506,164 @@ __global__ void k_small_eig(const double* __restrict__ G, int k, int ldg, double
         if (a[i][i] < a[best][best]) best = i;
     yth[0] = a[best][best];
     for (int i = 0; i < k; ++i) yth[1 + i] = v[i][best];
+}
+
+// Lowest eigenpair (theta, y) of a small symmetric matrix G (k <= 32), one warp.
+// The matrix is tiny, so dependent FP64 instructions (each tens of clocks here, a division or root a
+// thousand) are the whole cost of an FP64 Jacobi: about 300 us at k = 4-8 on one thread.  Instead a
+// parallel Jacobi in FP32 (round-robin pairs, on the matrix scaled by a power of two) gives an
+// approximate eigenbasis Q, and the lowest pair is refined in FP64: theta = y.Gy, r = Gy - theta y,
+// y <- y - sum_m q_m (q_m.r) / (lambda_m - theta), the sum in FP32 since it only has to be right to a
+// few digits.  The residual falls by ~1e-6 a pass; passes go on while it falls, and the pair is
+// accepted at |r| <= 32 eps |G|_F (the serial Jacobi's own backward error), else -- a cluster at the
+// bottom, or non-finite entries -- the serial form runs.  One call at k = 6: 300 -> about 10 us.
+__global__ void k_small_eig(const double* __restrict__ G, int k, int ldg, double* __restrict__ yth) {
+    constexpr unsigned ALL = 0xffffffffu;
+    __shared__ double A[32][33];
+    __shared__ float F[32][33], Q[32][33], cs[16], sn[16], rf[32], wf[32];
+    __shared__ double ys[32];
+    const int lane = threadIdx.x;
+    double amax = 0.0, fro = 0.0;
+    for (int i = 0; i < k; ++i)
+        if (lane < k) {
+            const double x = 0.5 * (G[i * ldg + lane] + G[lane * ldg + i]);
+            A[i][lane] = x;
+            amax = fmax(amax, fabs(x));
+        }
+    for (int o = 16; o > 0; o >>= 1) amax = fmax(amax, __shfl_xor_sync(ALL, amax, o));
+    bool ok = amax > 0.0 && amax < 1e300;
+    int ex = 0;
+    if (ok) frexp(amax, &ex);
+    const double sc = ok ? ldexp(1.0, -ex) : 1.0;
+    ok = ok && ex > -900;
+    if (ok) {
+        for (int i = 0; i < k; ++i)
+            if (lane < k) {
+                const double x = A[i][lane] * sc;
+                A[i][lane] = x;
+                F[i][lane] = (float)x;
+                Q[i][lane] = i == lane ? 1.f : 0.f;
+                fro = fma(x, x, fro);
+            }
+        fro = sqrt(warp_sum(fro));
+        ok = fro < 1e300;                                  // false for NaN
+    }
+    __syncwarp();
+    double y = 0.0, theta = 0.0;
+    if (ok) {
+        const int kp = k + (k & 1), np = kp / 2;
+        for (int sweep = 0; sweep < 12 && k > 1; ++sweep) {
+            float off = 0.f, dia = 0.f;
+            for (int i = 0; i < k; ++i)
+                if (lane < k) {
+                    const float x = F[i][lane];
+                    if (i == lane) dia = fmaf(x, x, dia);
+                    else off = fmaf(x, x, off);
+                }
+            for (int o = 16; o > 0; o >>= 1) {
+                off += __shfl_xor_sync(ALL, off, o);
+                dia += __shfl_xor_sync(ALL, dia, o);
+            }
+            if (off <= 1e-13f * dia) break;
+            for (int round = 0; round < kp - 1; ++round) {
+                auto player = [&](int pos) { return pos == 0 ? 0 : ((pos - 1 + round) % (kp - 1)) + 1; };
+                if (lane < np) {
+                    const int p = player(lane), q = player(kp - 1 - lane);
+                    float c = 1.f, s = 0.f;
+                    if (p < k && q < k) {
+                        const float g = F[p][q];
+                        if (g != 0.f) {
+                            const float z = (F[q][q] - F[p][p]) / (2.f * g);
+                            const float t = copysignf(1.f, z) / (fabsf(z) + sqrtf(fmaf(z, z, 1.f)));
+                            c = 1.f / sqrtf(fmaf(t, t, 1.f));
+                            s = c * t;
+                        }
+                    }
+                    cs[lane] = c;
+                    sn[lane] = s;
+                }
+                __syncwarp();
+                for (int e = lane; e < np * np; e += 32) {     // 2 x 2 blocks: they partition F
+                    const int bi = e / np, bj = e % np;
+                    const int p0 = player(bi), q0 = player(kp - 1 - bi), p1 = player(bj), q1 = player(kp - 1 - bj);
+                    const float ci = cs[bi], si = sn[bi], cj = cs[bj], sj = sn[bj];
+                    const float a = p0 < k && p1 < k ? F[p0][p1] : 0.f, b = p0 < k && q1 < k ? F[p0][q1] : 0.f;
+                    const float c = q0 < k && p1 < k ? F[q0][p1] : 0.f, d = q0 < k && q1 < k ? F[q0][q1] : 0.f;
+                    const float a1 = cj * a - sj * b, b1 = sj * a + cj * b, c1 = cj * c - sj * d, d1 = sj * c + cj * d;
+                    if (p0 < k && p1 < k) F[p0][p1] = ci * a1 - si * c1;
+                    if (q0 < k && p1 < k) F[q0][p1] = si * a1 + ci * c1;
+                    if (p0 < k && q1 < k) F[p0][q1] = ci * b1 - si * d1;
+                    if (q0 < k && q1 < k) F[q0][q1] = si * b1 + ci * d1;
+                }
+                for (int e = lane; e < k * np; e += 32) {
+                    const int r = e / np, b = e % np, p = player(b), q = player(kp - 1 - b);
+                    if (p < k && q < k) {
+                        const float x = Q[r][p], z = Q[r][q];
+                        Q[r][p] = cs[b] * x - sn[b] * z;
+                        Q[r][q] = sn[b] * x + cs[b] * z;
+                    }
+                }
+                __syncwarp();
+            }
+        }
+        int best = 0;
+        for (int i = 1; i < k; ++i)
+            if (F[i][i] < F[best][best]) best = i;
+        const float lam0 = F[best][best];
+        float inv = 0.f;                                       // 1 / (lambda_lane - lambda_best)
+        bool apart = true;
+        if (lane < k && lane != best) {
+            apart = F[lane][lane] - lam0 > 4e-6f;
+            inv = 1.f / fmaxf(F[lane][lane] - lam0, 4e-6f);
+        }
+        const bool isolated = __all_sync(ALL, apart);
+        y = lane < k ? (double)Q[lane][best] : 0.0;
+        y /= sqrt(warp_sum(y * y));
+        double last = 1e300;
+        for (int it = 0; it < 8; ++it) {
+            ys[lane] = y;
+            __syncwarp();
+            double z0 = 0.0, z1 = 0.0;
+            if (lane < k) {
+                int j = 0;
+                for (; j + 1 < k; j += 2) {
+                    z0 = fma(A[j][lane], ys[j], z0);
+                    z1 = fma(A[j + 1][lane], ys[j + 1], z1);
+                }
+                if (j < k) z0 = fma(A[j][lane], ys[j], z0);
+            }
+            z0 += z1;
+            theta = warp_sum(y * z0);
+            const double r = fma(-theta, y, z0);
+            const double rn = warp_sum(r * r);
+            // done when the residual no longer falls (squared: by less than 4) or is at rounding
+            const double eps = 2.220446049250313e-16 * fro;
+            if (!(rn > eps * eps) || !(rn < 0.25 * last)) {
+                ok = isolated && rn <= 1024.0 * eps * eps;
+                break;
+            }
+            last = rn;
+            rf[lane] = (float)r;
+            __syncwarp();
+            float t = 0.f;
+            if (lane < k)
+                for (int i = 0; i < k; ++i) t = fmaf(Q[i][lane], rf[i], t);
+            wf[lane] = -t * inv;
+            __syncwarp();
+            float dy = 0.f;
+            if (lane < k)
+                for (int m = 0; m < k; ++m) dy = fmaf(Q[lane][m], wf[m], dy);
+            y += (double)dy;
+            y *= fma(-0.5, warp_sum(y * y), 1.5);              // |y| is 1 to the correction squared
+            if (it == 7) ok = false;
+        }
+    }
+    if (!ok) {
+        if (lane == 0) small_eig_serial(G, k, ldg, yth);
+        return;
+    }
+    if (lane == 0) yth[0] = ldexp(theta, ex);
+    if (lane < k) yth[1 + lane] = y;
 }
 
 // ------------------------------------------------------------------------------------------
