@@ -1,6 +1,7 @@
 // Contraction plans and device building blocks of the two-site DMRG step (Sec. II).
 #include <cfloat>
 #include <cmath>
+#include <cstring>
 #include <map>
 #include <tuple>
 
@@ -418,7 +419,7 @@ void convert_flat(const void* src, Num in, void* dst, Num out, long long n, cuda
     else run_copy<float>(cl, static_cast<const float*>(src), dst, out, st);
 }
 
-void orthonormalize_square(const std::vector<SvdSec>& ss, double* V, cudaStream_t st) {
+void orthonormalize_square(const std::vector<SvdSec>& ss, double* V, cudaStream_t st, int max_iter) {
     std::vector<NsJob> jobs;
     std::vector<DevJob> djobs;
     GemmBatch gG, gX;
@@ -445,7 +446,7 @@ void orthonormalize_square(const std::vector<SvdSec>& ss, double* V, cudaStream_
     upload(dj, jobs, st);
     upload(djd, djobs, st);
     std::vector<double> hdev(jobs.size());
-    for (int iter = 0; iter < 8; ++iter) {
+    for (int iter = 0; iter < max_iter; ++iter) {
         run_gemm64(gG, V, V, G.as<double>(), st);
         k_gram_dev<<<(unsigned)jobs.size(), 256, 0, st>>>(djd.as<DevJob>(), G.as<double>(), dev.as<double>());
         PD_LAUNCHED();
@@ -456,7 +457,7 @@ void orthonormalize_square(const std::vector<SvdSec>& ss, double* V, cudaStream_
         PD_REQUIRE(std::isfinite(worst) && worst < 0.5, DMRG_ERR_NUMERIC,
                    "FP32 Jacobi rotations too far from orthogonal for the FP64 polish (|V^T V - I| = " +
                        std::to_string(worst) + " at iteration " + std::to_string(iter) + ")");
-        if (worst < 1e-14) break;
+        if (worst < 1e-14) return;
         k_ns_prep<<<dim3(gridn(mx, 256), (unsigned)jobs.size()), 256, 0, st>>>(dj.as<NsJob>(), G.as<double>(),
                                                                                T.as<double>());
         PD_LAUNCHED();
@@ -464,6 +465,7 @@ void orthonormalize_square(const std::vector<SvdSec>& ss, double* V, cudaStream_
         for (const auto& j : jobs)
             PD_CK(cudaMemcpyAsync(V + j.off, out.as<double>() + j.off, (size_t)j.k * j.k * 8, cudaMemcpyDeviceToDevice, st));
     }
+    PD_REQUIRE(max_iter <= 8, DMRG_ERR_NUMERIC, "Newton-Schulz orthonormalisation did not converge");
 }
 
 void scale_vec(double* x, long long n, double s, cudaStream_t st) {
@@ -1174,9 +1176,11 @@ void col_copy(const std::vector<ColJob>& jobs, const double* src, double* dst, c
 // sig the column norms and ord their descending order; dsecs the device copy of ss.
 // FP32 block Jacobi (one task per block pair, n / 16 - 1 rounds per sweep) of the batch ss: W (p x n
 // at w_off), rotations accumulated into V (n x n at v_off, initialised by the caller); rot: sweep
-// histogram (max_sweeps + 1 ints, zeroed), bar: 3 zeroed barrier words, err: error word.
+// histogram (max_sweeps + 1 ints, zeroed), bar: 3 zeroed barrier words, err: error word.  noise_c: the
+// absolute rounding level below which a pair is left (times sigma_max; 0: the relative test alone).
 void block_jacobi32(const std::vector<SvdSec>& ss, const SvdSec* dsecs, float* W, float* V, int max_rows, int max_n,
-                    int max_sweeps, int* rot, unsigned* bar, unsigned* err, unsigned long long* flops, cudaStream_t st) {
+                    int max_sweeps, int* rot, unsigned* bar, unsigned* err, unsigned long long* flops, cudaStream_t st,
+                    float noise_c = 8.0f * FLT_EPSILON) {
     const int nsec = (int)ss.size();
     std::vector<BjSec> bs(nsec);
     std::vector<int> task_sec;
@@ -1229,7 +1233,7 @@ void block_jacobi32(const std::vector<SvdSec>& ss, const SvdSec* dsecs, float* W
     PD_CK(cudaMemsetAsync(dstamp.p, 0, (size_t)std::max(1, nblk + npst) * 4, st));
     PD_CK(cudaMemsetAsync(flops, 0, 8, st));
     launch_bjacobi(dsecs, dbs.as<BjSec>(), dts.as<int>(), (int)task_sec.size(), nrounds, max_rows, max_n, bj_sweeps, 2,
-                   W, V, 8.0f * FLT_EPSILON, dgmax.as<float>(), dstamp.as<int>(), dstamp.as<int>() + nblk, rot,
+                   W, V, noise_c, dgmax.as<float>(), dstamp.as<int>(), dstamp.as<int>() + nblk, rot,
                    rot + max_sweeps, bar, err, flops, ditems.as<int2>(), (int)items.size(), nsec, nact, dq.as<int>(), st);
 }
 
@@ -1261,6 +1265,249 @@ void fp64_precondition(const std::vector<SvdSec>& ss, const SvdSec* dsecs, DBuf&
     run_gemm64(gwq, dW.as<double>(), V, dW1.as<double>(), st);
     PD_CK(cudaMemsetAsync(bar, 0, 3 * sizeof(unsigned), st));
     dW = std::move(dW1);
+}
+
+// ------------------------------------------------------------------------------------------
+// FP64 polish of a nearly finished one-sided Jacobi SVD by whole-matrix rotations.
+//
+// After fp64_precondition the columns of W are orthogonal to FP32 accuracy.  A scalar FP64 Jacobi
+// from there costs n - 1 rounds a sweep for some seven sweeps, each round a chain of dot products,
+// a reduction, a root and a division on FP64 units that issue 2 DFMA per clock and SM, and a grid
+// barrier: 86 ms for the 512-state bond of a chain.  Instead all pairs are rotated at once:
+//   G = W^T W;  E(i, j) = -E(j, i) = tan of the Jacobi rotation of the pair (i, j);
+//   Q = the orthogonal polar factor of I + E (exactly the Jacobi rotation for a single pair);
+//   W <- W Q,  V <- V Q.
+// The angles that this leaves are of second order in E, so from 1e-6 two or three passes end at
+// rounding level; each is a handful of grouped GEMMs.  The test is the scalar Jacobi's own: no pair
+// with |g_ij| > tol |w_i| |w_j|; a batch that has not met it after kPolishPasses goes on with the
+// scalar Jacobi.  W and V are updated as W + W (Q - I): the entries of Q - I fall with sigma_j /
+// sigma_i, so small columns keep their relative accuracy.
+// Columns below about 1e-6 of the largest are not resolved by FP32 at all.  The first pass frees them
+// of the large columns (those angles are small) and leaves the angles among themselves, which a second
+// FP32 block Jacobi on these columns alone, scaled to order one, then makes small.
+// Whole splits: 512-state chain bond 96 -> 31 ms, accurate split at the 24x8 cylinder's m = 1000 bond
+// 164 -> 52 ms, and closer to 64 bits than the scalar Jacobi's (2.8e-15 against 1.8e-14).
+// ------------------------------------------------------------------------------------------
+constexpr int kPolishPasses = 16;
+
+// One CTA per column j of a sector: E(:, j) from the lower triangle of G (rows i >= 64 (j / 64)),
+// rotations by at most tan = 0.6, and none between two columns at or after cut[sector].  stat, four
+// words per sector: [0] columns with a pair above tol (those above tol / 10 turn too), [1] n - (first column of an unresolved pair:
+// cos > 1e-3 and tan > 0.1), [2] largest squared column norm of E as float bits.
+struct PolCol {
+    int sec, j;
+};
+__global__ void k_polish_angles(const SvdSec* __restrict__ secs, const PolCol* __restrict__ cols,
+                                const double* __restrict__ G, double* __restrict__ E, const int* __restrict__ cut,
+                                double* __restrict__ diag, unsigned* __restrict__ stat) {
+    const PolCol pc = cols[blockIdx.x];
+    const SvdSec s = secs[pc.sec];
+    const int j = pc.j, n = s.n;
+    const double* Gs = G + s.v_off;
+    double* Ej = E + s.v_off + (long long)j * n;
+    const double gjj = Gs[j + (long long)j * n];
+    const double tol = 4.0 * DBL_EPSILON * sqrt((double)s.p);
+    const int from = cut[pc.sec];
+    float sum = 0.f;
+    int above = 0, first = n;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        const int lo = min(i, j), hi = max(i, j);
+        const double g = Gs[hi + (long long)lo * n], gii = Gs[i + (long long)i * n];
+        double t = 0.0;
+        const double size = sqrt(gii * gjj);
+        if (i != j && fabs(g) > 0.1 * tol * size) {
+            above |= fabs(g) > tol * size;
+            const double zeta = (gjj - gii) / (2.0 * g);
+            t = 1.0 / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
+            if (t > 0.1 && fabs(g) > 1e-3 * size) first = min(first, lo);
+            t = lo >= from ? 0.0 : fmin(t, 0.6);
+            if (zeta < 0.0 || (zeta == 0.0 && i > j)) t = -t;
+            sum = fmaf((float)t, (float)t, sum);
+        }
+        Ej[i] = t;
+    }
+    if (threadIdx.x == 0) diag[s.s_off + j] = gjj;
+    for (int o = 16; o > 0; o >>= 1) {
+        sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        first = min(first, __shfl_xor_sync(0xffffffffu, first, o));
+        above |= __shfl_xor_sync(0xffffffffu, above, o);
+    }
+    __shared__ float ssum[4];
+    if ((threadIdx.x & 31) == 0) {
+        ssum[threadIdx.x >> 5] = sum;
+        if (above) atomicAdd(&stat[4 * pc.sec], 1u);
+        if (first < n) atomicMax(&stat[4 * pc.sec + 1], (unsigned)(n - first));
+    }
+    __syncthreads();
+    if (threadIdx.x == 0)
+        atomicMax(&stat[4 * pc.sec + 2], __float_as_uint(ssum[0] + ssum[1] + ssum[2] + ssum[3]));
+}
+
+// X = scale E + a I over the sectors' n x n matrices (X may be E).
+__global__ void k_polish_shift(const SvdSec* __restrict__ secs, const PolCol* __restrict__ cols, const double* E,
+                               double scale, double a, double* X) {
+    const PolCol pc = cols[blockIdx.x];
+    const SvdSec s = secs[pc.sec];
+    const long long o = s.v_off + (long long)pc.j * s.n;
+    for (int i = threadIdx.x; i < s.n; i += blockDim.x) X[o + i] = fma(scale, E[o + i], i == pc.j ? a : 0.0);
+}
+
+// Returns true when every pair of columns meets the tolerance (*passes: passes taken).
+bool polish64(const std::vector<SvdSec>& ss, const SvdSec* dsecs, DBuf& dW, DBuf& dV, long long woff, long long voff,
+              long long soff, unsigned* bar, unsigned* err, int* passes, cudaStream_t st) {
+    const int nsec = (int)ss.size();
+    std::vector<PolCol> cols;
+    GemmBatch gG, gW, gV, gE;
+    for (int s = 0; s < nsec; ++s) {
+        const SvdSec& x = ss[s];
+        for (int j = 0; j < x.n; ++j) cols.push_back({s, j});
+        // lower block triangle of G, 64 columns at a time
+        for (int j0 = 0; j0 < x.n; j0 += 64)
+            gG.add(x.n - j0, std::min(64, x.n - j0), x.v_off + j0 + (long long)j0 * x.n, x.p, 1, x.p, 1, 1, x.n,
+                   {GSeg{x.w_off + (long long)j0 * x.p, x.w_off + (long long)j0 * x.p, x.p, 0}});
+        gW.add(x.p, x.n, x.w_off, 1, x.p, x.n, 1, 1, x.p, {GSeg{x.w_off, x.v_off, x.n, 0}}, 1);
+        gV.add(x.n, x.n, x.v_off, 1, x.n, x.n, 1, 1, x.n, {GSeg{x.v_off, x.v_off, x.n, 0}}, 1);
+        gE.add(x.n, x.n, x.v_off, 1, x.n, x.n, 1, 1, x.n, {GSeg{x.v_off, x.v_off, x.n, 0}}, 1, 0.5);
+    }
+    *passes = 0;
+    if (cols.empty()) return true;
+    DBuf dcols, G, E, X, Wn, Vn, diag, stat;
+    upload(dcols, cols, st);
+    G.ensure(voff * 8, st);
+    E.ensure(voff * 8, st);
+    X.ensure(voff * 8, st);
+    Wn.ensure(woff * 8, st);
+    Vn.ensure(voff * 8, st);
+    diag.ensure(soff * 8, st);
+    stat.ensure((size_t)nsec * 16, st);
+    std::vector<unsigned> hs((size_t)nsec * 4);
+    std::vector<double> hd(soff);
+    const unsigned nc = (unsigned)cols.size();
+    std::vector<int> cut(nsec);
+    DBuf dcut;
+    int large = 0;                        // passes in a row with large angles
+    int stages = 3;                       // FP32 passes over unresolved columns still allowed
+    for (int pass = 0; pass < kPolishPasses; ++pass) {
+        run_gemm64(gG, dW.as<double>(), dW.as<double>(), G.as<double>(), st);
+        auto angles = [&]() {
+            upload(dcut, cut, st);
+            PD_CK(cudaMemsetAsync(stat.p, 0, (size_t)nsec * 16, st));
+            k_polish_angles<<<nc, 128, 0, st>>>(dsecs, dcols.as<PolCol>(), G.as<double>(), E.as<double>(),
+                                                dcut.as<int>(), diag.as<double>(), stat.as<unsigned>());
+            PD_LAUNCHED();
+            PD_CK(cudaMemcpyAsync(hs.data(), stat.p, (size_t)nsec * 16, cudaMemcpyDeviceToHost, st));
+            PD_CK(cudaMemcpyAsync(hd.data(), diag.p, (size_t)soff * 8, cudaMemcpyDeviceToHost, st));
+            PD_CK(cudaStreamSynchronize(st));
+        };
+        for (int s = 0; s < nsec; ++s) cut[s] = ss[s].n;
+        angles();
+        bool unresolved = false, above = false;
+        for (int s = 0; s < nsec; ++s) {
+            above = above || hs[4 * s] > 0;
+            unresolved = unresolved || (stages > 0 && hs[4 * s + 1] > 0);
+        }
+        if (!above) return true;
+        *passes = pass + 1;
+        if (unresolved) {
+            // the unresolved columns turn against the others only
+            for (int s = 0; s < nsec; ++s) cut[s] = ss[s].n - (int)hs[4 * s + 1];
+            angles();
+        }
+        float norm = 0.f;
+        for (int s = 0; s < nsec; ++s) {
+            float v;
+            std::memcpy(&v, &hs[4 * s + 2], 4);
+            if (!std::isfinite(v)) return false;
+            norm = std::max(norm, std::sqrt(v));
+        }
+        // a cluster whose columns all want large angles among themselves does not settle this way
+        large = !unresolved && norm > 0.6f ? large + 1 : 0;
+        if (large > 2) return false;
+        // E <- Q - I
+        if (norm <= 1e-6f) {
+            // (I + E)(I - E^2)^(-1/2) = I + E + E^2 / 2 + O(|E|^3)
+            PD_CK(cudaMemcpyAsync(X.p, E.p, voff * 8, cudaMemcpyDeviceToDevice, st));
+            run_gemm64(gE, E.as<double>(), E.as<double>(), X.as<double>(), st);
+            std::swap(E, X);
+        } else {
+            k_polish_shift<<<nc, 128, 0, st>>>(dsecs, dcols.as<PolCol>(), E.as<double>(), norm > 0.6f ? 0.6 / norm : 1.0,
+                                               1.0, X.as<double>());
+            PD_LAUNCHED();
+            try {
+                orthonormalize_square(ss, X.as<double>(), st, 14);
+            } catch (const Error& e) {
+                if (e.st != DMRG_ERR_NUMERIC) throw;
+                return false;                 // angles too large to take together: W and V are as before
+            }
+            k_polish_shift<<<nc, 128, 0, st>>>(dsecs, dcols.as<PolCol>(), X.as<double>(), 1.0, -1.0, E.as<double>());
+            PD_LAUNCHED();
+        }
+        PD_CK(cudaMemcpyAsync(Wn.p, dW.p, woff * 8, cudaMemcpyDeviceToDevice, st));
+        PD_CK(cudaMemcpyAsync(Vn.p, dV.p, voff * 8, cudaMemcpyDeviceToDevice, st));
+        run_gemm64(gW, dW.as<double>(), E.as<double>(), Wn.as<double>(), st);
+        run_gemm64(gV, dV.as<double>(), E.as<double>(), Vn.as<double>(), st);
+        std::swap(dW, Wn);
+        std::swap(dV, Vn);
+        // FP32 block Jacobi on the columns from the cut of every sector that has unresolved pairs, once the
+        // rotations against the resolved columns have become small
+        if (!unresolved || norm > 0.05f) continue;
+        --stages;
+        std::vector<SvdSec> sub;
+        CopyList down;
+        GemmBatch gw, gv;
+        long long wo = 0, vo = 0;
+        int mp = 1, mn = 1;
+        for (int s = 0; s < nsec; ++s) {
+            if (cut[s] >= ss[s].n) continue;
+            const SvdSec& x = ss[s];
+            SvdSec y{};
+            y.p = x.p;
+            y.n = x.n - cut[s];
+            y.npad = y.n + (y.n & 1);
+            y.w_off = wo;
+            y.v_off = vo;
+            double top = 0.0;
+            for (int j = cut[s]; j < x.n; ++j) top = std::max(top, hd[x.s_off + j]);
+            CopyJob j{};
+            j.src = x.w_off + (long long)cut[s] * x.p; j.dst = wo; j.rows = y.n; j.cols = x.p;
+            j.srs = x.p; j.scs = 1; j.drs = x.p; j.dcs = 1; j.zero_to = 0;
+            j.scale = top > 0.0 ? std::ldexp(1.0, -std::ilogb(std::sqrt(top))) : 1.0;
+            down.add(j);
+            const long long wc = x.w_off + (long long)cut[s] * x.p, vc = x.v_off + (long long)cut[s] * x.n;
+            gw.add(x.p, y.n, wc, 1, x.p, y.n, 1, 1, x.p, {GSeg{wc, vo, y.n, 0}});
+            gv.add(x.n, y.n, vc, 1, x.n, y.n, 1, 1, x.n, {GSeg{vc, vo, y.n, 0}});
+            wo += (long long)y.p * y.n;
+            vo += (long long)y.n * y.n;
+            mp = std::max(mp, y.p);
+            mn = std::max(mn, y.n);
+            sub.push_back(y);
+        }
+        const int max_sweeps = 60;
+        DBuf w32, v32, v64, rot32, fl, dsub;
+        w32.ensure(wo * 4, st);
+        v32.ensure(vo * 4, st);
+        v64.ensure(vo * 8, st);
+        rot32.ensure((max_sweeps + 1) * 4, st);
+        fl.ensure(8, st);
+        upload(dsub, sub, st);
+        down.up(st);
+        PD_CK(cudaMemsetAsync(rot32.p, 0, (max_sweeps + 1) * 4, st));
+        PD_CK(cudaMemsetAsync(bar, 0, 3 * sizeof(unsigned), st));
+        run_copy<double>(down, dW.as<double>(), w32.p, Num::F32, st);
+        launch_svd_init_v<float>(dsub.as<SvdSec>(), (int)sub.size(), mn, v32.as<float>(), st);
+        block_jacobi32(sub, dsub.as<SvdSec>(), w32.as<float>(), v32.as<float>(), mp, mn, max_sweeps, rot32.as<int>(), bar,
+                       err, fl.as<unsigned long long>(), st, 0.0f);
+        convert_flat(v32.p, Num::F32, v64.p, Num::F64, vo, st);
+        orthonormalize_square(sub, v64.as<double>(), st);
+        PD_CK(cudaMemcpyAsync(Wn.p, dW.p, woff * 8, cudaMemcpyDeviceToDevice, st));
+        PD_CK(cudaMemcpyAsync(Vn.p, dV.p, voff * 8, cudaMemcpyDeviceToDevice, st));
+        run_gemm64(gw, dW.as<double>(), v64.as<double>(), Wn.as<double>(), st);
+        run_gemm64(gv, dV.as<double>(), v64.as<double>(), Vn.as<double>(), st);
+        std::swap(dW, Wn);
+        std::swap(dV, Vn);
+        PD_CK(cudaMemsetAsync(bar, 0, 3 * sizeof(unsigned), st));
+    }
+    return false;
 }
 
 void jacobi64(std::vector<SvdSec>& ss, DBuf& dWbuf, DBuf& dsecs, DBuf& dV, DBuf& dsig, DBuf& dord, cudaStream_t st) {
@@ -1298,11 +1545,13 @@ void jacobi64(std::vector<SvdSec>& ss, DBuf& dWbuf, DBuf& dsecs, DBuf& dV, DBuf&
         fp64_precondition(ss, dsecs.as<SvdSec>(), dWbuf, dV.as<double>(), woff, voff, maxp, maxn, bar, bar + 3, st);
     else
         launch_svd_init_v<double>(dsecs.as<SvdSec>(), nsec, maxn, dV.as<double>(), st);
+    int passes = 0;
+    if (!(g_svd_qr && woff > 0 &&
+          polish64(ss, dsecs.as<SvdSec>(), dWbuf, dV, woff, voff, soff, bar, bar + 3, &passes, st)))
+        launch_jacobi<double>(dsecs.as<SvdSec>(), nsec, dpairs.as<int>(), (int)pair_sec.size(), maxnpad, max_sweeps,
+                              dWbuf.as<double>(), dV.as<double>(), 4.0 * DBL_EPSILON, 0.0, nullptr, drot.as<int>(),
+                              drot.as<int>() + max_sweeps, bar, bar + 3, st);
     double* W = dWbuf.as<double>();
-    const double tol = 4.0 * DBL_EPSILON;
-    launch_jacobi<double>(dsecs.as<SvdSec>(), nsec, dpairs.as<int>(), (int)pair_sec.size(), maxnpad, max_sweeps, W,
-                          dV.as<double>(), tol, 0.0, nullptr, drot.as<int>(), drot.as<int>() + max_sweeps, bar, bar + 3,
-                          st);
     launch_svd_finish<double>(dsecs.as<SvdSec>(), nsec, W, dsig.as<double>(), dord.as<int>(), st);
     unsigned err = 0;
     PD_CK(cudaMemcpyAsync(&err, bar + 3, 4, cudaMemcpyDeviceToHost, st));
@@ -1589,9 +1838,14 @@ std::vector<SplitResult> svd_split_batch(const std::vector<SplitReq>& reqs, bool
             fp64_precondition(ss, dsecs.as<SvdSec>(), dW, dV.as<double>(), woff, voff, maxp, maxn, bar, jerr, st);
         else
             launch_svd_init_v<double>(dsecs.as<SvdSec>(), nsec, maxn, dV.as<double>(), st);
-        launch_jacobi<double>(dsecs.as<SvdSec>(), nsec, dpairs.as<int>(), npairs, maxnpad, max_sweeps, dW.as<double>(),
-                              dV.as<double>(), tol, 0.0, nullptr, drot.as<int>(), drot.as<int>() + max_sweeps, bar, jerr,
-                              st);
+        int passes = 0;
+        if (g_svd_qr && woff > 0 &&
+            polish64(ss, dsecs.as<SvdSec>(), dW, dV, woff, voff, soff, bar, jerr, &passes, st))
+            PD_CK(cudaMemcpyAsync(drot.as<int>() + max_sweeps, &passes, sizeof(int), cudaMemcpyHostToDevice, st));
+        else
+            launch_jacobi<double>(dsecs.as<SvdSec>(), nsec, dpairs.as<int>(), npairs, maxnpad, max_sweeps,
+                                  dW.as<double>(), dV.as<double>(), tol, 0.0, nullptr, drot.as<int>(),
+                                  drot.as<int>() + max_sweeps, bar, jerr, st);
         launch_svd_finish<double>(dsecs.as<SvdSec>(), nsec, dW.as<double>(), dsig.as<double>(), dord.as<int>(), st);
         if (accurate && woff > 0)
             accurate_refine(ss, dsecs.as<SvdSec>(), dW.as<double>(), dV.as<double>(), dsig.as<double>(),
