@@ -100,8 +100,9 @@ typedef struct {
     int fp64_emulation;     /* 1 = the context's FP64 grouped GEMMs (FP64-mode matvec and
                                environment updates, wavefunction formation, gauge moves, local
                                measurements) run FP64-accurate on the bf16 tensor cores
-                               (dmrg_gemm64 mode 1); batches outside its K limit stay on the
-                               FP64 units.  0 = FP64 units throughout.                          */
+                               (dmrg_gemm64 mode 1); batches outside its K limit, and those too
+                               small to gain from it (below about 1 GFLOP), stay on the FP64
+                               units.  0 = FP64 units throughout.                               */
     int svd_plain_jacobi;   /* 1 = every split's one-sided Jacobi runs on the sector matrix W
                                itself; 0 (default) = on R^T from a Householder QR W = QR (a
                                few sweeps instead of many; sectors taller than the QR panel's

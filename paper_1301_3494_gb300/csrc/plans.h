@@ -158,6 +158,7 @@ struct GemmBatch {
     int ntiles = 0;
     int tile_m = 0, tile_n = 0;         // shape of the uploaded tile list
     F64Shape f64{0, 0};                 // FP64 tile shape (0: not chosen yet)
+    int uses = 0;                       // runs so far with FP64 emulation on
     int bn_choice = 0;                  // tensor-core tile width chosen for this batch (0: not yet)
     long long a_rows = 0, b_rows = 0;   // slab extents (tensor-core path)
     int lda = 0, ldb = 0;
