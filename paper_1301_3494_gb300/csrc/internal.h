@@ -232,10 +232,10 @@ void launch_bjacobi(const SvdSec* secs, const BjSec* bsecs, const int* task_sec,
                     unsigned long long* flops, const int2* items, int per_sweep, int nsec, int nact, int* qstate,
                     cudaStream_t st);
 template <class T>
-void launch_svd_finish(const SvdSec* secs, int nsec, const T* W, double* sig, int* order, cudaStream_t st);
+void launch_svd_finish(const SvdSec* secs, int nsec, int max_n, const T* W, double* sig, int* order, cudaStream_t st);
 
 // Truncation selection over all sectors.  sig sorted per sector by `order`; sectors packed
-// back to back (s_off = prefix sums).  Scratch: (total + nsec) doubles, 3*total ints.
+// back to back (s_off = prefix sums).  Scratch: (total + nsec) doubles, 2*total ints.
 void launch_truncate(const SvdSec* secs, int nsec, const double* sig, const int* order, int total, int m_max,
                      double rel_cutoff, double degen_tol, int* kept, double* weights, double* scratch_d, int* scratch_i,
                      cudaStream_t st);

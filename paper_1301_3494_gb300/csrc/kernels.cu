@@ -840,40 +840,54 @@ __global__ void k_svd_floor(const SvdSec* __restrict__ secs, const T* __restrict
     if (threadIdx.x == 0) floor2[blockIdx.x] = eta * eta * a;
 }
 
-// sig[s_off + i] = |W_i| (FP64), order[s_off + r] = column with the r-th largest norm (ties: lower index).
+// sig[s_off + i] = |W_i| (FP64): one warp per column.
 template <class T>
-__global__ void k_svd_finish(const SvdSec* __restrict__ secs, const T* __restrict__ W, double* __restrict__ sig,
-                             int* __restrict__ order) {
-    const SvdSec s = secs[blockIdx.x];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    for (int c = wid; c < s.n; c += nw) {
-        const T* col = W + s.w_off + (long long)c * s.p;
-        double a = 0.0;
-        for (int r = lane; r < s.p; r += 32) a = fma((double)col[r], (double)col[r], a);
-        a = warp_sum(a);
-        if (lane == 0) sig[s.s_off + c] = sqrt(a);
+__global__ void k_svd_norms(const SvdSec* __restrict__ secs, const T* __restrict__ W, double* __restrict__ sig) {
+    const SvdSec s = secs[blockIdx.y];
+    const int lane = threadIdx.x & 31, c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (c >= s.n) return;
+    const T* col = W + s.w_off + (long long)c * s.p;
+    double a = 0.0, b = 0.0;
+    int r = lane;
+    for (; r + 32 < s.p; r += 64) {
+        const double x = (double)col[r], y = (double)col[r + 32];
+        a = fma(x, x, a);
+        b = fma(y, y, b);
     }
-    __syncthreads();
-    for (int c = threadIdx.x; c < s.n; c += blockDim.x) {
-        double v = sig[s.s_off + c];
-        int rank = 0;
-        for (int o = 0; o < s.n; ++o) {
-            double w = sig[s.s_off + o];
-            rank += (w > v) || (w == v && o < c);
-        }
-        order[s.s_off + rank] = c;
+    if (r < s.p) a = fma((double)col[r], (double)col[r], a);
+    a = warp_sum(a + b);
+    if (lane == 0) sig[s.s_off + c] = sqrt(a);
+}
+
+// Norms are not negative, so they order like their bit patterns (integer comparisons: a double's
+// would run on the FP64 pipe).
+__device__ __forceinline__ long long norm_bits(double x) { return __double_as_longlong(x); }
+
+// order[s_off + r] = column with the r-th largest norm (ties: lower index): one warp per column.  (One
+// CTA per sector did norms and ranks before: 600 us for the 68 sectors of four m = 2000 bonds, 20 now.)
+__global__ void k_svd_order(const SvdSec* __restrict__ secs, const double* __restrict__ sig, int* __restrict__ order) {
+    const SvdSec s = secs[blockIdx.y];
+    const int lane = threadIdx.x & 31, c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (c >= s.n) return;
+    const long long v = norm_bits(sig[s.s_off + c]);
+    int rank = 0;
+    for (int o = lane; o < s.n; o += 32) {
+        const long long w = norm_bits(sig[s.s_off + o]);
+        rank += (w > v) || (w == v && o < c);
     }
+    rank = __reduce_add_sync(0xffffffffu, rank);
+    if (lane == 0) order[s.s_off + rank] = c;
 }
 
 // ------------------------------------------------------------------------------------------
 // Truncation selection.  Keys (lambda desc, sector asc, position asc) over all sectors' values.
-//   k_trunc_flat   flat arrays lam[g], sec[g], pos[g] (sector order, descending inside)
+//   k_trunc_flat   flat arrays lam[g], sec[g] (sector order, descending inside)
 //   k_trunc_rank   rank of every candidate (lambda > rel_cutoff * lambda_max) among candidates
 //   k_trunc_count  kept[s] and weights: total sum lambda^2, kept sum lambda^2
 // ------------------------------------------------------------------------------------------
 __global__ void k_trunc_flat(const SvdSec* __restrict__ secs, int nsec, const double* __restrict__ sig,
                              const int* __restrict__ order, double* __restrict__ lam, int* __restrict__ sec,
-                             int* __restrict__ pos, double* __restrict__ lmax) {
+                             double* __restrict__ lmax) {
     const int s = blockIdx.x;
     const SvdSec S = secs[s];
     double mx = 0.0;
@@ -881,7 +895,6 @@ __global__ void k_trunc_flat(const SvdSec* __restrict__ secs, int nsec, const do
         double v = sig[S.s_off + order[S.s_off + i]];
         lam[S.s_off + i] = v;
         sec[S.s_off + i] = s;
-        pos[S.s_off + i] = i;
         mx = fmax(mx, v);
     }
     for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
@@ -895,30 +908,28 @@ __global__ void k_trunc_flat(const SvdSec* __restrict__ secs, int nsec, const do
     }
 }
 
-__global__ void k_trunc_rank(const double* __restrict__ lam, const int* __restrict__ sec, const int* __restrict__ pos,
-                             int total, const double* __restrict__ lmax_sec, int nsec, double rel_cutoff,
-                             int* __restrict__ rank) {
-    __shared__ double thr_s;
-    if (threadIdx.x == 0) {
-        double m = 0.0;
-        for (int s = 0; s < nsec; ++s) m = fmax(m, lmax_sec[s]);
-        thr_s = rel_cutoff * m;
-    }
-    __syncthreads();
-    const double thr = thr_s;
-    const int g = blockIdx.x * blockDim.x + threadIdx.x;
+// One warp per value; the flat index orders like (sector, position), so it breaks ties.  (A thread per
+// value and double comparisons before: 580 us for the 4000 values of an m = 2000 bond, 20 now.)
+__global__ void k_trunc_rank(const double* __restrict__ lam, int total, const double* __restrict__ lmax_sec, int nsec,
+                             double rel_cutoff, int* __restrict__ rank) {
+    const int lane = threadIdx.x & 31, g = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (g >= total) return;
-    const double v = lam[g];
-    const int sg = sec[g], pg = pos[g];
+    double m = 0.0;
+    for (int s = lane; s < nsec; s += 32) m = fmax(m, lmax_sec[s]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+    const double thr = rel_cutoff * m, v = lam[g];
     int r = -1;
-    if (v > thr) {
+    if (v > thr) {                                   // the same in every lane
+        const long long tb = norm_bits(thr), vb = norm_bits(v), inf = 0x7FF0000000000000ll;
         r = 0;
-        for (int o = 0; o < total; ++o) {
-            const double w = lam[o];
-            r += (w > thr) && ((w > v) || (w == v && (sec[o] < sg || (sec[o] == sg && pos[o] < pg))));
+        for (int o = lane; o < total; o += 32) {
+            const long long w = norm_bits(lam[o]);
+            r += w > tb && w <= inf && (w > vb || (w == vb && o < g));
         }
+        r = __reduce_add_sync(0xffffffffu, r);
     }
-    rank[g] = r;
+    if (lane == 0) rank[g] = r;
 }
 
 __global__ void __launch_bounds__(1024) k_trunc_count(const double* __restrict__ lam, const int* __restrict__ sec,
@@ -1175,13 +1186,16 @@ template void launch_jacobi<float>(const SvdSec*, int, const int*, int, int, int
                                    double*, int*, int*, unsigned*, unsigned*, cudaStream_t);
 
 template <class T>
-void launch_svd_finish(const SvdSec* secs, int nsec, const T* W, double* sig, int* order, cudaStream_t st) {
-    if (nsec <= 0) return;
-    k_svd_finish<T><<<nsec, 256, 0, st>>>(secs, W, sig, order);
+void launch_svd_finish(const SvdSec* secs, int nsec, int max_n, const T* W, double* sig, int* order, cudaStream_t st) {
+    if (nsec <= 0 || max_n <= 0) return;
+    const dim3 grid((max_n + 7) / 8, nsec);
+    k_svd_norms<T><<<grid, 256, 0, st>>>(secs, W, sig);
+    PD_LAUNCHED();
+    k_svd_order<<<grid, 256, 0, st>>>(secs, sig, order);
     PD_LAUNCHED();
 }
-template void launch_svd_finish<double>(const SvdSec*, int, const double*, double*, int*, cudaStream_t);
-template void launch_svd_finish<float>(const SvdSec*, int, const float*, double*, int*, cudaStream_t);
+template void launch_svd_finish<double>(const SvdSec*, int, int, const double*, double*, int*, cudaStream_t);
+template void launch_svd_finish<float>(const SvdSec*, int, int, const float*, double*, int*, cudaStream_t);
 
 void launch_truncate(const SvdSec* secs, int nsec, const double* sig, const int* order, int total, int m_max,
                      double rel_cutoff, double degen_tol, int* kept, double* weights, double* scratch_d, int* scratch_i,
@@ -1191,11 +1205,10 @@ void launch_truncate(const SvdSec* secs, int nsec, const double* sig, const int*
     double* lam = scratch_d;
     double* lmax = scratch_d + total;
     int* sec = scratch_i;
-    int* pos = scratch_i + total;
-    int* rank = scratch_i + 2 * total;
-    k_trunc_flat<<<nsec, 256, 0, st>>>(secs, nsec, sig, order, lam, sec, pos, lmax);
+    int* rank = scratch_i + total;
+    k_trunc_flat<<<nsec, 256, 0, st>>>(secs, nsec, sig, order, lam, sec, lmax);
     PD_LAUNCHED();
-    k_trunc_rank<<<(total + 127) / 128, 128, 0, st>>>(lam, sec, pos, total, lmax, nsec, rel_cutoff, rank);
+    k_trunc_rank<<<(total + 7) / 8, 256, 0, st>>>(lam, total, lmax, nsec, rel_cutoff, rank);
     PD_LAUNCHED();
     k_trunc_count<<<1, 1024, 0, st>>>(lam, sec, rank, total, nsec, m_max, degen_tol, kept, weights);
     PD_LAUNCHED();

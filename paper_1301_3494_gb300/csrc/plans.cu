@@ -305,37 +305,67 @@ void scale_site(const Sec& bl, const Sec& br, const std::vector<int>& qn, const 
 }
 
 namespace {
-// T_j = 1.5 I - 0.5 G_j for square blocks (off, k)
+// Symmetric k x k blocks G_j = sum A^T A at off, formed as the lower triangle only (see add_gram): an
+// element (r, c), r >= c, is at off + r + c k.
 struct NsJob { long long off; int k, pad_; };
+__device__ __forceinline__ double gram_at(const double* G, const NsJob& j, int r, int c) {
+    return G[j.off + max(r, c) + (long long)min(r, c) * j.k];
+}
+// T_j = 1.5 I - 0.5 G_j
 __global__ void k_ns_prep(const NsJob* jobs, const double* G, double* T) {
     const NsJob j = jobs[blockIdx.y];
-    long long total = (long long)j.k * j.k;
-    for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (long long)gridDim.x * blockDim.x) {
-        int r = (int)(e / j.k), c = (int)(e % j.k);
-        T[j.off + e] = (r == c ? 1.5 : 0.0) - 0.5 * G[j.off + e];
+    const int total = j.k * j.k;
+    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < total; e += gridDim.x * blockDim.x) {
+        const int c = e / j.k, r = e - c * j.k;
+        T[j.off + e] = (r == c ? 1.5 : 0.0) - 0.5 * gram_at(G, j, r, c);
     }
 }
-}  // namespace
-
-namespace {
-// max over sectors of |G - I|_max, written by one block per sector into dev[s]
-struct DevJob { long long off; int k, pad_; };
-__global__ void k_gram_dev(const DevJob* jobs, const double* G, double* dev) {
-    const DevJob j = jobs[blockIdx.x];
-    double m = 0.0;
-    const long long total = (long long)j.k * j.k;
-    for (long long e = threadIdx.x; e < total; e += blockDim.x) {
-        int r = (int)(e / j.k), c = (int)(e % j.k);
-        m = fmax(m, fabs(G[j.off + e] - (r == c ? 1.0 : 0.0)));
+// dev[s] = max |G - I| of block s (zeroed before; non-negative doubles order like their bits).  CTAs
+// share a block: one CTA each took 1.2 ms for the blocks of an m = 2000 bond.
+__global__ void k_gram_dev(const NsJob* jobs, const double* G, unsigned long long* dev) {
+    const NsJob j = jobs[blockIdx.y];
+    unsigned long long m = 0;
+    for (int c = blockIdx.x; c < j.k; c += gridDim.x)
+        for (int r = c + threadIdx.x; r < j.k; r += blockDim.x) {
+            const double d = fabs(G[j.off + r + (long long)c * j.k] - (r == c ? 1.0 : 0.0));
+            const unsigned long long b = (unsigned long long)__double_as_longlong(d);
+            if (d == d && b > m) m = b;
+        }
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long w = __shfl_xor_sync(0xffffffffu, m, o);
+        m = w > m ? w : m;
     }
-    for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-    __shared__ double red[32];
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double x = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) x = fmax(x, red[w]);
-        dev[blockIdx.x] = x;
+    if ((threadIdx.x & 31) == 0 && m) atomicMax(dev + blockIdx.y, m);
+}
+
+// max |G - I| over all blocks, on the host.
+double gram_deviation(const DBuf& djobs, const std::vector<NsJob>& jobs, const DBuf& G, DBuf& dev, cudaStream_t st) {
+    const int n = (int)jobs.size();
+    int kmax = 1;
+    for (const NsJob& j : jobs) kmax = std::max(kmax, j.k);
+    dev.ensure((size_t)n * 8, st);
+    PD_CK(cudaMemsetAsync(dev.p, 0, (size_t)n * 8, st));
+    k_gram_dev<<<dim3(std::min(kmax, 32), (unsigned)n), 128, 0, st>>>(djobs.as<NsJob>(), G.as<double>(),
+                                                                      dev.as<unsigned long long>());
+    PD_LAUNCHED();
+    std::vector<double> h(n);
+    PD_CK(cudaMemcpyAsync(h.data(), dev.p, (size_t)n * 8, cudaMemcpyDeviceToHost, st));
+    PD_CK(cudaStreamSynchronize(st));
+    double worst = 0.0;
+    for (double v : h) worst = std::max(worst, v);
+    return worst;
+}
+
+// Adds to g the lower triangle of the k x k Gram block at c_off, 64 columns at a time: half the work of
+// the square.  Column i of segment s starts at segs[s].a_off + i sam; strides as for GemmBatch::add.
+void add_gram(GemmBatch& g, int k, long long c_off, int sam, int sak, const std::vector<GSeg>& segs, int accumulate = 0) {
+    for (int j0 = 0; j0 < k; j0 += 64) {
+        std::vector<GSeg> sg = segs;
+        for (GSeg& x : sg) {
+            x.a_off += (long long)j0 * sam;
+            x.b_off = x.a_off;
+        }
+        g.add(k - j0, std::min(64, k - j0), c_off + j0 + (long long)j0 * k, sam, sak, sam, sak, 1, k, sg, accumulate);
     }
 }
 }  // namespace
@@ -346,21 +376,17 @@ void orthonormalize_factor(const Sec& bl, const Sec& br, const std::vector<int>&
     const Sec& mid = left ? br : bl;            // the bond carrying the kept index
     std::vector<long long> goff(mid.n() + 1, 0);
     for (int i = 0; i < mid.n(); ++i) goff[i + 1] = goff[i] + (long long)mid.m[i] * mid.m[i];
-    DBuf G, T, out, dev, dj, djd;
+    DBuf G, T, out, dev, dj;
     G.ensure(std::max<long long>(1, goff.back()) * 8, st);
     T.ensure(std::max<long long>(1, goff.back()) * 8, st);
     out.ensure(std::max<long long>(1, S.size) * 8, st);
-    dev.ensure(std::max(1, mid.n()) * 8, st);
     std::vector<NsJob> jobs;
-    std::vector<DevJob> djobs;
     int mx = 1;
     for (int j = 0; j < mid.n(); ++j) {
         jobs.push_back({goff[j], mid.m[j], 0});
-        djobs.push_back({goff[j], mid.m[j], 0});
         mx = std::max(mx, mid.m[j] * mid.m[j]);
     }
     upload(dj, jobs, st);
-    upload(djd, djobs, st);
     GemmBatch gA;
     for (const auto& b : S.blk) {
         if (left) {
@@ -371,37 +397,27 @@ void orthonormalize_factor(const Sec& bl, const Sec& br, const std::vector<int>&
             gA.add(b.cols, k, b.off, 1, b.cols, k, 1, 1, b.cols, {GSeg{b.off, goff[b.i], k, 0}});
         }
     }
-    GemmBatch gG;
-    std::vector<GemmBatch> per_block;
+    // G_j = sum over the blocks of sector j of A^T A (left: all blocks share k_j columns, one problem)
+    // or B B^T (right: the blocks' row strides differ, so the n-th block of every sector goes into the
+    // n-th, accumulating launch)
+    std::vector<GemmBatch> gG;
     if (left) {
-        // G_j = sum over the blocks (a, s) of sector j of A^T A; all blocks share k_j columns
+        gG.emplace_back();
         std::vector<std::vector<GSeg>> segs(mid.n());
         for (const auto& b : S.blk) segs[b.j].push_back({b.off, b.off, b.rows, 0});
-        for (int j = 0; j < mid.n(); ++j) gG.add(mid.m[j], mid.m[j], goff[j], 1, mid.m[j], 1, mid.m[j], 1, mid.m[j], segs[j]);
+        for (int j = 0; j < mid.n(); ++j) add_gram(gG[0], mid.m[j], goff[j], 1, mid.m[j], segs[j]);
     } else {
-        // G_j = sum over the blocks of B B^T; row strides differ per block, so one accumulating
-        // launch per block (stream order serialises them)
-        std::vector<int> first(mid.n(), 1);
+        std::vector<int> nth(mid.n(), 0);
         for (const auto& b : S.blk) {
-            per_block.emplace_back();
-            int k = b.rows;
-            per_block.back().add(k, k, goff[b.i], b.cols, 1, b.cols, 1, 1, k, {GSeg{b.off, b.off, b.cols, 0}},
-                                 first[b.i] ? 0 : 1);
-            first[b.i] = 0;
+            const int t = nth[b.i]++;
+            if ((int)gG.size() <= t) gG.emplace_back();
+            add_gram(gG[t], b.rows, goff[b.i], b.cols, 1, {GSeg{b.off, b.off, b.cols, 0}}, t > 0);
         }
     }
-    std::vector<double> hdev(mid.n());
     for (int iter = 0; iter < 6; ++iter) {
         PD_CK(cudaMemsetAsync(G.p, 0, std::max<long long>(1, goff.back()) * 8, st));
-        if (left) run_gemm64(gG, X, X, G.as<double>(), st);
-        else
-            for (auto& g1 : per_block) run_gemm64(g1, X, X, G.as<double>(), st);
-        k_gram_dev<<<mid.n(), 256, 0, st>>>(djd.as<DevJob>(), G.as<double>(), dev.as<double>());
-        PD_LAUNCHED();
-        PD_CK(cudaMemcpyAsync(hdev.data(), dev.p, mid.n() * 8, cudaMemcpyDeviceToHost, st));
-        PD_CK(cudaStreamSynchronize(st));
-        double worst = 0.0;
-        for (double v : hdev) worst = std::max(worst, v);
+        for (auto& g1 : gG) run_gemm64(g1, X, X, G.as<double>(), st);
+        const double worst = gram_deviation(dj, jobs, G, dev, st);
         PD_REQUIRE(std::isfinite(worst) && worst < 0.9, DMRG_ERR_NUMERIC,
                    "kept singular vectors too far from orthonormal for the FP64 re-orthonormalisation (|I - X^T X| = " +
                        std::to_string(worst) + " at iteration " + std::to_string(iter) + ")");
@@ -435,7 +451,6 @@ void convert_flat(const void* src, Num in, void* dst, Num out, long long n, cuda
 
 void orthonormalize_square(const std::vector<SvdSec>& ss, double* V, cudaStream_t st, int max_iter) {
     std::vector<NsJob> jobs;
-    std::vector<DevJob> djobs;
     GemmBatch gG, gX;
     long long tot = 0;
     int mx = 1;
@@ -443,31 +458,22 @@ void orthonormalize_square(const std::vector<SvdSec>& ss, double* V, cudaStream_
         if (x.n <= 0) continue;
         const int n = x.n;
         jobs.push_back({x.v_off, n, 0});
-        djobs.push_back({x.v_off, n, 0});
         mx = std::max(mx, n * n);
         // G = V^T V:  G(i, j) = sum_k V(k, i) V(k, j), V column-major (V(r, c) = V[off + r + c n])
-        gG.add(n, n, x.v_off, n, 1, n, 1, n, 1, {GSeg{x.v_off, x.v_off, n, 0}});
+        add_gram(gG, n, x.v_off, n, 1, {GSeg{x.v_off, x.v_off, n, 0}});
         // V' = V T:   V'(r, c) = sum_u V(r, u) T(u, c), T symmetric
         gX.add(n, n, x.v_off, 1, n, n, 1, 1, n, {GSeg{x.v_off, x.v_off, n, 0}});
         tot = std::max(tot, x.v_off + (long long)n * n);
     }
     if (jobs.empty()) return;
-    DBuf G, T, out, dev, dj, djd;
+    DBuf G, T, out, dev, dj;
     G.ensure(tot * 8, st);
     T.ensure(tot * 8, st);
     out.ensure(tot * 8, st);
-    dev.ensure(jobs.size() * 8, st);
     upload(dj, jobs, st);
-    upload(djd, djobs, st);
-    std::vector<double> hdev(jobs.size());
     for (int iter = 0; iter < max_iter; ++iter) {
         run_gemm64(gG, V, V, G.as<double>(), st);
-        k_gram_dev<<<(unsigned)jobs.size(), 256, 0, st>>>(djd.as<DevJob>(), G.as<double>(), dev.as<double>());
-        PD_LAUNCHED();
-        PD_CK(cudaMemcpyAsync(hdev.data(), dev.p, jobs.size() * 8, cudaMemcpyDeviceToHost, st));
-        PD_CK(cudaStreamSynchronize(st));
-        double worst = 0.0;
-        for (double v : hdev) worst = std::max(worst, v);
+        const double worst = gram_deviation(dj, jobs, G, dev, st);
         PD_REQUIRE(std::isfinite(worst) && worst < 0.5, DMRG_ERR_NUMERIC,
                    "FP32 Jacobi rotations too far from orthogonal for the FP64 polish (|V^T V - I| = " +
                        std::to_string(worst) + " at iteration " + std::to_string(iter) + ")");
@@ -1375,10 +1381,7 @@ bool polish64(const std::vector<SvdSec>& ss, const SvdSec* dsecs, DBuf& dW, DBuf
     for (int s = 0; s < nsec; ++s) {
         const SvdSec& x = ss[s];
         for (int j = 0; j < x.n; ++j) cols.push_back({s, j});
-        // lower block triangle of G, 64 columns at a time
-        for (int j0 = 0; j0 < x.n; j0 += 64)
-            gG.add(x.n - j0, std::min(64, x.n - j0), x.v_off + j0 + (long long)j0 * x.n, x.p, 1, x.p, 1, 1, x.n,
-                   {GSeg{x.w_off + (long long)j0 * x.p, x.w_off + (long long)j0 * x.p, x.p, 0}});
+        add_gram(gG, x.n, x.v_off, x.p, 1, {GSeg{x.w_off, x.w_off, x.p, 0}});
         gW.add(x.p, x.n, x.w_off, 1, x.p, x.n, 1, 1, x.p, {GSeg{x.w_off, x.v_off, x.n, 0}}, 1);
         gV.add(x.n, x.n, x.v_off, 1, x.n, x.n, 1, 1, x.n, {GSeg{x.v_off, x.v_off, x.n, 0}}, 1);
         gE.add(x.n, x.n, x.v_off, 1, x.n, x.n, 1, 1, x.n, {GSeg{x.v_off, x.v_off, x.n, 0}}, 1, 0.5);
@@ -1566,7 +1569,7 @@ void jacobi64(std::vector<SvdSec>& ss, DBuf& dWbuf, DBuf& dsecs, DBuf& dV, DBuf&
                               dWbuf.as<double>(), dV.as<double>(), 4.0 * DBL_EPSILON, 0.0, nullptr, drot.as<int>(),
                               drot.as<int>() + max_sweeps, bar, bar + 3, st);
     double* W = dWbuf.as<double>();
-    launch_svd_finish<double>(dsecs.as<SvdSec>(), nsec, W, dsig.as<double>(), dord.as<int>(), st);
+    launch_svd_finish<double>(dsecs.as<SvdSec>(), nsec, maxn, W, dsig.as<double>(), dord.as<int>(), st);
     unsigned err = 0;
     PD_CK(cudaMemcpyAsync(&err, bar + 3, 4, cudaMemcpyDeviceToHost, st));
     PD_CK(cudaStreamSynchronize(st));
@@ -1696,7 +1699,9 @@ void accurate_refine(const std::vector<SvdSec>& ss, const SvdSec* dsecs, double*
     }
     col_copy(sw, dT.as<double>(), W, nullptr, st);
     col_copy(sv, dVn.as<double>(), V, nullptr, st);
-    launch_svd_finish<double>(dsecs, nsec, W, sig, ord, st);
+    int maxn = 0;
+    for (const SvdSec& x : ss) maxn = std::max(maxn, x.n);
+    launch_svd_finish<double>(dsecs, nsec, maxn, W, sig, ord, st);
 }
 
 }  // namespace
@@ -1839,7 +1844,7 @@ std::vector<SplitResult> svd_split_batch(const std::vector<SplitReq>& reqs, bool
             qp.finish<float>(dW.as<float>(), dV.as<float>(), dVJ.as<float>(), dWo.as<float>(), st);
             dW = std::move(dWo);
         }
-        launch_svd_finish<float>(dsecs.as<SvdSec>(), nsec, dW.as<float>(), dsig.as<double>(), dord.as<int>(), st);
+        launch_svd_finish<float>(dsecs.as<SvdSec>(), nsec, maxn, dW.as<float>(), dsig.as<double>(), dord.as<int>(), st);
     } else {
         for (int q = 0; q < nreq; ++q) run_copy<double>(gather[q], reqs[q].psi, dW.p, Num::F64, st);
         DBuf dM;
@@ -1860,7 +1865,7 @@ std::vector<SplitResult> svd_split_batch(const std::vector<SplitReq>& reqs, bool
             launch_jacobi<double>(dsecs.as<SvdSec>(), nsec, dpairs.as<int>(), npairs, maxnpad, max_sweeps,
                                   dW.as<double>(), dV.as<double>(), tol, 0.0, nullptr, drot.as<int>(),
                                   drot.as<int>() + max_sweeps, bar, jerr, st);
-        launch_svd_finish<double>(dsecs.as<SvdSec>(), nsec, dW.as<double>(), dsig.as<double>(), dord.as<int>(), st);
+        launch_svd_finish<double>(dsecs.as<SvdSec>(), nsec, maxn, dW.as<double>(), dsig.as<double>(), dord.as<int>(), st);
         if (accurate && woff > 0)
             accurate_refine(ss, dsecs.as<SvdSec>(), dW.as<double>(), dV.as<double>(), dsig.as<double>(),
                             dord.as<int>(), dM.as<double>(), 0, st);
@@ -1895,7 +1900,7 @@ std::vector<SplitResult> svd_split_batch(const std::vector<SplitReq>& reqs, bool
     DBuf dtl, tsd, tsi;
     upload(dtl, tl, st);
     tsd.ensure((size_t)(max_total + max_nsec + 1) * 8, st);
-    tsi.ensure((size_t)(3 * max_total + 1) * 4, st);
+    tsi.ensure((size_t)(2 * max_total + 1) * 4, st);
     // an FP32 SVD reports exact zeros at ~1e-7 of the largest singular value: keep its cutoff
     // above that noise floor (the discarded weight stays below 1e-10)
     for (int q = 0; q < nreq; ++q) {
