@@ -14,9 +14,6 @@
 // every entry W1 x W2 can produce (not only the nonzero entries of their product), so W1bar and
 // W2bar are exact at every nonzero entry of W1 and W2; entries that are zero in W1 (resp. W2)
 // get no gradient (the structure of the MPO is fixed).
-#include <map>
-#include <tuple>
-
 #include "plans.h"
 
 namespace pd {
@@ -72,12 +69,14 @@ std::vector<GTile> square_tiles(const std::vector<GProb>& probs, int edge) {
 void gemm64(const std::vector<GProb>& p, const std::vector<GSeg>& s, const double* A, const double* B, double* C,
             cudaStream_t st) {
     if (p.empty()) return;
-    DBuf dp, ds, dt;
+    DBuf lists, dp, ds, dt;
     const F64Shape shape = f64_shape(p, s);
     const std::vector<GTile> t = square_tiles(p, shape.tile);
-    upload(dp, p, st);
-    upload(ds, s, st);
-    upload(dt, t, st);
+    ListPack pk;
+    pk.add(dp, p);
+    pk.add(ds, s);
+    pk.add(dt, t);
+    pk.upload(lists, st);
     launch_gemm_f64(dp.as<GProb>(), ds.as<GSeg>(), dt.as<GTile>(), (int)t.size(), shape.tile, shape, A, B, C, st);
 }
 
@@ -136,9 +135,10 @@ void heff_backward(const Sec& bl, const Sec& br, const std::vector<int>& qn, con
             }
         // mix terms from the nonzero two-site MPO entries: Y(o, w2) += v X(w, b)
         std::vector<std::vector<std::pair<int, double>>> yterm(yb.size()), xterm(xb.size());
+        std::vector<std::vector<int>> by_pair((size_t)d * d);   // psi blocks of each (s1, s2)
+        for (int b = 0; b < nb; ++b) by_pair[(size_t)pb[b].s1 * d + pb[b].s2].push_back(b);
         for (const auto& e : t.nz)
-            for (int b = 0; b < nb; ++b) {
-                if (pb[b].s1 != e.s1p || pb[b].s2 != e.s2p) continue;
+            for (const int b : by_pair[(size_t)e.s1p * d + e.s2p]) {
                 const int xi = xidx[(size_t)e.w * nb + b];
                 if (xi < 0) continue;
                 const int o = P.at(xb[xi].iab, e.s1, e.s2);
@@ -192,11 +192,13 @@ void heff_backward(const Sec& bl, const Sec& br, const std::vector<int>& qn, con
                 el.push_back((long long)j.rows * j.cols);
             }
             if (!mj.empty()) {
-                DBuf dj, dt2, dc;
+                DBuf lists, dj, dt2, dc;
                 const std::vector<int2> ch = make_chunks(el);
-                upload(dj, mj, st);
-                upload(dt2, mt, st);
-                upload(dc, ch, st);
+                ListPack pk;
+                pk.add(dj, mj);
+                pk.add(dt2, mt);
+                pk.add(dc, ch);
+                pk.upload(lists, st);
                 launch_mix<double, double>(dj.as<MixJob>(), dc.as<int2>(), (int)ch.size(), dt2.as<MixTerm>(), X, Y, st);
             }
         }
@@ -247,11 +249,13 @@ void heff_backward(const Sec& bl, const Sec& br, const std::vector<int>& qn, con
                 el.push_back((long long)j.rows * j.cols);
             }
             if (!mj.empty()) {
-                DBuf dj, dt2, dc;
+                DBuf lists, dj, dt2, dc;
                 const std::vector<int2> ch = make_chunks(el);
-                upload(dj, mj, st);
-                upload(dt2, mt, st);
-                upload(dc, ch, st);
+                ListPack pk;
+                pk.add(dj, mj);
+                pk.add(dt2, mt);
+                pk.add(dc, ch);
+                pk.upload(lists, st);
                 launch_mix<double, double>(dj.as<MixJob>(), dc.as<int2>(), (int)ch.size(), dt2.as<MixTerm>(), Yb, Xb, st);
             }
         }
@@ -299,31 +303,33 @@ void heff_backward(const Sec& bl, const Sec& br, const std::vector<int>& qn, con
         if (W1bar || W2bar) {
             struct Combo { int w, s1, s1p, s2, s2p, w2; };
             std::vector<Combo> combos;
-            std::map<std::tuple<int, int, int, int, int, int>, int> cidx;
+            std::vector<int> cidx((size_t)w1.Dl * d * d * d * d * w2.Dr, -1);
             // pairs (W1 entry, W2 entry, combo)
             struct Pair { long long i1, i2; int c; };
             std::vector<Pair> pairs;
+            struct E2 { int s2, s2p, w2; long long i2; };   // nonzero entries of W2 by its left channel
+            std::vector<std::vector<E2>> second(w2.Dl);
+            for (int wp = 0; wp < w2.Dl; ++wp)
+                for (int s2 = 0; s2 < d; ++s2)
+                    for (int s2p = 0; s2p < d; ++s2p)
+                        for (int w2i = 0; w2i < w2.Dr; ++w2i) {
+                            const long long i2 = (((long long)wp * d + s2) * d + s2p) * w2.Dr + w2i;
+                            if (w2.W[i2] != 0.0) second[wp].push_back({s2, s2p, w2i, i2});
+                        }
             for (int w = 0; w < w1.Dl; ++w)
                 for (int s1 = 0; s1 < d; ++s1)
                     for (int s1p = 0; s1p < d; ++s1p)
                         for (int wp = 0; wp < w1.Dr; ++wp) {
                             const long long i1 = (((long long)w * d + s1) * d + s1p) * w1.Dr + wp;
                             if (w1.W[i1] == 0.0) continue;
-                            for (int s2 = 0; s2 < d; ++s2)
-                                for (int s2p = 0; s2p < d; ++s2p)
-                                    for (int w2i = 0; w2i < w2.Dr; ++w2i) {
-                                        const long long i2 = (((long long)wp * d + s2) * d + s2p) * w2.Dr + w2i;
-                                        if (w2.W[i2] == 0.0) continue;
-                                        auto key = std::make_tuple(w, s1, s1p, s2, s2p, w2i);
-                                        auto it = cidx.find(key);
-                                        int c;
-                                        if (it == cidx.end()) {
-                                            c = (int)combos.size();
-                                            cidx[key] = c;
-                                            combos.push_back({w, s1, s1p, s2, s2p, w2i});
-                                        } else c = it->second;
-                                        pairs.push_back({i1, i2, c});
-                                    }
+                            for (const E2& e : second[wp]) {
+                                int& c = cidx[(((((size_t)w * d + s1) * d + s1p) * d + e.s2) * d + e.s2p) * w2.Dr + e.w2];
+                                if (c < 0) {
+                                    c = (int)combos.size();
+                                    combos.push_back({w, s1, s1p, e.s2, e.s2p, e.w2});
+                                }
+                                pairs.push_back({i1, e.i2, c});
+                            }
                         }
             // dot jobs per combo (in combo order) over the psi blocks it connects
             std::vector<DotJob> jobs;
@@ -331,8 +337,7 @@ void heff_backward(const Sec& bl, const Sec& br, const std::vector<int>& qn, con
             for (size_t c = 0; c < combos.size(); ++c) {
                 jt0[c] = (int)jidx.size();
                 const Combo& C = combos[c];
-                for (int b = 0; b < nb; ++b) {
-                    if (pb[b].s1 != C.s1p || pb[b].s2 != C.s2p) continue;
+                for (const int b : by_pair[(size_t)C.s1p * d + C.s2p]) {
                     const int xi = xidx[(size_t)C.w * nb + b];
                     if (xi < 0) continue;
                     const int o = P.at(xb[xi].iab, C.s1, C.s2);
@@ -344,11 +349,15 @@ void heff_backward(const Sec& bl, const Sec& br, const std::vector<int>& qn, con
                 }
             }
             jt0[combos.size()] = (int)jidx.size();
-            DBuf dj, dpart, djt0, djidx, dW12;
-            upload(dj, jobs, st);
+            DBuf lists, dj, dpart, djt0, djidx, dW12;
+            {
+                ListPack pk;
+                pk.add(dj, jobs);
+                pk.add(djt0, jt0);
+                pk.add(djidx, jidx);
+                pk.upload(lists, st);
+            }
             dpart.ensure(std::max<size_t>(1, jobs.size()) * 8, st);
-            upload(djt0, jt0, st);
-            upload(djidx, jidx, st);
             dW12.ensure(std::max<size_t>(1, combos.size()) * 8, st);
             if (!jobs.empty()) {
                 k_block_dot<<<(unsigned)jobs.size(), 256, 0, st>>>(dj.as<DotJob>(), Yb, X, dpart.as<double>());
@@ -360,31 +369,45 @@ void heff_backward(const Sec& bl, const Sec& br, const std::vector<int>& qn, con
                                                                               dW12.as<double>());
                 PD_LAUNCHED();
             }
-            // W1bar[i1] = sum over its pairs W12bar[c] W2[i2]; W2bar[i2] = sum W12bar[c] W1[i1]
+            // W1bar[i1] = sum over its pairs W12bar[c] W2[i2]; W2bar[i2] = sum W12bar[c] W1[i1]; only the
+            // entries that have pairs are computed, the others are zero
             auto reduce = [&](bool first, double* out) {
                 if (!out) return;
-                const size_t nout = first ? w1.W.size() : w2.W.size();
-                std::vector<std::vector<std::pair<int, double>>> lst(nout);
-                for (const auto& pr : pairs)
-                    if (first) lst[pr.i1].push_back({pr.c, w2.W[pr.i2]});
-                    else lst[pr.i2].push_back({pr.c, w1.W[pr.i1]});
-                std::vector<int> t0(nout + 1, 0), idx;
-                std::vector<double> coef;
-                for (size_t i = 0; i < nout; ++i) {
-                    t0[i] = (int)idx.size();
-                    for (auto& e : lst[i]) { idx.push_back(e.first); coef.push_back(e.second); }
+                const std::vector<double>& mine = first ? w1.W : w2.W;
+                const std::vector<double>& other = first ? w2.W : w1.W;
+                std::vector<int> slot(mine.size(), 0), t0{0}, idx(pairs.size());
+                std::vector<long long> at;                  // entry of slot i
+                std::vector<double> coef(pairs.size());
+                for (const auto& pr : pairs) ++slot[first ? pr.i1 : pr.i2];
+                for (size_t i = 0; i < mine.size(); ++i)
+                    if (slot[i]) {
+                        t0.push_back(t0.back() + slot[i]);
+                        slot[i] = (int)at.size();
+                        at.push_back((long long)i);
+                    }
+                std::vector<int> next(t0.begin(), t0.end());
+                for (const auto& pr : pairs) {
+                    const int k = next[slot[first ? pr.i1 : pr.i2]]++;
+                    idx[k] = pr.c;
+                    coef[k] = other[first ? pr.i2 : pr.i1];
                 }
-                t0[nout] = (int)idx.size();
-                DBuf dt0, didx, dco, dout;
-                upload(dt0, t0, st);
-                upload(didx, idx, st);
-                upload(dco, coef, st);
-                dout.ensure(std::max<size_t>(1, nout) * 8, st);
-                k_gather_sum<<<((int)nout + 127) / 128, 128, 0, st>>>(dt0.as<int>(), didx.as<int>(), dco.as<double>(),
-                                                                     dW12.as<double>(), (int)nout, dout.as<double>());
+                std::fill(out, out + mine.size(), 0.0);
+                if (at.empty()) return;
+                DBuf own, dt0, didx, dco, dout;
+                ListPack pk;
+                pk.add(dt0, t0);
+                pk.add(didx, idx);
+                pk.add(dco, coef);
+                pk.upload(own, st);
+                dout.ensure(at.size() * 8, st);
+                k_gather_sum<<<((int)at.size() + 127) / 128, 128, 0, st>>>(dt0.as<int>(), didx.as<int>(), dco.as<double>(),
+                                                                          dW12.as<double>(), (int)at.size(),
+                                                                          dout.as<double>());
                 PD_LAUNCHED();
-                PD_CK(cudaMemcpyAsync(out, dout.p, nout * 8, cudaMemcpyDeviceToHost, st));
+                std::vector<double> h(at.size());
+                PD_CK(cudaMemcpyAsync(h.data(), dout.p, at.size() * 8, cudaMemcpyDeviceToHost, st));
                 PD_CK(cudaStreamSynchronize(st));
+                for (size_t i = 0; i < at.size(); ++i) out[at[i]] = h[i];
             };
             reduce(true, W1bar);
             reduce(false, W2bar);

@@ -94,7 +94,8 @@ struct StreamHolder {
 }  // namespace
 
 struct dmrg_ctx {
-    StreamHolder streams;                            // first member: destroyed last
+    PoolHold pool;                                   // first members: destroyed last
+    StreamHolder streams;
     int L = 0, d = 0, qtot = 0;
     std::vector<int> qn;
     std::vector<SiteMPO> W;
@@ -844,26 +845,6 @@ struct EmuGuard {
         return DMRG_ERR_STATE;                                \
     }
 
-namespace {
-// Work buffers come from the device's default stream-ordered pool.  With its default release
-// threshold (0) every stream synchronisation hands freed memory back to the driver, and the next
-// allocation maps it again; region threads that synchronise independently then spend their time
-// re-mapping.  Keep freed memory in the pool instead (process-wide, set once).
-void keep_pool_memory() {
-    static const cudaError_t st = [] {
-        int dev = 0;
-        cudaError_t e = cudaGetDevice(&dev);
-        if (e != cudaSuccess) return e;
-        cudaMemPool_t pool;
-        e = cudaDeviceGetDefaultMemPool(&pool, dev);
-        if (e != cudaSuccess) return e;
-        uint64_t keep = UINT64_MAX;
-        return cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
-    }();
-    PD_CK(st);
-}
-}  // namespace
-
 extern "C" {
 
 dmrg_status dmrg_init_mpo(dmrg_ctx** out, const dmrg_mpo_desc* mpo, const dmrg_config* cfg) {
@@ -876,7 +857,6 @@ dmrg_status dmrg_init_mpo(dmrg_ctx** out, const dmrg_mpo_desc* mpo, const dmrg_c
     PD_REQUIRE(cfg->precision == DMRG_FP64 || cfg->precision == DMRG_TF32 || cfg->precision == DMRG_BF16,
                DMRG_ERR_ARG, "unknown precision");
     PD_REQUIRE(cfg->precision == DMRG_FP64 || tc_available(), DMRG_ERR_STATE, "tensor-core engine unavailable");
-    keep_pool_memory();
     std::unique_ptr<dmrg_ctx> C(new dmrg_ctx());
     c = C.get();
     C->L = mpo->n_sites;

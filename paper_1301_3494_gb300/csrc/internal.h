@@ -33,6 +33,17 @@ struct Error {
         if (!(cond)) throw ::pd::Error{code, what};                                       \
     } while (0)
 
+// Stream-ordered device memory from the library's pool on the current device (pool.cu); freed with
+// cudaFreeAsync.  A PoolHold makes the pool keep all freed memory while it lives.
+void* pool_alloc(size_t bytes, cudaStream_t st);
+struct PoolHold {
+    int dev = 0;
+    PoolHold();
+    ~PoolHold();
+    PoolHold(const PoolHold&) = delete;
+    PoolHold& operator=(const PoolHold&) = delete;
+};
+
 // Kernel launches issued by the library (process-wide counter).
 extern std::atomic<long long> g_launches;
 #define PD_LAUNCHED()                                                   \
@@ -171,6 +182,9 @@ void launch_diag(const DiagJob* jobs, const int2* chunks, int nchunks, const Dia
 // Chunk table for jobs of the given element counts.
 inline std::vector<int2> make_chunks(const std::vector<long long>& elems) {
     std::vector<int2> c;
+    size_t n = 0;
+    for (long long e : elems) n += (size_t)((e + CHUNK - 1) / CHUNK);
+    c.reserve(n);
     for (size_t j = 0; j < elems.size(); ++j)
         for (long long e = 0; e < elems[j]; e += CHUNK) c.push_back(make_int2((int)j, (int)e));
     return c;

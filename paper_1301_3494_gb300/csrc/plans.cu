@@ -3,7 +3,6 @@
 #include <cmath>
 #include <cstring>
 #include <map>
-#include <tuple>
 
 #include "plans.h"
 
@@ -81,50 +80,87 @@ TwoSiteMPO two_site_mpo(const SiteMPO& a, const SiteMPO& b) {
     T.d = d;
     T.f0 = a.fl;
     T.f2 = b.fr;
-    std::vector<double> acc((size_t)a.Dl * d * d * d * d * b.Dr, 0.0);
-    auto idx = [&](int w, int s1, int s1p, int s2, int s2p, int w2) {
-        return (((((size_t)w * d + s1) * d + s1p) * d + s2) * d + s2p) * b.Dr + w2;
-    };
-    for (int w = 0; w < a.Dl; ++w)
+    // nonzero entries of W2 by its left channel; one left channel's entries are summed in a dense
+    // scratch indexed [s1][s1'][s2][s2'][w2]
+    struct E2 { int s2, s2p, w2; double y; };
+    std::vector<std::vector<E2>> second(b.Dl);
+    for (int w1 = 0; w1 < b.Dl; ++w1)
+        for (int s2 = 0; s2 < d; ++s2)
+            for (int s2p = 0; s2p < d; ++s2p)
+                for (int w2 = 0; w2 < b.Dr; ++w2) {
+                    const double y = b.at(w1, s2, s2p, w2);
+                    if (y != 0.0) second[w1].push_back({s2, s2p, w2, y});
+                }
+    const int n = d * d * d * d * b.Dr;
+    std::vector<double> acc(n, 0.0);
+    std::vector<char> seen(n, 0);
+    std::vector<int> touched;
+    for (int w = 0; w < a.Dl; ++w) {
+        touched.clear();
         for (int s1 = 0; s1 < d; ++s1)
             for (int s1p = 0; s1p < d; ++s1p)
                 for (int w1 = 0; w1 < a.Dr; ++w1) {
-                    double x = a.at(w, s1, s1p, w1);
+                    const double x = a.at(w, s1, s1p, w1);
                     if (x == 0.0) continue;
-                    for (int s2 = 0; s2 < d; ++s2)
-                        for (int s2p = 0; s2p < d; ++s2p)
-                            for (int w2 = 0; w2 < b.Dr; ++w2) {
-                                double y = b.at(w1, s2, s2p, w2);
-                                if (y != 0.0) acc[idx(w, s1, s1p, s2, s2p, w2)] += x * y;
-                            }
-                }
-    for (int w = 0; w < a.Dl; ++w)
-        for (int s1 = 0; s1 < d; ++s1)
-            for (int s1p = 0; s1p < d; ++s1p)
-                for (int s2 = 0; s2 < d; ++s2)
-                    for (int s2p = 0; s2p < d; ++s2p)
-                        for (int w2 = 0; w2 < b.Dr; ++w2) {
-                            double v = acc[idx(w, s1, s1p, s2, s2p, w2)];
-                            if (v != 0.0) T.nz.push_back({w, s1, s1p, s2, s2p, w2, v});
+                    for (const E2& e : second[w1]) {
+                        const int i = (((s1 * d + s1p) * d + e.s2) * d + e.s2p) * b.Dr + e.w2;
+                        if (!seen[i]) {
+                            seen[i] = 1;
+                            touched.push_back(i);
                         }
+                        acc[i] += x * e.y;
+                    }
+                }
+        std::sort(touched.begin(), touched.end());
+        for (const int i : touched) {
+            const int w2 = i % b.Dr, s2p = i / b.Dr % d, s2 = i / b.Dr / d % d, s1p = i / b.Dr / d / d % d;
+            if (acc[i] != 0.0) T.nz.push_back({w, i / b.Dr / d / d / d, s1p, s2, s2p, w2, acc[i]});
+            acc[i] = 0.0;
+            seen[i] = 0;
+        }
+    }
     return T;
 }
 
 // ------------------------------------------------------------------------------------------
 // Batches and job lists
 // ------------------------------------------------------------------------------------------
-void GemmBatch::upload_tiles(int tm, int tn, cudaStream_t st) {
-    if (tile_m == tm && tile_n == tn && dtiles.p) return;
+static std::vector<GTile> tile_list(const std::vector<GProb>& probs, int tm, int tn) {
     std::vector<GTile> tiles;
+    tiles.reserve(probs.size());
     for (int p = 0; p < (int)probs.size(); ++p)
         for (int m0 = 0; m0 < probs[p].M; m0 += tm)
             for (int n0 = 0; n0 < probs[p].N; n0 += tn) tiles.push_back({p, m0, n0, 0});
+    return tiles;
+}
+
+void GemmBatch::upload_tiles(int tm, int tn, cudaStream_t st) {
+    if (tile_m == tm && tile_n == tn && dtiles.p) return;
+    const std::vector<GTile> tiles = tile_list(probs, tm, tn);
     ntiles = (int)tiles.size();
-    upload(dprobs, probs, st);
-    upload(dsegs, segs, st);
+    if (!dprobs.p) upload(dprobs, probs, st);
+    if (!dsegs.p) upload(dsegs, segs, st);
     upload(dtiles, tiles, st);
     tile_m = tm;
     tile_n = tn;
+}
+
+void GemmBatch::stage(ListPack& pk, int tm, int tn) {
+    if (empty()) return;
+    pk.add(dprobs, probs);
+    pk.add(dsegs, segs);
+    if (!tm) return;
+    const std::vector<GTile> tiles = tile_list(probs, tm, tn);
+    ntiles = (int)tiles.size();
+    pk.add(dtiles, tiles);
+    tile_m = tm;
+    tile_n = tn;
+}
+
+void GemmBatch::stage_f64(ListPack& pk) {
+    if (empty()) return;
+    f64 = f64_shape(probs, segs);
+    stage(pk, f64.tile, f64.tile);
 }
 
 // Whether a batch gains from the emulation.  Its plan is built on the host (one to several ms for the
@@ -443,7 +479,10 @@ void convert_flat(const void* src, Num in, void* dst, Num out, long long n, cuda
         j.srs = 0; j.scs = 1; j.drs = 0; j.dcs = 1; j.zero_to = 0; j.scale = 1.0;
         cl.add(j);
     }
-    cl.up(st);
+    ListPack pk;
+    DBuf lists;
+    cl.stage(pk);
+    pk.upload(lists, st);
     PD_REQUIRE(in == Num::F64 || in == Num::F32, DMRG_ERR_ARG, "convert_flat: source must be FP64 or FP32");
     if (in == Num::F64) run_copy<double>(cl, static_cast<const double*>(src), dst, out, st);
     else run_copy<float>(cl, static_cast<const float*>(src), dst, out, st);
@@ -543,6 +582,11 @@ std::unique_ptr<HeffPlan> make_heff_plan(const Sec& bl, const Sec& br, const std
     }
     P->psiT_rows = row;
 
+    // nonzero two-site entries by (s1, s2), ordered by w'' (and as listed within it)
+    std::vector<std::vector<int>> by_out((size_t)d * d);
+    for (int e = 0; e < (int)w12.nz.size(); ++e) by_out[(size_t)w12.nz[e].s1 * d + w12.nz[e].s2].push_back(e);
+    for (auto& v : by_out)
+        std::stable_sort(v.begin(), v.end(), [&](int x, int y) { return w12.nz[x].w2 < w12.nz[y].w2; });
     // which (w, s1', s2') combinations feed anything
     std::vector<char> used((size_t)w12.D0 * d * d, 0);
     for (const auto& e : w12.nz) used[((size_t)e.w * d + e.s1p) * d + e.s2p] = 1;
@@ -550,96 +594,102 @@ std::unique_ptr<HeffPlan> make_heff_plan(const Sec& bl, const Sec& br, const std
     // L stage: X[w, b] = L_w psi_b, block [a_bra][c].  X blocks that feed exactly one Y block,
     // and that Y block has no other term, are written by the GEMM epilogue straight into the Y
     // operand slab (coefficient as alpha); only the rest goes through X and the mixing kernel.
-    struct XB { int rows, cols, iab, lb, b; long long off; int fan; };
+    struct XB { int rows, cols, lb, b; long long off; int fan; };
     std::vector<XB> xs;
-    std::map<std::pair<int, int>, int> xidx;   // (w, b) -> X block
+    std::vector<int> xidx((size_t)w12.D0 * nb, -1);   // (w, b) -> X block
+    std::vector<int> raised((size_t)w12.D0 * bl.n()), lowered((size_t)w12.D0 * bl.n());
+    for (int w = 0; w < w12.D0; ++w)                  // left sector reached from i by channel w, and back
+        for (int i = 0; i < bl.n(); ++i) {
+            raised[(size_t)w * bl.n() + i] = bl.find(bl.q[i] + w12.f0[w]);
+            lowered[(size_t)w * bl.n() + i] = bl.find(bl.q[i] - w12.f0[w]);
+        }
     for (int b = 0; b < nb; ++b) {
         const auto& B = pb[b];
         for (int w = 0; w < w12.D0; ++w) {
             if (!used[((size_t)w * d + B.s1) * d + B.s2]) continue;
-            int iab = bl.find(bl.q[B.i] + w12.f0[w]);
+            const int iab = raised[(size_t)w * bl.n() + B.i];
             if (iab < 0) continue;
-            int lb = L.at(iab, w);
+            const int lb = L.at(iab, w);
             if (lb < 0) continue;
-            xidx[{w, b}] = (int)xs.size();
-            xs.push_back({bl.m[iab], B.cols, iab, lb, b, -1, 0});
+            xidx[(size_t)w * nb + b] = (int)xs.size();
+            xs.push_back({bl.m[iab], B.cols, lb, b, -1, 0});
         }
     }
     // MPO mix: Y[w2, o] = sum coef X[w, b]   (o = output block (iab, s1, s2))
-    std::map<std::pair<int, int>, std::vector<std::pair<int, double>>> yterms;   // (o, w2)
-    for (const auto& e : w12.nz) {
-        for (int b = 0; b < nb; ++b) {
-            const auto& B = pb[b];
-            if (B.s1 != e.s1p || B.s2 != e.s2p) continue;
-            auto it = xidx.find({e.w, b});
-            if (it == xidx.end()) continue;
-            int o = P->psi.at(xs[it->second].iab, e.s1, e.s2);
-            if (o < 0) continue;
-            int rb = R.at(pb[o].k, e.w2);
-            if (rb < 0) continue;
-            PD_REQUIRE(R.blk[rb].k == B.k, DMRG_ERR_QN, "MPO flux rule violated in the two-site operator");
-            yterms[{o, e.w2}].push_back({it->second, e.v});
-            xs[it->second].fan++;
-        }
-    }
-    // Y slab rows
+    struct YB { int o, rb, t0, nt; long long row; };
+    std::vector<YB> ys;
+    std::vector<std::pair<int, double>> yt;           // terms of the Y blocks: (X block, coefficient)
     long long yrow = 0;
-    std::map<std::pair<int, int>, long long> yrow_of;
-    for (auto& kv : yterms) {
-        yrow_of[kv.first] = yrow;
-        yrow += xs[kv.second.front().first].rows;
+    for (int o = 0; o < nb; ++o) {
+        const auto& O = pb[o];
+        int last = -1;
+        for (const int ei : by_out[(size_t)O.s1 * d + O.s2]) {
+            const auto& e = w12.nz[ei];
+            const int i = lowered[(size_t)e.w * bl.n() + O.i];
+            const int b = i < 0 ? -1 : P->psi.at(i, e.s1p, e.s2p);
+            const int xi = b < 0 ? -1 : xidx[(size_t)e.w * nb + b];
+            if (xi < 0) continue;
+            const int rb = R.at(O.k, e.w2);
+            if (rb < 0) continue;
+            PD_REQUIRE(R.blk[rb].k == pb[b].k, DMRG_ERR_QN, "MPO flux rule violated in the two-site operator");
+            if (e.w2 != last) {
+                ys.push_back({o, rb, (int)yt.size(), 0, yrow});
+                yrow += xs[xi].rows;
+                last = e.w2;
+            }
+            yt.push_back({xi, e.v});
+            ys.back().nt++;
+            xs[xi].fan++;
+        }
     }
     P->y_rows = yrow;
     // direct targets
-    std::vector<long long> direct_row(xs.size(), -1);
-    std::vector<double> direct_coef(xs.size(), 0.0);
-    for (auto& kv : yterms)
-        if (kv.second.size() == 1 && xs[kv.second[0].first].fan == 1) {
-            direct_row[kv.second[0].first] = yrow_of[kv.first];
-            direct_coef[kv.second[0].first] = kv.second[0].second;
-        }
+    std::vector<int> direct(xs.size(), -1);
+    for (int y = 0; y < (int)ys.size(); ++y)
+        if (ys[y].nt == 1 && xs[yt[ys[y].t0].first].fan == 1) direct[yt[ys[y].t0].first] = y;
     long long xoff = 0;
     for (size_t xi = 0; xi < xs.size(); ++xi) {
         XB& x = xs[xi];
         const auto& B = pb[x.b];
-        GSeg sg{prow[x.b] * P->ld_psi, L.blk[x.lb].row * L.ld, B.rows, 0};
-        if (direct_row[xi] >= 0) {
-            P->ldirect.add(x.cols, x.rows, direct_row[xi] * P->ld_y, P->ld_psi, 1, L.ld, 1, 1, P->ld_y, {sg}, 0,
-                           direct_coef[xi]);
+        const GSeg sg{prow[x.b] * P->ld_psi, L.blk[x.lb].row * L.ld, B.rows, 0};
+        if (direct[xi] >= 0) {
+            const YB& y = ys[direct[xi]];
+            P->ldirect.add(x.cols, x.rows, y.row * P->ld_y, P->ld_psi, 1, L.ld, 1, 1, P->ld_y, &sg, 1, 0, yt[y.t0].second);
         } else {
             x.off = xoff;
-            P->lstage.add(x.cols, x.rows, xoff, P->ld_psi, 1, L.ld, 1, 1, x.cols, {sg});
+            P->lstage.add(x.cols, x.rows, xoff, P->ld_psi, 1, L.ld, 1, 1, x.cols, &sg, 1, 0, 1.0);
             xoff += (long long)x.rows * x.cols;
         }
     }
     P->x_size = xoff;
     // mixing jobs for the remaining Y blocks, R-stage segments for all of them
-    std::map<int, std::vector<GSeg>> rsegs;
-    for (auto& kv : yterms) {
-        int o = kv.first.first, w2 = kv.first.second;
-        const XB& x0 = xs[kv.second.front().first];
-        const long long yr = yrow_of[kv.first];
-        P->mix.flops += 2.0 * x0.rows * x0.cols * (double)kv.second.size();
-        const bool direct = kv.second.size() == 1 && direct_row[kv.second[0].first] >= 0;
-        if (!direct) {
-            MixJob mj{};
-            mj.dst = yr * P->ld_y;
-            mj.rows = x0.rows;
-            mj.cols = x0.cols;
-            mj.ldo = P->ld_y;
-            mj.zero_to = kpad(x0.cols, prec);
-            mj.t0 = (int)P->mix.terms.size();
-            mj.nt = (int)kv.second.size();
-            for (auto& t : kv.second) P->mix.terms.push_back({xs[t.first].off, xs[t.first].cols, 0, t.second});
-            P->mix.jobs.push_back(mj);
-            P->mix.max_elems = std::max(P->mix.max_elems, mj.rows * std::max(mj.cols, mj.zero_to));
+    std::vector<GSeg> rs;
+    for (size_t y = 0; y < ys.size();) {
+        const int o = ys[y].o;
+        rs.clear();
+        for (; y < ys.size() && ys[y].o == o; ++y) {
+            const YB& Y = ys[y];
+            const int x0i = yt[Y.t0].first;
+            const XB& x0 = xs[x0i];
+            P->mix.flops += 2.0 * x0.rows * x0.cols * (double)Y.nt;
+            if (direct[x0i] != (int)y) {
+                MixJob mj{};
+                mj.dst = Y.row * P->ld_y;
+                mj.rows = x0.rows;
+                mj.cols = x0.cols;
+                mj.ldo = P->ld_y;
+                mj.zero_to = kpad(x0.cols, prec);
+                mj.t0 = (int)P->mix.terms.size();
+                mj.nt = Y.nt;
+                for (int t = Y.t0; t < Y.t0 + Y.nt; ++t)
+                    P->mix.terms.push_back({xs[yt[t].first].off, xs[yt[t].first].cols, 0, yt[t].second});
+                P->mix.jobs.push_back(mj);
+                P->mix.max_elems = std::max(P->mix.max_elems, mj.rows * std::max(mj.cols, mj.zero_to));
+            }
+            rs.push_back({R.blk[Y.rb].row * R.ld, Y.row * P->ld_y, x0.cols, 0});
         }
-        int rb = R.at(pb[o].k, w2);
-        rsegs[o].push_back({R.blk[rb].row * R.ld, yr * P->ld_y, x0.cols, 0});
-    }
-    for (auto& kv : rsegs) {
-        const auto& O = pb[kv.first];
-        P->rstage.add(O.cols, O.rows, O.off, R.ld, 1, P->ld_y, 1, 1, O.cols, kv.second);
+        const auto& O = pb[o];
+        P->rstage.add(O.cols, O.rows, O.off, R.ld, 1, P->ld_y, 1, 1, O.cols, rs);
     }
 
     // diagonal
@@ -660,19 +710,39 @@ std::unique_ptr<HeffPlan> make_heff_plan(const Sec& bl, const Sec& br, const std
     }
 
     P->flops = P->lstage.flops + P->ldirect.flops + P->rstage.flops + P->mix.flops;
-    // upload static lists
-    P->pack.up(st);
-    P->mix.up(st);
-    upload(P->ddj, P->djobs, st);
-    upload(P->ddt, P->dterms, st);
+    // every static list in one upload
+    const Num t = mv_num(prec);
     {
+        ListPack pk;
+        P->pack.stage(pk);
+        P->mix.stage(pk);
+        pk.add(P->ddj, P->djobs);
+        pk.add(P->ddt, P->dterms);
         std::vector<long long> el;
         for (const auto& j : P->djobs) el.push_back((long long)j.rows * j.cols);
-        std::vector<int2> c = make_chunks(el);
+        const std::vector<int2> c = make_chunks(el);
         P->diag_chunks = (int)c.size();
-        upload(P->ddc, c, st);
+        pk.add(P->ddc, c);
+        if (prec == PREC_F32) {
+            CopyJob j{};
+            j.src = 0; j.dst = 0; j.rows = 1; j.cols = (int)P->psi.size; j.srs = 0; j.scs = 1; j.drs = 0; j.dcs = 1;
+            j.zero_to = 0; j.scale = 1.0;
+            P->unpack.add(j);
+            P->unpack.stage(pk);
+        }
+        auto stage = [&](GemmBatch& g, Num cnum) {
+            if (prec == DMRG_FP64) g.stage_f64(pk);
+            else if (prec == PREC_F32) g.stage(pk, 64, 64);
+            else {
+                const int bn = g.empty() ? 0 : tc_width(g, t, cnum, true);
+                g.stage(pk, bn ? TC_TILE_M : 0, bn);
+            }
+        };
+        stage(P->lstage, Num::F32);
+        stage(P->ldirect, t);
+        stage(P->rstage, Num::F64);
+        pk.upload(P->lists, st);
     }
-    const Num t = mv_num(prec);
     P->psiT.ensure(std::max<long long>(1, P->psiT_rows) * P->ld_psi * num_size(t), st);
     P->Y.ensure(std::max<long long>(1, P->y_rows) * P->ld_y * num_size(t), st);
     // directly written Y blocks rely on zero padding columns: clear the slab once
@@ -717,13 +787,6 @@ void heff_apply(HeffPlan& P, const EnvSlab& L, const EnvSlab& R, const double* x
         run_gemm32(P.ldirect, P.psiT.as<float>(), Lf, P.Y.as<float>(), st);
         run_mix<float>(P.mix, P.X.as<float>(), P.Y.p, Num::F32, st);
         run_gemm32(P.rstage, Rf, P.Y.as<float>(), y32.as<float>(), st);
-        if (!P.unpack.d.p) {
-            CopyJob j{};
-            j.src = 0; j.dst = 0; j.rows = 1; j.cols = (int)P.psi.size; j.srs = 0; j.scs = 1; j.drs = 0; j.dcs = 1;
-            j.zero_to = 0; j.scale = 1.0;
-            P.unpack.add(j);
-            P.unpack.up(st);
-        }
         run_copy<float>(P.unpack, y32.as<float>(), y, Num::F64, st);
     } else {
         run_gemm_tc(P.lstage, t, P.psiT.p, P.psiT_rows, P.ld_psi, env_operand(L, prec), L.lay.rows, L.lay.ld,
@@ -773,7 +836,10 @@ void env_make_operand(EnvSlab& e, int prec, cudaStream_t st) {
         j.srs = 0; j.scs = 1; j.drs = 0; j.dcs = 1; j.zero_to = 0; j.scale = 1.0;
         c.add(j);
     }
-    c.up(st);
+    ListPack pk;
+    DBuf lists;
+    c.stage(pk);
+    pk.upload(lists, st);
     DBuf& dst = bf ? e.op : e.op32;
     dst.ensure(n * (bf ? 2 : 4), st);
     if (e.num == Num::F64) run_copy<double>(c, e.buf.as<double>(), dst.p, bf ? Num::BF16 : Num::F32, st);
@@ -789,7 +855,10 @@ void env_from_packed(EnvSlab& e, const double* packed, cudaStream_t st) {
         j.srs = b.cols; j.scs = 1; j.drs = e.lay.ld; j.dcs = 1; j.zero_to = 0; j.scale = 1.0;
         c.add(j);
     }
-    c.up(st);
+    ListPack pk;
+    DBuf lists;
+    c.stage(pk);
+    pk.upload(lists, st);
     run_copy<double>(c, packed, e.buf.p, e.num, st);
     e.op_valid = false;
     e.op32_valid = false;
@@ -804,7 +873,10 @@ void env_to_packed(const EnvSlab& e, double* packed, cudaStream_t st) {
         j.srs = e.lay.ld; j.scs = 1; j.drs = b.cols; j.dcs = 1; j.zero_to = 0; j.scale = 1.0;
         c.add(j);
     }
-    c.up(st);
+    ListPack pk;
+    DBuf lists;
+    c.stage(pk);
+    pk.upload(lists, st);
     if (e.num == Num::F64) run_copy<double>(c, e.buf.as<double>(), packed, Num::F64, st);
     else run_copy<float>(c, e.buf.as<float>(), packed, Num::F64, st);
     PD_CK(cudaStreamSynchronize(st));   // the job list is freed on return
@@ -849,6 +921,18 @@ struct EnvProfClass {
 };
 }  // namespace
 
+// Every list of an environment update in one upload (`lists` owns them).
+static void stage_env_lists(CopyList& pk, MixList& mx, GemmBatch& g1, GemmBatch& g3, int prec, DBuf& lists,
+                            cudaStream_t st) {
+    ListPack all;
+    pk.stage(all);
+    mx.stage(all);
+    for (GemmBatch* g : {&g1, &g3})
+        if (env_num(prec) == Num::F64) g->stage_f64(all);
+        else g->stage(all, 64, 64);
+    all.upload(lists, st);
+}
+
 void env_update_left(const Sec& ba, const Sec& bb, const std::vector<int>& qn, const SiteMPO& W,
                      const EnvSlab& Lin, const double* A, EnvSlab& Lout, int prec, unsigned* err, cudaStream_t st) {
     EnvProfClass prof_class;
@@ -858,6 +942,7 @@ void env_update_left(const Sec& ba, const Sec& bb, const std::vector<int>& qn, c
     const Num tn = env_num(prec);
     const int ldS = pad_ld(ba.maxm(), prec);
     // A^T slab: block (ia, s) rows b, cols a
+    DBuf lists;
     CopyList pk;
     std::vector<long long> srow(S.blk.size());
     long long row = 0;
@@ -871,16 +956,23 @@ void env_update_left(const Sec& ba, const Sec& bb, const std::vector<int>& qn, c
         row += B.cols;
     }
     const long long srows = row;
-    // which (w, s') pairs feed anything
+    // nonzero entries (w, s') of W by (w', s), and which (w, s') feed anything
+    struct WE { int w, sp; double c; };
+    std::vector<std::vector<WE>> went((size_t)W.Dr * d);
     std::vector<char> usedws((size_t)W.Dl * d, 0);
     for (int w = 0; w < W.Dl; ++w)
         for (int s = 0; s < d; ++s)
             for (int sp = 0; sp < d; ++sp)
-                for (int wp = 0; wp < W.Dr; ++wp)
-                    if (W.at(w, s, sp, wp) != 0.0) usedws[(size_t)w * d + sp] = 1;
+                for (int wp = 0; wp < W.Dr; ++wp) {
+                    const double c = W.at(w, s, sp, wp);
+                    if (c == 0.0) continue;
+                    usedws[(size_t)w * d + sp] = 1;
+                    went[(size_t)wp * d + s].push_back({w, sp, c});
+                }
     // stage 1: T1(iab, w, s') [b][a_bra] = L_w A_s'
     struct TB { long long off; int rows, cols; };   // rows = b, cols = a_bra
-    std::map<std::tuple<int, int, int>, TB> t1;
+    std::vector<TB> t1;
+    std::vector<int> t1idx((size_t)ba.n() * W.Dl * d, -1);
     GemmBatch g1;
     long long toff = 0;
     for (const auto& lb : Li.blk) {
@@ -889,62 +981,63 @@ void env_update_left(const Sec& ba, const Sec& bb, const std::vector<int>& qn, c
             int ab = S.at(lb.k, sp);
             if (ab < 0) continue;
             const auto& AB = S.blk[ab];
-            TB t{toff, AB.cols, lb.rows};
-            t1[{lb.i, lb.w, sp}] = t;
-            g1.add(lb.rows, AB.cols, toff, Li.ld, 1, ldS, 1, 1, lb.rows,
-                   {GSeg{lb.row * Li.ld, srow[ab] * ldS, lb.cols, 0}});
-            toff += (long long)t.rows * t.cols;
+            t1idx[((size_t)lb.i * W.Dl + lb.w) * d + sp] = (int)t1.size();
+            t1.push_back({toff, AB.cols, lb.rows});
+            const GSeg sg{lb.row * Li.ld, srow[ab] * ldS, lb.cols, 0};
+            g1.add(lb.rows, AB.cols, toff, Li.ld, 1, ldS, 1, 1, lb.rows, &sg, 1, 0, 1.0);
+            toff += (long long)AB.cols * lb.rows;
         }
     }
     // stage 2: T2(w', s, iab) [b][a_bra] = sum W[w,s,s',w'] T1(iab, w, s')
     const EnvLayout& Lo = Lout.lay;
     const int ldT = pad_ld(ba.maxm(), prec);
     MixList mx;
-    std::map<std::tuple<int, int, int>, long long> t2row;
-    std::map<std::tuple<int, int, int>, std::vector<std::pair<const TB*, double>>> t2terms;
-    for (const auto& kv : t1) {
-        int iab, w, sp;
-        std::tie(iab, w, sp) = kv.first;
-        for (int s = 0; s < d; ++s)
-            for (int wp = 0; wp < W.Dr; ++wp) {
-                double c = W.at(w, s, sp, wp);
-                if (c == 0.0) continue;
-                if (S.at(iab, s) < 0) continue;
-                int ibb = bb.find(ba.q[iab] + qn[s]);
-                if (ibb < 0 || Lo.at(ibb, wp) < 0) continue;
-                t2terms[{wp, s, iab}].push_back({&kv.second, c});
-            }
-    }
+    std::vector<long long> t2row((size_t)W.Dr * d * ba.n(), -1);
     long long trow = 0;
-    for (auto& kv : t2terms) {
-        const TB* x0 = kv.second.front().first;
-        t2row[kv.first] = trow;
-        MixJob mj{};
-        mj.dst = trow * ldT; mj.rows = x0->rows; mj.cols = x0->cols; mj.ldo = ldT;
-        mj.zero_to = kpad(x0->cols, prec); mj.t0 = (int)mx.terms.size(); mj.nt = (int)kv.second.size();
-        for (auto& t : kv.second) mx.terms.push_back({t.first->off, t.first->cols, 0, t.second});
-        mx.jobs.push_back(mj);
-        mx.max_elems = std::max(mx.max_elems, mj.rows * std::max(mj.cols, mj.zero_to));
-        trow += x0->rows;
-    }
+    for (int wp = 0; wp < W.Dr; ++wp)
+        for (int s = 0; s < d; ++s) {
+            const std::vector<WE>& we = went[(size_t)wp * d + s];
+            if (we.empty()) continue;
+            for (int iab = 0; iab < ba.n(); ++iab) {
+                if (S.at(iab, s) < 0) continue;
+                const int ibb = bb.find(ba.q[iab] + qn[s]);
+                if (ibb < 0 || Lo.at(ibb, wp) < 0) continue;
+                const int first = (int)mx.terms.size();
+                const TB* x0 = nullptr;
+                for (const WE& e : we) {
+                    const int ti = t1idx[((size_t)iab * W.Dl + e.w) * d + e.sp];
+                    if (ti < 0) continue;
+                    x0 = x0 ? x0 : &t1[ti];
+                    mx.terms.push_back({t1[ti].off, t1[ti].cols, 0, e.c});
+                }
+                if (!x0) continue;
+                t2row[((size_t)wp * d + s) * ba.n() + iab] = trow;
+                MixJob mj{};
+                mj.dst = trow * ldT; mj.rows = x0->rows; mj.cols = x0->cols; mj.ldo = ldT;
+                mj.zero_to = kpad(x0->cols, prec); mj.t0 = first; mj.nt = (int)mx.terms.size() - first;
+                mx.jobs.push_back(mj);
+                mx.max_elems = std::max(mx.max_elems, mj.rows * std::max(mj.cols, mj.zero_to));
+                trow += x0->rows;
+            }
+        }
     // stage 3: Lout(ibb, w') [b_bra][b] = sum_{s, iab} A_s^T T2(w', s, iab)
     GemmBatch g3;
+    std::vector<GSeg> sg;
     for (const auto& ob : Lo.blk) {
-        std::vector<GSeg> sg;
+        sg.clear();
         for (int s = 0; s < d; ++s) {
             int iab = ba.find(bb.q[ob.i] - qn[s]);
             if (iab < 0) continue;
             int ab = S.at(iab, s);
             if (ab < 0) continue;
-            auto it = t2row.find({ob.w, s, iab});
-            if (it == t2row.end()) continue;
-            sg.push_back({it->second * ldT, srow[ab] * ldS, ba.m[iab], 0});
+            const long long tr = t2row[((size_t)ob.w * d + s) * ba.n() + iab];
+            if (tr < 0) continue;
+            sg.push_back({tr * ldT, srow[ab] * ldS, ba.m[iab], 0});
         }
         g3.add(ob.cols, ob.rows, ob.row * Lo.ld, ldT, 1, ldS, 1, 1, Lo.ld, sg);
     }
     // execute
-    pk.up(st);
-    mx.up(st);
+    stage_env_lists(pk, mx, g1, g3, prec, lists, st);
     DBuf sl, t1b, t2b;
     sl.ensure(std::max<long long>(1, srows) * ldS * num_size(tn), st);
     t1b.ensure(std::max<long long>(1, toff) * num_size(tn), st);
@@ -968,6 +1061,7 @@ void env_update_right(const Sec& ba, const Sec& bc, const std::vector<int>& qn, 
     const Num tn = env_num(prec);
     const int ldS = pad_ld(bc.maxm(), prec);
     // B slab: block (ia, s) rows a, cols c (same orientation as the packed block)
+    DBuf lists;
     CopyList pk;
     std::vector<long long> srow(S.blk.size());
     long long row = 0;
@@ -981,15 +1075,23 @@ void env_update_right(const Sec& ba, const Sec& bc, const std::vector<int>& qn, 
         row += B.rows;
     }
     const long long srows = row;
-    std::vector<char> usedws((size_t)W.Dr * d, 0);   // (w', s')
-    for (int w = 0; w < W.Dl; ++w)
-        for (int s = 0; s < d; ++s)
-            for (int sp = 0; sp < d; ++sp)
-                for (int wp = 0; wp < W.Dr; ++wp)
-                    if (W.at(w, s, sp, wp) != 0.0) usedws[(size_t)wp * d + sp] = 1;
+    // nonzero entries (w', s') of W by (w, s), and which (w', s') feed anything
+    struct WE { int wp, sp; double c; };
+    std::vector<std::vector<WE>> went((size_t)W.Dl * d);
+    std::vector<char> usedws((size_t)W.Dr * d, 0);
+    for (int wp = 0; wp < W.Dr; ++wp)
+        for (int w = 0; w < W.Dl; ++w)
+            for (int s = 0; s < d; ++s)
+                for (int sp = 0; sp < d; ++sp) {
+                    const double c = W.at(w, s, sp, wp);
+                    if (c == 0.0) continue;
+                    usedws[(size_t)wp * d + sp] = 1;
+                    went[(size_t)w * d + s].push_back({wp, sp, c});
+                }
     // stage 1: T1(icb, w', s') [a][c_bra] = R_w' B_s'^T
     struct TB { long long off; int rows, cols; };   // rows = a, cols = c_bra
-    std::map<std::tuple<int, int, int>, TB> t1;
+    std::vector<TB> t1;
+    std::vector<int> t1idx((size_t)bc.n() * W.Dr * d, -1);
     GemmBatch g1;
     long long toff = 0;
     for (const auto& rb : Ri.blk) {
@@ -1000,61 +1102,61 @@ void env_update_right(const Sec& ba, const Sec& bc, const std::vector<int>& qn, 
             int bbk = S.at(ia, sp);
             if (bbk < 0) continue;
             const auto& BB = S.blk[bbk];
-            TB t{toff, BB.rows, rb.rows};
-            t1[{rb.i, rb.w, sp}] = t;
-            g1.add(rb.rows, BB.rows, toff, Ri.ld, 1, ldS, 1, 1, rb.rows,
-                   {GSeg{rb.row * Ri.ld, srow[bbk] * ldS, rb.cols, 0}});
-            toff += (long long)t.rows * t.cols;
+            t1idx[((size_t)rb.i * W.Dr + rb.w) * d + sp] = (int)t1.size();
+            t1.push_back({toff, BB.rows, rb.rows});
+            const GSeg sg{rb.row * Ri.ld, srow[bbk] * ldS, rb.cols, 0};
+            g1.add(rb.rows, BB.rows, toff, Ri.ld, 1, ldS, 1, 1, rb.rows, &sg, 1, 0, 1.0);
+            toff += (long long)BB.rows * rb.rows;
         }
     }
     // stage 2: T2(w, s, icb) [a][c_bra] = sum W[w,s,s',w'] T1(icb, w', s')
     const EnvLayout& Ro = Rout.lay;
     const int ldT = pad_ld(bc.maxm(), prec);
     MixList mx;
-    std::map<std::tuple<int, int, int>, long long> t2row;
-    std::map<std::tuple<int, int, int>, std::vector<std::pair<const TB*, double>>> t2terms;
-    for (const auto& kv : t1) {
-        int icb, wp, sp;
-        std::tie(icb, wp, sp) = kv.first;
-        for (int w = 0; w < W.Dl; ++w)
-            for (int s = 0; s < d; ++s) {
-                double c = W.at(w, s, sp, wp);
-                if (c == 0.0) continue;
-                int iab = ba.find(bc.q[icb] - qn[s]);
-                if (iab < 0 || S.at(iab, s) < 0) continue;
-                if (Ro.at(iab, w) < 0) continue;
-                t2terms[{w, s, icb}].push_back({&kv.second, c});
-            }
-    }
+    std::vector<long long> t2row((size_t)W.Dl * d * bc.n(), -1);
     long long trow = 0;
-    for (auto& kv : t2terms) {
-        const TB* x0 = kv.second.front().first;
-        t2row[kv.first] = trow;
-        MixJob mj{};
-        mj.dst = trow * ldT; mj.rows = x0->rows; mj.cols = x0->cols; mj.ldo = ldT;
-        mj.zero_to = kpad(x0->cols, prec); mj.t0 = (int)mx.terms.size(); mj.nt = (int)kv.second.size();
-        for (auto& t : kv.second) mx.terms.push_back({t.first->off, t.first->cols, 0, t.second});
-        mx.jobs.push_back(mj);
-        mx.max_elems = std::max(mx.max_elems, mj.rows * std::max(mj.cols, mj.zero_to));
-        trow += x0->rows;
-    }
+    for (int w = 0; w < W.Dl; ++w)
+        for (int s = 0; s < d; ++s) {
+            const std::vector<WE>& we = went[(size_t)w * d + s];
+            if (we.empty()) continue;
+            for (int icb = 0; icb < bc.n(); ++icb) {
+                const int iab = ba.find(bc.q[icb] - qn[s]);
+                if (iab < 0 || S.at(iab, s) < 0 || Ro.at(iab, w) < 0) continue;
+                const int first = (int)mx.terms.size();
+                const TB* x0 = nullptr;
+                for (const WE& e : we) {
+                    const int ti = t1idx[((size_t)icb * W.Dr + e.wp) * d + e.sp];
+                    if (ti < 0) continue;
+                    x0 = x0 ? x0 : &t1[ti];
+                    mx.terms.push_back({t1[ti].off, t1[ti].cols, 0, e.c});
+                }
+                if (!x0) continue;
+                t2row[((size_t)w * d + s) * bc.n() + icb] = trow;
+                MixJob mj{};
+                mj.dst = trow * ldT; mj.rows = x0->rows; mj.cols = x0->cols; mj.ldo = ldT;
+                mj.zero_to = kpad(x0->cols, prec); mj.t0 = first; mj.nt = (int)mx.terms.size() - first;
+                mx.jobs.push_back(mj);
+                mx.max_elems = std::max(mx.max_elems, mj.rows * std::max(mj.cols, mj.zero_to));
+                trow += x0->rows;
+            }
+        }
     // stage 3: Rout(iab, w) [a_bra][a] = sum_{s, icb} B_s T2(w, s, icb)^T
     GemmBatch g3;
+    std::vector<GSeg> sg;
     for (const auto& ob : Ro.blk) {
-        std::vector<GSeg> sg;
+        sg.clear();
         for (int s = 0; s < d; ++s) {
             int icb = bc.find(ba.q[ob.i] + qn[s]);
             if (icb < 0) continue;
             int bbk = S.at(ob.i, s);
             if (bbk < 0) continue;
-            auto it = t2row.find({ob.w, s, icb});
-            if (it == t2row.end()) continue;
-            sg.push_back({it->second * ldT, srow[bbk] * ldS, bc.m[icb], 0});
+            const long long tr = t2row[((size_t)ob.w * d + s) * bc.n() + icb];
+            if (tr < 0) continue;
+            sg.push_back({tr * ldT, srow[bbk] * ldS, bc.m[icb], 0});
         }
         g3.add(ob.cols, ob.rows, ob.row * Ro.ld, ldT, 1, ldS, 1, 1, Ro.ld, sg);
     }
-    pk.up(st);
-    mx.up(st);
+    stage_env_lists(pk, mx, g1, g3, prec, lists, st);
     DBuf sl, t1b, t2b;
     sl.ensure(std::max<long long>(1, srows) * ldS * num_size(tn), st);
     t1b.ensure(std::max<long long>(1, toff) * num_size(tn), st);

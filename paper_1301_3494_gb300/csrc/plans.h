@@ -1,6 +1,7 @@
 // Block layouts, contraction plans and the device-side building blocks of one two-site step.
 #pragma once
 #include <algorithm>
+#include <cstring>
 #include <memory>
 #include <vector>
 
@@ -49,6 +50,7 @@ struct DBuf {
     void* p = nullptr;
     size_t bytes = 0;
     cudaStream_t st = nullptr;
+    bool own = true;                  // false: a part of another buffer (see ListPack)
     DBuf() = default;
     DBuf(const DBuf&) = delete;
     DBuf& operator=(const DBuf&) = delete;
@@ -56,23 +58,32 @@ struct DBuf {
     DBuf& operator=(DBuf&& o) noexcept {
         if (this != &o) {
             release();
-            p = o.p; bytes = o.bytes; st = o.st;
-            o.p = nullptr; o.bytes = 0;
+            p = o.p; bytes = o.bytes; st = o.st; own = o.own;
+            o.p = nullptr; o.bytes = 0; o.own = true;
         }
         return *this;
     }
     ~DBuf() { release(); }
     void release() {
-        if (p) cudaFreeAsync(p, st);
+        if (p && own) cudaFreeAsync(p, st);
         p = nullptr;
         bytes = 0;
+        own = true;
+    }
+    // Refer to a part of another buffer, which must outlive this one's use.
+    void view(void* part, size_t b, cudaStream_t s) {
+        release();
+        p = part;
+        bytes = b;
+        st = s;
+        own = false;
     }
     // (Re)allocate at least `b` bytes on stream s; contents undefined after growth.
     void ensure(size_t b, cudaStream_t s) {
         if (b == 0) b = 16;
         if (p && bytes >= b) { st = s; return; }
         release();
-        PD_CK(cudaMallocAsync(&p, b, s));
+        p = pool_alloc(b, s);
         bytes = b;
         st = s;
     }
@@ -86,6 +97,30 @@ inline void upload(DBuf& d, const std::vector<T>& h, cudaStream_t st) {
     d.ensure(h.size() * sizeof(T), st);
     if (!h.empty()) PD_CK(cudaMemcpyAsync(d.p, h.data(), h.size() * sizeof(T), cudaMemcpyHostToDevice, st));
 }
+
+// Several host lists uploaded as one allocation and one copy: a plan has some twenty lists of a few
+// kilobytes, and an allocation and a copy for each of them (5 us together) was most of a small call.
+// The lists' buffers become parts of `owner`.
+struct ListPack {
+    struct Item { DBuf* d; size_t off, bytes; };
+    std::vector<char> host;
+    std::vector<Item> items;
+    template <class T>
+    void add(DBuf& d, const std::vector<T>& v) {
+        const size_t off = (host.size() + 15) & ~size_t(15), n = v.size() * sizeof(T);
+        host.resize(off + std::max<size_t>(n, 16));
+        if (n) std::memcpy(host.data() + off, v.data(), n);
+        items.push_back({&d, off, std::max<size_t>(n, 16)});
+    }
+    void upload(DBuf& owner, cudaStream_t st) {
+        if (items.empty()) return;
+        owner.ensure(host.size(), st);
+        PD_CK(cudaMemcpyAsync(owner.p, host.data(), host.size(), cudaMemcpyHostToDevice, st));
+        for (const Item& i : items) i.d->view(static_cast<char*>(owner.p) + i.off, i.bytes, st);
+        host.clear();
+        items.clear();
+    }
+};
 
 // ------------------------------------------------------------------------------------------
 // Block layouts
@@ -164,22 +199,29 @@ struct GemmBatch {
     int lda = 0, ldb = 0;
     std::shared_ptr<EmuPlan> emu;       // plan of the FP64-emulated execution, built on first use
 
-    void add(int M, int N, long long c_off, int sam, int sak, int sbn, int sbk, int scm, int scn,
-             const std::vector<GSeg>& sg, int accumulate = 0, double alpha = 1.0) {
-        if (M <= 0 || N <= 0 || sg.empty()) return;
+    void add(int M, int N, long long c_off, int sam, int sak, int sbn, int sbk, int scm, int scn, const GSeg* sg, int nsg,
+             int accumulate, double alpha) {
+        if (M <= 0 || N <= 0 || nsg <= 0) return;
         GProb p{};
-        p.M = M; p.N = N; p.seg0 = (int)segs.size(); p.nseg = (int)sg.size();
+        p.M = M; p.N = N; p.seg0 = (int)segs.size(); p.nseg = nsg;
         p.c_off = c_off; p.sam = sam; p.sak = sak; p.sbn = sbn; p.sbk = sbk; p.scm = scm; p.scn = scn;
         p.accumulate = accumulate; p.alpha = alpha;
-        for (const auto& s : sg) {
-            segs.push_back(s);
-            flops += 2.0 * M * N * s.K;
+        for (int i = 0; i < nsg; ++i) {
+            segs.push_back(sg[i]);
+            flops += 2.0 * M * N * sg[i].K;
         }
         probs.push_back(p);
+    }
+    void add(int M, int N, long long c_off, int sam, int sak, int sbn, int sbk, int scm, int scn,
+             const std::vector<GSeg>& sg, int accumulate = 0, double alpha = 1.0) {
+        add(M, N, c_off, sam, sak, sbn, sbk, scm, scn, sg.data(), (int)sg.size(), accumulate, alpha);
     }
     bool empty() const { return probs.empty(); }
     // Upload for the FP32 SIMT engine (64x64 tiles) or the tensor-core engine (tile_m x tile_n).
     void upload_tiles(int tm, int tn, cudaStream_t st);
+    // The same lists as part of a pack (tm = 0: problems and segments only, tiles on first use).
+    void stage(ListPack& pk, int tm, int tn);
+    void stage_f64(ListPack& pk);
     // Upload for the FP64 engine, with the tile shape that suits the batch (chosen once).
     F64Shape upload_f64(cudaStream_t st);
 };
@@ -191,6 +233,10 @@ void run_gemm32(GemmBatch& g, const float* A, const float* B, float* C, cudaStre
 void run_gemm_tc(GemmBatch& g, Num t, const void* A, long long a_rows, int lda, const void* B,
                  long long b_rows, int ldb, void* C, Num cnum, unsigned* err, cudaStream_t st);
 bool tc_available();
+// Tile width of a batch on the tensor cores where the cost model or an earlier timing gives it, 0
+// where run_gemm_tc would time the widths first.
+int tc_width(const GemmBatch& g, Num t, Num cnum, bool repeatable);
+constexpr int TC_TILE_M = 128;
 // Tile-width autotuner of the tensor-core GEMM: shape classes timed so far, and how many of them
 // chose a different width than the cost model.
 void tune_stats(long long* classes, long long* changed);
@@ -221,6 +267,12 @@ struct CopyList {
         nchunks = (int)c.size();
         upload(dc, c, st);
     }
+    void stage(ListPack& pk) {
+        pk.add(d, jobs);
+        const std::vector<int2> c = make_chunks(elems);
+        nchunks = (int)c.size();
+        pk.add(dc, c);
+    }
 };
 struct MixList {
     std::vector<MixJob> jobs;
@@ -237,6 +289,15 @@ struct MixList {
         std::vector<int2> c = make_chunks(el);
         nchunks = (int)c.size();
         upload(dc, c, st);
+    }
+    void stage(ListPack& pk) {
+        pk.add(dj, jobs);
+        pk.add(dt, terms);
+        std::vector<long long> el;
+        for (const auto& j : jobs) el.push_back((long long)j.rows * std::max(j.cols, j.zero_to));
+        const std::vector<int2> c = make_chunks(el);
+        nchunks = (int)c.size();
+        pk.add(dc, c);
     }
 };
 
@@ -304,6 +365,7 @@ struct HeffPlan {
     DBuf ddj, ddt, ddc;
     int diag_max = 0, diag_chunks = 0;
     double flops = 0.0;
+    DBuf lists;               // every list above, one allocation
     // scratch
     DBuf psiT, X, Y;
 };

@@ -29,7 +29,7 @@ namespace pd {
 
 namespace {
 
-constexpr int BM = 128;
+constexpr int BM = TC_TILE_M;
 constexpr int THREADS = 192;
 constexpr uint64_t WAIT_NS = 2000000000ull;      // 2 s per wait before giving up
 constexpr uint64_t DRAIN_NS = 500000000ull;
@@ -477,6 +477,16 @@ void launch_bn(GemmBatch& g, int bn, Num t, const void* A, long long a_rows, int
 }
 }  // namespace
 
+int tc_width(const GemmBatch& g, Num t, Num cnum, bool repeatable) {
+    if (g.bn_choice) return g.bn_choice;
+    {
+        std::lock_guard<std::mutex> lk(g_tune_mu);
+        auto it = g_tune.find(tune_key(g, t, cnum));
+        if (it != g_tune.end()) return it->second;
+    }
+    return repeatable && g.flops >= 4e9 ? 0 : pick_bn(g, (int)num_size(t));
+}
+
 void run_gemm_tc(GemmBatch& g, Num t, const void* A, long long a_rows, int lda, const void* B, long long b_rows,
                  int ldb, void* C, Num cnum, unsigned* err, cudaStream_t st) {
     if (g.empty()) return;
@@ -487,20 +497,13 @@ void run_gemm_tc(GemmBatch& g, Num t, const void* A, long long a_rows, int lda, 
                    "tensor-core GEMM needs K-major slabs with uniform leading dimensions");
     int bn = g.bn_choice;
     if (!bn) {
-        const int model = pick_bn(g, (int)num_size(t));
         // small batches: timing noise exceeds any difference between widths
-        bool repeatable = C != A && C != B && g.flops >= 4e9;
+        bool repeatable = C != A && C != B;
         for (const auto& p : g.probs) repeatable = repeatable && !p.accumulate;
-        const TuneKey key = tune_key(g, t, cnum);
-        int cached = 0;
-        {
-            std::lock_guard<std::mutex> lk(g_tune_mu);
-            auto it = g_tune.find(key);
-            if (it != g_tune.end()) cached = it->second;
-        }
-        if (cached) {
-            bn = cached;
-        } else if (repeatable) {
+        bn = tc_width(g, t, cnum, repeatable);
+        if (!bn) {
+            const int model = pick_bn(g, (int)num_size(t));
+            const TuneKey key = tune_key(g, t, cnum);
             float best = -1.f;
             int best_bn = model;
             const int saved = g_prof_class;
@@ -536,8 +539,6 @@ void run_gemm_tc(GemmBatch& g, Num t, const void* A, long long a_rows, int lda, 
             }
             if (best_bn != model) g_tune_changed.fetch_add(1);
             bn = best_bn;
-        } else {
-            bn = model;
         }
         g.bn_choice = bn;
     }
