@@ -152,9 +152,10 @@ struct DiagTerm {
 // ------------------------------------------------------------------------------------------
 // Launch wrappers (kernels.cu)
 // ------------------------------------------------------------------------------------------
-template <class T>
-void launch_gemm_simt(const GProb* probs, const GSeg* segs, const GTile* tiles, int ntiles, const T* A, const T* B,
-                      T* C, cudaStream_t st);
+// FP32 GEMM, 64 x 64 tiles.  Operands K-major (sak = sbk = 1) with 16-byte aligned rows (offsets and row
+// strides multiples of 4) that are zero from K to the next multiple of 16 on both sides.
+void launch_gemm_f32(const GProb* probs, const GSeg* segs, const GTile* tiles, int ntiles, const float* A, const float* B,
+                     float* C, cudaStream_t st);
 // FP64 GEMM: `tile` = edge of a CTA's output tile, `ksplit` = warps that share it.  The tile list has
 // square tiles of `edge` (a multiple of shape.tile).
 struct F64Shape {

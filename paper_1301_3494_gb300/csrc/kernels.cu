@@ -228,65 +228,101 @@ __global__ void __launch_bounds__(KS == 1 ? 128 : 32 * KS)
 }
 
 // ------------------------------------------------------------------------------------------
-// Grouped SIMT GEMM (FP32): 64x64 output tile per CTA, 256 threads, 4x4 per thread, K chunks of 16.
+// Grouped FP32 GEMM (mixed-mode environments, refinement matvec) on the FMA units, which bound it:
+// 64 x 64 output tile per CTA of two warps, 8 x 8 values per thread, so a step in k is 64 FMA on four
+// 16-byte shared loads.  64 x 64 loses least to the blocks' edges (sectors of 40-320 states), and a
+// warp whose 32 rows lie outside the block does no products.  Operands are K-major slabs whose rows
+// are zero up to a multiple of 16 in k (the tensor-core layout): they come in as float4 along k, one
+// chunk of 16 ahead in registers, and are stored k-major into a double buffer -- one barrier a chunk.
+// Each value is one chain of FMA in k order, as in the 4 x 4 kernel before: the same bits.
+// FP32 environment update at the 24x8 cylinder's m = 2000 bond, its two GEMMs: see launch_gemm_f32.
 // ------------------------------------------------------------------------------------------
-template <class T>
-__global__ void __launch_bounds__(256) k_gemm_simt(const GProb* __restrict__ probs,
-                                                   const GSeg* __restrict__ segs,
-                                                   const GTile* __restrict__ tiles,
-                                                   const T* __restrict__ A,
-                                                   const T* __restrict__ B,
-                                                   T* __restrict__ C) {
-    __shared__ T As[16][65];
-    __shared__ T Bs[16][65];
+constexpr int F32_T = 64, F32_K = 16, F32_LD = F32_T + 4;
+__global__ void __launch_bounds__(64) k_gemm_f32(const GProb* __restrict__ probs, const GSeg* __restrict__ segs,
+                                                 const GTile* __restrict__ tiles, const float* __restrict__ A,
+                                                 const float* __restrict__ B, float* __restrict__ C) {
+    __shared__ __align__(16) float As[2][F32_K][F32_LD], Bs[2][F32_K][F32_LD];
     const GTile t = tiles[blockIdx.x];
     const GProb p = probs[t.prob];
-    const int tid = threadIdx.x;
-    const int tx = tid & 15, ty = tid >> 4;
-    T acc[4][4];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tr = 32 * warp + 4 * (lane >> 3), tc = 4 * (lane & 7);   // rows tr..+3, tr+16..; cols tc..+3, tc+32..
+    // loader: thread = row of A and of B (clamped into the block: rows outside are not stored)
+    const long long ra = (long long)min(t.m0 + tid, p.M - 1) * p.sam, rb = (long long)min(t.n0 + tid, p.N - 1) * p.sbn;
+    const bool busy = t.m0 + 32 * warp < p.M;
+    float acc[8][8];
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < 8; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = T(0);
-    for (int sgi = 0; sgi < p.nseg; ++sgi) {
-        const GSeg sg = segs[p.seg0 + sgi];
-        for (int k0 = 0; k0 < sg.K; k0 += 16) {
-            for (int e = tid; e < 1024; e += 256) {
-                int kk = e & 15, mm = e >> 4;
-                int m = t.m0 + mm, k = k0 + kk;
-                T va = T(0), vb = T(0);
-                if (m < p.M && k < sg.K) va = A[sg.a_off + (long long)m * p.sam + (long long)k * p.sak];
-                int n = t.n0 + mm;
-                if (n < p.N && k < sg.K) vb = B[sg.b_off + (long long)n * p.sbn + (long long)k * p.sbk];
-                As[kk][mm] = va;
-                Bs[kk][mm] = vb;
-            }
-            __syncthreads();
+        for (int j = 0; j < 8; ++j) acc[i][j] = 0.f;
+    float4 fa[4], fb[4];
+    int sgi = 0, k0 = 0, buf = 0;
+    GSeg sg = segs[p.seg0];
+    auto load = [&]() {
+        const float4* a = reinterpret_cast<const float4*>(A + sg.a_off + ra + k0);
+        const float4* b = reinterpret_cast<const float4*>(B + sg.b_off + rb + k0);
 #pragma unroll
-            for (int kk = 0; kk < 16; ++kk) {
-                T a[4], b[4];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) a[i] = As[kk][ty + 16 * i];
-#pragma unroll
-                for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tx + 16 * j];
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
-            }
-            __syncthreads();
+        for (int q = 0; q < 4; ++q) {
+            fa[q] = a[q];
+            fb[q] = b[q];
         }
+    };
+    auto store = [&](int to) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            As[to][4 * q][tid] = fa[q].x;
+            As[to][4 * q + 1][tid] = fa[q].y;
+            As[to][4 * q + 2][tid] = fa[q].z;
+            As[to][4 * q + 3][tid] = fa[q].w;
+            Bs[to][4 * q][tid] = fb[q].x;
+            Bs[to][4 * q + 1][tid] = fb[q].y;
+            Bs[to][4 * q + 2][tid] = fb[q].z;
+            Bs[to][4 * q + 3][tid] = fb[q].w;
+        }
+    };
+    load();
+    store(0);
+    __syncthreads();
+    for (;;) {
+        // next chunk: this segment's next 16, or the next segment's first
+        k0 += F32_K;
+        if (k0 >= sg.K) {
+            k0 = 0;
+            if (++sgi < p.nseg) sg = segs[p.seg0 + sgi];
+        }
+        const bool more = sgi < p.nseg;
+        if (more) load();
+        if (busy) {
+#pragma unroll
+            for (int k = 0; k < F32_K; ++k) {
+                const float4 a0 = *reinterpret_cast<const float4*>(&As[buf][k][tr]);
+                const float4 a1 = *reinterpret_cast<const float4*>(&As[buf][k][tr + 16]);
+                const float4 b0 = *reinterpret_cast<const float4*>(&Bs[buf][k][tc]);
+                const float4 b1 = *reinterpret_cast<const float4*>(&Bs[buf][k][tc + 32]);
+                const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+                const float b[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+#pragma unroll
+                for (int i = 0; i < 8; ++i)
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+            }
+        }
+        if (!more) break;
+        buf ^= 1;
+        store(buf);
+        __syncthreads();
     }
+    if (!busy) return;
+    const float alpha = (float)p.alpha;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        int m = t.m0 + ty + 16 * i;
-        if (m >= p.M) continue;
+    for (int j = 0; j < 8; ++j) {
+        const int n = t.n0 + tc + (j & 3) + (j >> 2) * 32;
+        if (n >= p.N) continue;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            int n = t.n0 + tx + 16 * j;
-            if (n >= p.N) continue;
-            long long idx = p.c_off + (long long)m * p.scm + (long long)n * p.scn;
-            T v = (T)p.alpha * acc[i][j];
+        for (int i = 0; i < 8; ++i) {
+            const int m = t.m0 + tr + (i & 3) + (i >> 2) * 16;
+            if (m >= p.M) continue;
+            const long long idx = p.c_off + (long long)m * p.scm + (long long)n * p.scn;
+            float v = alpha * acc[i][j];
             if (p.accumulate) v += C[idx];
             C[idx] = v;
         }
@@ -977,15 +1013,12 @@ inline int grid_for(long long elems, int cap = 4096) {
 // ------------------------------------------------------------------------------------------
 // Launch wrappers
 // ------------------------------------------------------------------------------------------
-template <class T>
-void launch_gemm_simt(const GProb* probs, const GSeg* segs, const GTile* tiles, int ntiles, const T* A, const T* B,
-                      T* C, cudaStream_t st) {
+void launch_gemm_f32(const GProb* probs, const GSeg* segs, const GTile* tiles, int ntiles, const float* A, const float* B,
+                     float* C, cudaStream_t st) {
     if (ntiles <= 0) return;
-    k_gemm_simt<T><<<ntiles, 256, 0, st>>>(probs, segs, tiles, A, B, C);
+    k_gemm_f32<<<ntiles, 64, 0, st>>>(probs, segs, tiles, A, B, C);
     PD_LAUNCHED();
 }
-template void launch_gemm_simt<float>(const GProb*, const GSeg*, const GTile*, int, const float*, const float*,
-                                      float*, cudaStream_t);
 
 F64Shape f64_shape(const std::vector<GProb>& probs, const std::vector<GSeg>& segs) {
     // 16 x 16 tiles and their mean K decide.  A tile's chain is 8 K warp instructions of 64 clocks on
@@ -1007,7 +1040,8 @@ F64Shape f64_shape(const std::vector<GProb>& probs, const std::vector<GSeg>& seg
     }
     const double kmean = tiles ? (double)kt / (double)tiles : 0.0;
     if (tiles >= 9728 || kmean < 16.0) return {32, 1};
-    if (tiles <= 608 && kmean >= 256.0) return {16, 16};
+    if (tiles <= 152 && kmean >= 256.0) return {16, 16};
+    if (tiles <= 608 && kmean >= 128.0) return {16, 8};
     return {16, 4};
 }
 
@@ -1019,6 +1053,7 @@ void launch_gemm_f64(const GProb* probs, const GSeg* segs, const GTile* tiles, i
     PD_REQUIRE(side >= 1 && side * shape.tile == edge && grid < (1LL << 31), DMRG_ERR_CAPACITY, "FP64 GEMM tile list");
     if (shape.ksplit == 1) k_gemm_f64<1><<<(unsigned)grid, 128, 0, st>>>(probs, segs, tiles, side, A, B, C);
     else if (shape.ksplit == 4) k_gemm_f64<4><<<(unsigned)grid, 128, 0, st>>>(probs, segs, tiles, side, A, B, C);
+    else if (shape.ksplit == 8) k_gemm_f64<8><<<(unsigned)grid, 256, 0, st>>>(probs, segs, tiles, side, A, B, C);
     else k_gemm_f64<16><<<(unsigned)grid, 512, 0, st>>>(probs, segs, tiles, side, A, B, C);
     PD_LAUNCHED();
 }

@@ -195,9 +195,14 @@ void run_gemm64(GemmBatch& g, const double* A, const double* B, double* C, cudaS
 
 void run_gemm32(GemmBatch& g, const float* A, const float* B, float* C, cudaStream_t st) {
     if (g.empty()) return;
+    for (const auto& p : g.probs)
+        PD_REQUIRE(p.sak == 1 && p.sbk == 1 && p.sam % 16 == 0 && p.sbn % 16 == 0, DMRG_ERR_ARG,
+                   "FP32 GEMM needs K-major slabs with padded rows");
+    for (const auto& x : g.segs)
+        PD_REQUIRE(x.a_off % 4 == 0 && x.b_off % 4 == 0, DMRG_ERR_ARG, "FP32 GEMM needs 16-byte aligned operand rows");
     g.upload_tiles(64, 64, st);
     void* tok = prof_on() ? prof_start(st) : nullptr;
-    launch_gemm_simt<float>(g.dprobs.as<GProb>(), g.dsegs.as<GSeg>(), g.dtiles.as<GTile>(), g.ntiles, A, B, C, st);
+    launch_gemm_f32(g.dprobs.as<GProb>(), g.dsegs.as<GSeg>(), g.dtiles.as<GTile>(), g.ntiles, A, B, C, st);
     if (tok) prof_stop(tok, st, PROF_F32, g.flops);
 }
 
