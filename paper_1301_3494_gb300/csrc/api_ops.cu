@@ -101,12 +101,8 @@ dmrg_status dmrg_heff_apply(const dmrg_bond_desc* bd, int prec, const double* L_
         BondCtx b = read_bond(bd, true);
         TwoSiteMPO t = two_site_mpo(b.w1, b.w2);
         EnvSlab L, R;
-        env_alloc(L, b.bl, b.w1.fl, prec, st);
-        env_from_packed(L, L_dev, st);
-        env_alloc(R, b.br, b.w2.fr, prec, st);
-        env_from_packed(R, R_dev, st);
-        env_make_operand(L, prec, st);
-        env_make_operand(R, prec, st);
+        env_operand_from_packed(L, b.bl, b.w1.fl, prec, L_dev, st);
+        env_operand_from_packed(R, b.br, b.w2.fr, prec, R_dev, st);
         auto plan = make_heff_plan(b.bl, b.br, b.qn, t, L.lay, R.lay, prec, st);
         DBuf err;
         err.ensure(4, st);

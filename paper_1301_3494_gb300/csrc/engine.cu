@@ -145,17 +145,8 @@ const EnvSlab& env64_view(const EnvSlab& e, EnvSlab& tmp, cudaStream_t st) {
     tmp.lay = e.lay;
     tmp.num = Num::F64;
     const long long n = std::max<long long>(1, e.lay.rows) * e.lay.ld;
-    CopyList cl;
-    const long long chunk = 1 << 20;
-    for (long long s0 = 0; s0 < n; s0 += chunk) {
-        CopyJob j{};
-        j.src = s0; j.dst = s0; j.rows = 1; j.cols = (int)std::min(chunk, n - s0);
-        j.srs = 0; j.scs = 1; j.drs = 0; j.dcs = 1; j.zero_to = 0; j.scale = 1.0;
-        cl.add(j);
-    }
-    cl.up(st);
     tmp.buf.ensure(n * 8, st);
-    run_copy<float>(cl, e.buf.as<float>(), tmp.buf.p, Num::F64, st);
+    convert_flat(e.buf.p, Num::F32, tmp.buf.p, Num::F64, n, st);
     tmp.valid = true;
     return tmp;
 }

@@ -167,10 +167,14 @@ void launch_gemm_f64(const GProb* probs, const GSeg* segs, const GTile* tiles, i
 
 // Elementwise block kernels run one CTA per chunk of CHUNK elements of one job; `chunks`
 // lists (job, first element) for every chunk (built on the host, see make_chunks).
-constexpr int CHUNK = 2048;
+constexpr int CHUNK = 4096;
 template <class Tin, class Tout>
 void launch_copy(const CopyJob* jobs, const int2* chunks, int nchunks, const Tin* src, Tout* dst,
                  cudaStream_t st);
+
+// Element type conversion of a contiguous array.
+template <class Tin, class Tout>
+void launch_convert(const Tin* src, Tout* dst, long long n, cudaStream_t st);
 
 template <class Tin, class Tout>
 void launch_mix(const MixJob* jobs, const int2* chunks, int nchunks, const MixTerm* terms,

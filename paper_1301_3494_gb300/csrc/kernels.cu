@@ -246,8 +246,16 @@ __global__ void __launch_bounds__(64) k_gemm_f32(const GProb* __restrict__ probs
     const GProb p = probs[t.prob];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int tr = 32 * warp + 4 * (lane >> 3), tc = 4 * (lane & 7);   // rows tr..+3, tr+16..; cols tc..+3, tc+32..
-    // loader: thread = row of A and of B (clamped into the block: rows outside are not stored)
-    const long long ra = (long long)min(t.m0 + tid, p.M - 1) * p.sam, rb = (long long)min(t.n0 + tid, p.N - 1) * p.sbn;
+    // loader: four threads take the 64 bytes of a row's chunk, 16 rows a pass (rows outside the block are
+    // clamped into it and not stored).  A row's values go to columns row ^ 8 in the upper half of the
+    // chunk, which keeps these transposing stores free of bank conflicts.
+    const int lr = tid >> 2, lk = 4 * (tid & 3), sw = lr ^ (lk & 8);
+    long long ra[4], rb[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        ra[q] = (long long)min(t.m0 + lr + 16 * q, p.M - 1) * p.sam + lk;
+        rb[q] = (long long)min(t.n0 + lr + 16 * q, p.N - 1) * p.sbn + lk;
+    }
     const bool busy = t.m0 + 32 * warp < p.M;
     float acc[8][8];
 #pragma unroll
@@ -258,25 +266,25 @@ __global__ void __launch_bounds__(64) k_gemm_f32(const GProb* __restrict__ probs
     int sgi = 0, k0 = 0, buf = 0;
     GSeg sg = segs[p.seg0];
     auto load = [&]() {
-        const float4* a = reinterpret_cast<const float4*>(A + sg.a_off + ra + k0);
-        const float4* b = reinterpret_cast<const float4*>(B + sg.b_off + rb + k0);
+        const float* a = A + sg.a_off + k0;
+        const float* b = B + sg.b_off + k0;
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-            fa[q] = a[q];
-            fb[q] = b[q];
+            fa[q] = *reinterpret_cast<const float4*>(a + ra[q]);
+            fb[q] = *reinterpret_cast<const float4*>(b + rb[q]);
         }
     };
     auto store = [&](int to) {
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-            As[to][4 * q][tid] = fa[q].x;
-            As[to][4 * q + 1][tid] = fa[q].y;
-            As[to][4 * q + 2][tid] = fa[q].z;
-            As[to][4 * q + 3][tid] = fa[q].w;
-            Bs[to][4 * q][tid] = fb[q].x;
-            Bs[to][4 * q + 1][tid] = fb[q].y;
-            Bs[to][4 * q + 2][tid] = fb[q].z;
-            Bs[to][4 * q + 3][tid] = fb[q].w;
+            As[to][lk][sw + 16 * q] = fa[q].x;
+            As[to][lk + 1][sw + 16 * q] = fa[q].y;
+            As[to][lk + 2][sw + 16 * q] = fa[q].z;
+            As[to][lk + 3][sw + 16 * q] = fa[q].w;
+            Bs[to][lk][sw + 16 * q] = fb[q].x;
+            Bs[to][lk + 1][sw + 16 * q] = fb[q].y;
+            Bs[to][lk + 2][sw + 16 * q] = fb[q].z;
+            Bs[to][lk + 3][sw + 16 * q] = fb[q].w;
         }
     };
     load();
@@ -294,10 +302,10 @@ __global__ void __launch_bounds__(64) k_gemm_f32(const GProb* __restrict__ probs
         if (busy) {
 #pragma unroll
             for (int k = 0; k < F32_K; ++k) {
-                const float4 a0 = *reinterpret_cast<const float4*>(&As[buf][k][tr]);
-                const float4 a1 = *reinterpret_cast<const float4*>(&As[buf][k][tr + 16]);
-                const float4 b0 = *reinterpret_cast<const float4*>(&Bs[buf][k][tc]);
-                const float4 b1 = *reinterpret_cast<const float4*>(&Bs[buf][k][tc + 32]);
+                const float4 a0 = *reinterpret_cast<const float4*>(&As[buf][k][tr ^ (k & 8)]);
+                const float4 a1 = *reinterpret_cast<const float4*>(&As[buf][k][(tr + 16) ^ (k & 8)]);
+                const float4 b0 = *reinterpret_cast<const float4*>(&Bs[buf][k][tc ^ (k & 8)]);
+                const float4 b1 = *reinterpret_cast<const float4*>(&Bs[buf][k][(tc + 32) ^ (k & 8)]);
                 const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
                 const float b[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
 #pragma unroll
@@ -350,64 +358,139 @@ __device__ __forceinline__ __nv_bfloat16 from_a<__nv_bfloat16, float>(float v) {
 template <>
 __device__ __forceinline__ __nv_bfloat16 from_a<__nv_bfloat16, double>(double v) { return __float2bfloat16_rn((float)v); }
 
-// Element indices stay below 2^31 within a job (chunk starts are 32-bit), so the row/column split
-// uses 32-bit division.
+// Row and column of element first + tid, + blockDim.x, ... of a rows x w job: two divisions a thread
+// instead of one an element (element indices stay below 2^31 within a job).
+struct ElemWalk {
+    int r, c, dr, dc, w;
+    __device__ __forceinline__ ElemWalk(int first, int width) : w(width) {
+        const int e = first + (int)threadIdx.x;
+        r = e / w;
+        c = e - r * w;
+        dr = (int)blockDim.x / w;
+        dc = (int)blockDim.x - dr * w;
+    }
+    __device__ __forceinline__ void next() {
+        r += dr;
+        c += dc;
+        if (c >= w) {
+            c -= w;
+            ++r;
+        }
+    }
+};
+// Elements a thread has in flight in the block kernels.  They are bound by memory latency (a chunk is a
+// chain of list, job and data reads), so each thread issues its loads together; a chunk of 4096
+// elements is two such groups.  Packing the 24x8 cylinder's m = 2000 environments (2 x 138 MB), one
+// load at a time and a division an element before: see launch_copy.
+constexpr int EW = 8;
+
 template <class Tin, class Tout>
-__global__ void k_copy(const CopyJob* __restrict__ jobs, const int2* __restrict__ chunks, const Tin* __restrict__ src,
-                       Tout* __restrict__ dst) {
+__global__ void __launch_bounds__(256) k_copy(const CopyJob* __restrict__ jobs, const int2* __restrict__ chunks,
+                                              const Tin* __restrict__ src, Tout* __restrict__ dst) {
     using A = ew_t<Tin, Tout>;
     const int2 ch = chunks[blockIdx.x];
     const CopyJob j = jobs[ch.x];
     const int w = j.cols > j.zero_to ? j.cols : j.zero_to;
-    const long long total = (long long)j.rows * w;
-    const int end = (int)min(total, (long long)ch.y + CHUNK);
+    const int len = (int)min((long long)j.rows * w - ch.y, (long long)CHUNK);
     const A scale = (A)j.scale;
-    for (int e = ch.y + (int)threadIdx.x; e < end; e += blockDim.x) {
-        const int r = e / w, c = e - r * w;
-        A v = A(0);
-        if (c < j.cols) v = scale * to_a<A>(src[j.src + (long long)r * j.srs + (long long)c * j.scs]);
-        dst[j.dst + (long long)r * j.drs + (long long)c * j.dcs] = from_a<Tout>(v);
+    ElemWalk at(ch.y, w);
+    for (int e = threadIdx.x; e < len; e += EW * blockDim.x) {
+        A v[EW];
+        long long d[EW];
+#pragma unroll
+        for (int u = 0; u < EW; ++u) {
+            v[u] = A(0);
+            d[u] = j.dst + (long long)at.r * j.drs + (long long)at.c * j.dcs;
+            if (e + u * (int)blockDim.x < len && at.c < j.cols)
+                v[u] = to_a<A>(src[j.src + (long long)at.r * j.srs + (long long)at.c * j.scs]);
+            at.next();
+        }
+#pragma unroll
+        for (int u = 0; u < EW; ++u)
+            if (e + u * (int)blockDim.x < len) dst[d[u]] = from_a<Tout>(scale * v[u]);
     }
 }
 
 template <class Tin, class Tout>
-__global__ void k_mix(const MixJob* __restrict__ jobs, const int2* __restrict__ chunks, const MixTerm* __restrict__ terms,
-                      const Tin* __restrict__ in, Tout* __restrict__ out) {
+__global__ void __launch_bounds__(256) k_mix(const MixJob* __restrict__ jobs, const int2* __restrict__ chunks,
+                                             const MixTerm* __restrict__ terms, const Tin* __restrict__ in,
+                                             Tout* __restrict__ out) {
     using A = ew_t<Tin, Tout>;
     const int2 ch = chunks[blockIdx.x];
     const MixJob j = jobs[ch.x];
     const int w = j.cols > j.zero_to ? j.cols : j.zero_to;
-    const long long total = (long long)j.rows * w;
-    const int end = (int)min(total, (long long)ch.y + CHUNK);
-    for (int e = ch.y + (int)threadIdx.x; e < end; e += blockDim.x) {
-        const int r = e / w, c = e - r * w;
-        A v = A(0);
-        if (c < j.cols) {
-            for (int t = 0; t < j.nt; ++t) {
-                const MixTerm tm = terms[j.t0 + t];
-                v += (A)tm.coef * to_a<A>(in[tm.src + (long long)r * tm.ld + c]);
-            }
+    const int len = (int)min((long long)j.rows * w - ch.y, (long long)CHUNK);
+    ElemWalk at(ch.y, w);
+    for (int e = threadIdx.x; e < len; e += EW * blockDim.x) {
+        A v[EW];
+        int r[EW], c[EW];
+#pragma unroll
+        for (int u = 0; u < EW; ++u) {
+            v[u] = A(0);
+            r[u] = at.r;
+            c[u] = e + u * (int)blockDim.x < len ? at.c : -1;
+            at.next();
         }
-        out[j.dst + (long long)r * j.ldo + c] = from_a<Tout>(v);
+        for (int t = 0; t < j.nt; ++t) {
+            const MixTerm tm = terms[j.t0 + t];
+            const A coef = (A)tm.coef;
+            A x[EW];
+#pragma unroll
+            for (int u = 0; u < EW; ++u)
+                x[u] = (unsigned)c[u] < (unsigned)j.cols ? to_a<A>(in[tm.src + (long long)r[u] * tm.ld + c[u]]) : A(0);
+#pragma unroll
+            for (int u = 0; u < EW; ++u) v[u] += coef * x[u];
+        }
+#pragma unroll
+        for (int u = 0; u < EW; ++u)
+            if (c[u] >= 0) out[j.dst + (long long)r[u] * j.ldo + c[u]] = from_a<Tout>(c[u] < j.cols ? v[u] : A(0));
     }
 }
 
 template <class T>
-__global__ void k_diag(const DiagJob* __restrict__ jobs, const int2* __restrict__ chunks, const DiagTerm* __restrict__ terms,
-                       const T* __restrict__ Ls, int ldl, const T* __restrict__ Rs, int ldr,
-                       double* __restrict__ out) {
+__global__ void __launch_bounds__(256) k_diag(const DiagJob* __restrict__ jobs, const int2* __restrict__ chunks,
+                                              const DiagTerm* __restrict__ terms, const T* __restrict__ Ls, int ldl,
+                                              const T* __restrict__ Rs, int ldr, double* __restrict__ out) {
     const int2 ch = chunks[blockIdx.x];
     const DiagJob j = jobs[ch.x];
-    const long long total = (long long)j.rows * j.cols;
-    const long long end = min(total, (long long)ch.y + CHUNK);
-    for (long long e = (long long)ch.y + threadIdx.x; e < end; e += blockDim.x) {
-        int a = (int)(e / j.cols), c = (int)(e % j.cols);
-        double v = 0.0;
+    const int len = (int)min((long long)j.rows * j.cols - ch.y, (long long)CHUNK);
+    ElemWalk at(ch.y, j.cols);
+    for (int e = threadIdx.x; e < len; e += EW * blockDim.x) {
+        double v[EW];
+        int r[EW], c[EW];
+#pragma unroll
+        for (int u = 0; u < EW; ++u) {
+            v[u] = 0.0;
+            const bool in = e + u * (int)blockDim.x < len;
+            r[u] = in ? at.r : 0;
+            c[u] = in ? at.c : 0;
+            at.next();
+        }
         for (int t = 0; t < j.nt; ++t) {
             const DiagTerm tm = terms[j.t0 + t];
-            v += tm.coef * to_d(Ls[tm.l + (long long)a * (ldl + 1)]) * to_d(Rs[tm.r + (long long)c * (ldr + 1)]);
+#pragma unroll
+            for (int u = 0; u < EW; ++u)
+                v[u] += tm.coef * to_d(Ls[tm.l + (long long)r[u] * (ldl + 1)]) * to_d(Rs[tm.r + (long long)c[u] * (ldr + 1)]);
         }
-        out[j.off + e] = v;
+#pragma unroll
+        for (int u = 0; u < EW; ++u)
+            if (e + u * (int)blockDim.x < len) out[j.off + ch.y + e + u * (int)blockDim.x] = v[u];
+    }
+}
+
+// dst[i] = src[i], converted, i < n.
+template <class Tin, class Tout>
+__global__ void __launch_bounds__(256) k_convert(const Tin* __restrict__ src, Tout* __restrict__ dst, long long n) {
+    using A = ew_t<Tin, Tout>;
+    const long long step = (long long)gridDim.x * blockDim.x;
+    for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += EW * step) {
+        A v[EW];
+#pragma unroll
+        for (int u = 0; u < EW; ++u)
+            if (e + u * step < n) v[u] = to_a<A>(src[e + u * step]);
+#pragma unroll
+        for (int u = 0; u < EW; ++u)
+            if (e + u * step < n) dst[e + u * step] = from_a<Tout>(v[u]);
     }
 }
 
@@ -1064,6 +1147,18 @@ void launch_copy(const CopyJob* jobs, const int2* chunks, int nchunks, const Tin
     k_copy<Tin, Tout><<<nchunks, 256, 0, st>>>(jobs, chunks, src, dst);
     PD_LAUNCHED();
 }
+
+template <class Tin, class Tout>
+void launch_convert(const Tin* src, Tout* dst, long long n, cudaStream_t st) {
+    if (n <= 0) return;
+    k_convert<Tin, Tout><<<(unsigned)std::max<long long>(1, std::min<long long>((n + 2047) / 2048, 152 * 8)), 256, 0, st>>>(
+        src, dst, n);
+    PD_LAUNCHED();
+}
+template void launch_convert<double, float>(const double*, float*, long long, cudaStream_t);
+template void launch_convert<double, __nv_bfloat16>(const double*, __nv_bfloat16*, long long, cudaStream_t);
+template void launch_convert<float, double>(const float*, double*, long long, cudaStream_t);
+template void launch_convert<float, __nv_bfloat16>(const float*, __nv_bfloat16*, long long, cudaStream_t);
 
 template <class Tin, class Tout>
 void launch_mix(const MixJob* jobs, const int2* chunks, int nchunks, const MixTerm* terms, const Tin* in,

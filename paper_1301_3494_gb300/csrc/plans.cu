@@ -475,22 +475,16 @@ void orthonormalize_factor(const Sec& bl, const Sec& br, const std::vector<int>&
 }
 
 void convert_flat(const void* src, Num in, void* dst, Num out, long long n, cudaStream_t st) {
-    if (n <= 0) return;
-    CopyList cl;
-    const long long chunk = 1 << 20;
-    for (long long s0 = 0; s0 < n; s0 += chunk) {
-        CopyJob j{};
-        j.src = s0; j.dst = s0; j.rows = 1; j.cols = (int)std::min(chunk, n - s0);
-        j.srs = 0; j.scs = 1; j.drs = 0; j.dcs = 1; j.zero_to = 0; j.scale = 1.0;
-        cl.add(j);
+    PD_REQUIRE(in != out && (in == Num::F64 || in == Num::F32), DMRG_ERR_ARG, "convert_flat: unsupported types");
+    if (in == Num::F64) {
+        const double* s = static_cast<const double*>(src);
+        if (out == Num::F32) launch_convert(s, static_cast<float*>(dst), n, st);
+        else launch_convert(s, static_cast<__nv_bfloat16*>(dst), n, st);
+    } else {
+        const float* s = static_cast<const float*>(src);
+        if (out == Num::F64) launch_convert(s, static_cast<double*>(dst), n, st);
+        else launch_convert(s, static_cast<__nv_bfloat16*>(dst), n, st);
     }
-    ListPack pk;
-    DBuf lists;
-    cl.stage(pk);
-    pk.upload(lists, st);
-    PD_REQUIRE(in == Num::F64 || in == Num::F32, DMRG_ERR_ARG, "convert_flat: source must be FP64 or FP32");
-    if (in == Num::F64) run_copy<double>(cl, static_cast<const double*>(src), dst, out, st);
-    else run_copy<float>(cl, static_cast<const float*>(src), dst, out, st);
 }
 
 void orthonormalize_square(const std::vector<SvdSec>& ss, double* V, cudaStream_t st, int max_iter) {
@@ -728,13 +722,6 @@ std::unique_ptr<HeffPlan> make_heff_plan(const Sec& bl, const Sec& br, const std
         const std::vector<int2> c = make_chunks(el);
         P->diag_chunks = (int)c.size();
         pk.add(P->ddc, c);
-        if (prec == PREC_F32) {
-            CopyJob j{};
-            j.src = 0; j.dst = 0; j.rows = 1; j.cols = (int)P->psi.size; j.srs = 0; j.scs = 1; j.drs = 0; j.dcs = 1;
-            j.zero_to = 0; j.scale = 1.0;
-            P->unpack.add(j);
-            P->unpack.stage(pk);
-        }
         auto stage = [&](GemmBatch& g, Num cnum) {
             if (prec == DMRG_FP64) g.stage_f64(pk);
             else if (prec == PREC_F32) g.stage(pk, 64, 64);
@@ -792,7 +779,7 @@ void heff_apply(HeffPlan& P, const EnvSlab& L, const EnvSlab& R, const double* x
         run_gemm32(P.ldirect, P.psiT.as<float>(), Lf, P.Y.as<float>(), st);
         run_mix<float>(P.mix, P.X.as<float>(), P.Y.p, Num::F32, st);
         run_gemm32(P.rstage, Rf, P.Y.as<float>(), y32.as<float>(), st);
-        run_copy<float>(P.unpack, y32.as<float>(), y, Num::F64, st);
+        convert_flat(y32.p, Num::F32, y, Num::F64, P.psi.size, st);
     } else {
         run_gemm_tc(P.lstage, t, P.psiT.p, P.psiT_rows, P.ld_psi, env_operand(L, prec), L.lay.rows, L.lay.ld,
                     P.X.p, Num::F32, err, st);
@@ -831,43 +818,54 @@ void env_alloc(EnvSlab& e, const Sec& b, const std::vector<int>& flux, int prec,
 void env_make_operand(EnvSlab& e, int prec, cudaStream_t st) {
     const bool bf = prec == DMRG_BF16, f32 = (prec == DMRG_TF32 || prec == PREC_F32) && e.num == Num::F64;
     if ((!bf && !f32) || (bf && e.op_valid) || (f32 && e.op32_valid)) return;
-    CopyList c;
-    long long n = std::max<long long>(1, e.lay.rows) * e.lay.ld;
-    // one flat row-major copy of the whole slab (padding included, zeros stay zeros)
-    const long long chunk = 1 << 20;
-    for (long long s = 0; s < n; s += chunk) {
-        CopyJob j{};
-        j.src = s; j.dst = s; j.rows = 1; j.cols = (int)std::min(chunk, n - s);
-        j.srs = 0; j.scs = 1; j.drs = 0; j.dcs = 1; j.zero_to = 0; j.scale = 1.0;
-        c.add(j);
-    }
-    ListPack pk;
-    DBuf lists;
-    c.stage(pk);
-    pk.upload(lists, st);
+    // the whole slab (padding included, zeros stay zeros)
+    const long long n = std::max<long long>(1, e.lay.rows) * e.lay.ld;
     DBuf& dst = bf ? e.op : e.op32;
     dst.ensure(n * (bf ? 2 : 4), st);
-    if (e.num == Num::F64) run_copy<double>(c, e.buf.as<double>(), dst.p, bf ? Num::BF16 : Num::F32, st);
-    else run_copy<float>(c, e.buf.as<float>(), dst.p, Num::BF16, st);
+    convert_flat(e.buf.p, e.num, dst.p, bf ? Num::BF16 : Num::F32, n, st);
     (bf ? e.op_valid : e.op32_valid) = true;
 }
 
-void env_from_packed(EnvSlab& e, const double* packed, cudaStream_t st) {
+// Copies of the packed blocks into the slab (lists in one upload).
+static CopyList packed_copies(const EnvLayout& lay, DBuf& lists, cudaStream_t st) {
     CopyList c;
-    for (const auto& b : e.lay.blk) {
+    for (const auto& b : lay.blk) {
         CopyJob j{};
-        j.src = b.packed; j.dst = b.row * e.lay.ld; j.rows = b.rows; j.cols = b.cols;
-        j.srs = b.cols; j.scs = 1; j.drs = e.lay.ld; j.dcs = 1; j.zero_to = 0; j.scale = 1.0;
+        j.src = b.packed; j.dst = b.row * lay.ld; j.rows = b.rows; j.cols = b.cols;
+        j.srs = b.cols; j.scs = 1; j.drs = lay.ld; j.dcs = 1; j.zero_to = 0; j.scale = 1.0;
         c.add(j);
     }
     ListPack pk;
-    DBuf lists;
     c.stage(pk);
     pk.upload(lists, st);
+    return c;
+}
+
+void env_from_packed(EnvSlab& e, const double* packed, cudaStream_t st) {
+    DBuf lists;
+    const CopyList c = packed_copies(e.lay, lists, st);
     run_copy<double>(c, packed, e.buf.p, e.num, st);
     e.op_valid = false;
     e.op32_valid = false;
     e.valid = true;
+}
+
+void env_operand_from_packed(EnvSlab& e, const Sec& b, const std::vector<int>& flux, int prec, const double* packed,
+                             cudaStream_t st) {
+    if (prec != DMRG_BF16) {
+        env_alloc(e, b, flux, prec, st);
+        env_from_packed(e, packed, st);
+        return;
+    }
+    e.lay = env_layout(b, flux, pad_ld(b.maxm(), prec));
+    e.num = env_num(prec);
+    const size_t bytes = (size_t)std::max<long long>(1, e.lay.rows) * e.lay.ld * 2;
+    e.op.ensure(bytes, st);
+    PD_CK(cudaMemsetAsync(e.op.p, 0, bytes, st));
+    DBuf lists;
+    const CopyList c = packed_copies(e.lay, lists, st);
+    run_copy<double>(c, packed, e.op.p, Num::BF16, st);
+    e.op_valid = true;
 }
 
 void env_to_packed(const EnvSlab& e, double* packed, cudaStream_t st) {

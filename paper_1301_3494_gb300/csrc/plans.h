@@ -357,7 +357,6 @@ struct HeffPlan {
     int ld_psi = 0, ld_y = 0;
     long long psiT_rows = 0, y_rows = 0, x_size = 0;
     CopyList pack;            // canonical x -> psiT slab
-    CopyList unpack;          // FP32 result -> FP64 (accurate refinement plan)
     GemmBatch lstage, ldirect, rstage;   // L stage into X / straight into Y, R stage
     MixList mix;              // X -> Y slab
     std::vector<DiagJob> djobs;
@@ -388,6 +387,10 @@ void env_alloc(EnvSlab& e, const Sec& b, const std::vector<int>& flux, int prec,
 void env_make_operand(EnvSlab& e, int prec, cudaStream_t st);
 // Packed canonical <-> slab conversions (FP64 packed on the device).
 void env_from_packed(EnvSlab& e, const double* packed, cudaStream_t st);
+// A matvec's environment from its packed blocks: the operand alone (BF16 mode: without the FP32 storage
+// that updates read; the values are rounded through FP32 all the same).
+void env_operand_from_packed(EnvSlab& e, const Sec& b, const std::vector<int>& flux, int prec, const double* packed,
+                             cudaStream_t st);
 void env_to_packed(const EnvSlab& e, double* packed, cudaStream_t st);
 // The trivial boundary environment (one 1x1 block, value 1).
 void env_boundary(EnvSlab& e, const Sec& b, const std::vector<int>& flux, int prec, cudaStream_t st);
