@@ -244,12 +244,11 @@ struct BjSec {
     float tol;
     int blk0, pst0;
 };
-int bjacobi_max_rows();
+// border: 2 nblk words of scratch (zeroed; nblk = blocks of all sectors).
 void launch_bjacobi(const SvdSec* secs, const BjSec* bsecs, const int* task_sec, int ntasks, int nrounds, int max_rows,
-                    int max_n, int max_sweeps, int inner_sweeps, float* W, float* V, float noise_c, float* gmax,
-                    int* bmod, int* pchk, int* rot, int* sweeps, unsigned* bar, unsigned* err,
-                    unsigned long long* flops, const int2* items, int per_sweep, int nsec, int nact, int* qstate,
-                    cudaStream_t st);
+                    int max_sweeps, float* W, float* V, float noise_c, float* gmax, int* bmod, int* pchk, int* border,
+                    int nblk, int* rot, int* sweeps, unsigned* err, unsigned long long* flops, const int2* items,
+                    int per_sweep, int nsec, int nact, int* qstate, cudaStream_t st);
 template <class T>
 void launch_svd_finish(const SvdSec* secs, int nsec, int max_n, const T* W, double* sig, int* order, cudaStream_t st);
 

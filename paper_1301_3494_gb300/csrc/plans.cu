@@ -1301,11 +1301,10 @@ void col_copy(const std::vector<ColJob>& jobs, const double* src, double* dst, c
 // sig the column norms and ord their descending order; dsecs the device copy of ss.
 // FP32 block Jacobi (one task per block pair, n / 16 - 1 rounds per sweep) of the batch ss: W (p x n
 // at w_off), rotations accumulated into V (n x n at v_off, initialised by the caller); rot: sweep
-// histogram (max_sweeps + 1 ints, zeroed), bar: 3 zeroed barrier words, err: error word.  noise_c: the
-// absolute rounding level below which a pair is left (times sigma_max; 0: the relative test alone).
-void block_jacobi32(const std::vector<SvdSec>& ss, const SvdSec* dsecs, float* W, float* V, int max_rows, int max_n,
-                    int max_sweeps, int* rot, unsigned* bar, unsigned* err, unsigned long long* flops, cudaStream_t st,
-                    float noise_c = 8.0f * FLT_EPSILON) {
+// histogram (max_sweeps + 1 ints, zeroed), err: error word.  noise_c: the absolute rounding level below
+// which a pair is left (times sigma_max; 0: the relative test alone).
+void block_jacobi32(const std::vector<SvdSec>& ss, const SvdSec* dsecs, float* W, float* V, int max_rows, int max_sweeps,
+                    int* rot, unsigned* err, unsigned long long* flops, cudaStream_t st, float noise_c = 8.0f * FLT_EPSILON) {
     const int nsec = (int)ss.size();
     std::vector<BjSec> bs(nsec);
     std::vector<int> task_sec;
@@ -1348,18 +1347,20 @@ void block_jacobi32(const std::vector<SvdSec>& ss, const SvdSec* dsecs, float* W
     upload(dbs, bs, st);
     upload(dts, task_sec, st);
     upload(ditems, items, st);
-    const size_t nq = 3 + (size_t)nsec * (2 + bj_sweeps);
+    const size_t nq = 3 + (size_t)nsec * (1 + 2 * bj_sweeps);
     dq.ensure(nq * 4, st);
     PD_CK(cudaMemsetAsync(dq.p, 0, nq * 4, st));
     dgmax.ensure(std::max(1, nsec) * 4, st);
     PD_CK(cudaMemsetAsync(dgmax.p, 0, std::max(1, nsec) * 4, st));
-    // block / pair stamps (zero: never rotated / never found converged)
-    dstamp.ensure((size_t)std::max(1, nblk + npst) * 4, st);
-    PD_CK(cudaMemsetAsync(dstamp.p, 0, (size_t)std::max(1, nblk + npst) * 4, st));
+    // block / pair stamps (zero: never rotated / never found converged), the queue's ordering words
+    const size_t nstamp = (size_t)std::max(1, 3 * nblk + npst);
+    dstamp.ensure(nstamp * 4, st);
+    PD_CK(cudaMemsetAsync(dstamp.p, 0, nstamp * 4, st));
     PD_CK(cudaMemsetAsync(flops, 0, 8, st));
-    launch_bjacobi(dsecs, dbs.as<BjSec>(), dts.as<int>(), (int)task_sec.size(), nrounds, max_rows, max_n, bj_sweeps, 2,
-                   W, V, noise_c, dgmax.as<float>(), dstamp.as<int>(), dstamp.as<int>() + nblk, rot,
-                   rot + max_sweeps, bar, err, flops, ditems.as<int2>(), (int)items.size(), nsec, nact, dq.as<int>(), st);
+    int* stamps = dstamp.as<int>();
+    launch_bjacobi(dsecs, dbs.as<BjSec>(), dts.as<int>(), (int)task_sec.size(), nrounds, max_rows, bj_sweeps, W, V,
+                   noise_c, dgmax.as<float>(), stamps, stamps + nblk, stamps + nblk + npst, nblk, rot, rot + max_sweeps,
+                   err, flops, ditems.as<int2>(), (int)items.size(), nsec, nact, dq.as<int>(), st);
 }
 
 // Preconditioning of an FP64 one-sided Jacobi SVD of the batch ss (W FP64, p x n at w_off): the FP32
@@ -1367,7 +1368,7 @@ void block_jacobi32(const std::vector<SvdSec>& ss, const SvdSec* dsecs, float* W
 // (n x n at v_off), and W <- W V in FP64.  The FP64 Jacobi then starts from V with columns that are
 // orthogonal to FP32 accuracy, so its sweeps converge in the quadratic regime.
 void fp64_precondition(const std::vector<SvdSec>& ss, const SvdSec* dsecs, DBuf& dW, double* V, long long woff,
-                       long long voff, int maxp, int maxn, unsigned* bar, unsigned* err, cudaStream_t st) {
+                       long long voff, int maxp, int maxn, unsigned* err, cudaStream_t st) {
     const int max_sweeps = 60;
     DBuf w32, v32, rot32, fl, dW1;
     w32.ensure(woff * 4, st);
@@ -1375,10 +1376,9 @@ void fp64_precondition(const std::vector<SvdSec>& ss, const SvdSec* dsecs, DBuf&
     rot32.ensure((max_sweeps + 1) * 4, st);
     fl.ensure(8, st);
     PD_CK(cudaMemsetAsync(rot32.p, 0, (max_sweeps + 1) * 4, st));
-    PD_CK(cudaMemsetAsync(bar, 0, 3 * sizeof(unsigned), st));
     convert_flat(dW.p, Num::F64, w32.p, Num::F32, woff, st);
     launch_svd_init_v<float>(dsecs, (int)ss.size(), maxn, v32.as<float>(), st);
-    block_jacobi32(ss, dsecs, w32.as<float>(), v32.as<float>(), maxp, maxn, max_sweeps, rot32.as<int>(), bar, err,
+    block_jacobi32(ss, dsecs, w32.as<float>(), v32.as<float>(), maxp, max_sweeps, rot32.as<int>(), err,
                    fl.as<unsigned long long>(), st);
     convert_flat(v32.p, Num::F32, V, Num::F64, voff, st);
     orthonormalize_square(ss, V, st);
@@ -1388,7 +1388,6 @@ void fp64_precondition(const std::vector<SvdSec>& ss, const SvdSec* dsecs, DBuf&
             gwq.add(x.p, x.n, x.w_off, 1, x.p, x.n, 1, 1, x.p, {GSeg{x.w_off, x.v_off, x.n, 0}});
     dW1.ensure(woff * 8, st);
     run_gemm64(gwq, dW.as<double>(), V, dW1.as<double>(), st);
-    PD_CK(cudaMemsetAsync(bar, 0, 3 * sizeof(unsigned), st));
     dW = std::move(dW1);
 }
 
@@ -1479,7 +1478,7 @@ __global__ void k_polish_shift(const SvdSec* __restrict__ secs, const PolCol* __
 
 // Returns true when every pair of columns meets the tolerance (*passes: passes taken).
 bool polish64(const std::vector<SvdSec>& ss, const SvdSec* dsecs, DBuf& dW, DBuf& dV, long long woff, long long voff,
-              long long soff, unsigned* bar, unsigned* err, int* passes, cudaStream_t st) {
+              long long soff, unsigned* err, int* passes, cudaStream_t st) {
     const int nsec = (int)ss.size();
     std::vector<PolCol> cols;
     GemmBatch gG, gW, gV, gE;
@@ -1614,11 +1613,10 @@ bool polish64(const std::vector<SvdSec>& ss, const SvdSec* dsecs, DBuf& dW, DBuf
         upload(dsub, sub, st);
         down.up(st);
         PD_CK(cudaMemsetAsync(rot32.p, 0, (max_sweeps + 1) * 4, st));
-        PD_CK(cudaMemsetAsync(bar, 0, 3 * sizeof(unsigned), st));
         run_copy<double>(down, dW.as<double>(), w32.p, Num::F32, st);
         launch_svd_init_v<float>(dsub.as<SvdSec>(), (int)sub.size(), mn, v32.as<float>(), st);
-        block_jacobi32(sub, dsub.as<SvdSec>(), w32.as<float>(), v32.as<float>(), mp, mn, max_sweeps, rot32.as<int>(), bar,
-                       err, fl.as<unsigned long long>(), st, 0.0f);
+        block_jacobi32(sub, dsub.as<SvdSec>(), w32.as<float>(), v32.as<float>(), mp, max_sweeps, rot32.as<int>(), err,
+                       fl.as<unsigned long long>(), st, 0.0f);
         convert_flat(v32.p, Num::F32, v64.p, Num::F64, vo, st);
         orthonormalize_square(sub, v64.as<double>(), st);
         PD_CK(cudaMemcpyAsync(Wn.p, dW.p, woff * 8, cudaMemcpyDeviceToDevice, st));
@@ -1627,7 +1625,6 @@ bool polish64(const std::vector<SvdSec>& ss, const SvdSec* dsecs, DBuf& dW, DBuf
         run_gemm64(gv, dV.as<double>(), v64.as<double>(), Vn.as<double>(), st);
         std::swap(dW, Wn);
         std::swap(dV, Vn);
-        PD_CK(cudaMemsetAsync(bar, 0, 3 * sizeof(unsigned), st));
     }
     return false;
 }
@@ -1664,12 +1661,12 @@ void jacobi64(std::vector<SvdSec>& ss, DBuf& dWbuf, DBuf& dsecs, DBuf& dV, DBuf&
     unsigned* bar = dbar.as<unsigned>();
     const long long woff = ss.empty() ? 0 : ss.back().w_off + (long long)ss.back().p * ss.back().n;
     if (g_svd_qr && woff > 0)
-        fp64_precondition(ss, dsecs.as<SvdSec>(), dWbuf, dV.as<double>(), woff, voff, maxp, maxn, bar, bar + 3, st);
+        fp64_precondition(ss, dsecs.as<SvdSec>(), dWbuf, dV.as<double>(), woff, voff, maxp, maxn, bar + 3, st);
     else
         launch_svd_init_v<double>(dsecs.as<SvdSec>(), nsec, maxn, dV.as<double>(), st);
     int passes = 0;
     if (!(g_svd_qr && woff > 0 &&
-          polish64(ss, dsecs.as<SvdSec>(), dWbuf, dV, woff, voff, soff, bar, bar + 3, &passes, st)))
+          polish64(ss, dsecs.as<SvdSec>(), dWbuf, dV, woff, voff, soff, bar + 3, &passes, st)))
         launch_jacobi<double>(dsecs.as<SvdSec>(), nsec, dpairs.as<int>(), (int)pair_sec.size(), maxnpad, max_sweeps,
                               dWbuf.as<double>(), dV.as<double>(), 4.0 * DBL_EPSILON, 0.0, nullptr, drot.as<int>(),
                               drot.as<int>() + max_sweeps, bar, bar + 3, st);
@@ -1941,7 +1938,7 @@ std::vector<SplitResult> svd_split_batch(const std::vector<SplitReq>& reqs, bool
         }
         launch_svd_init_v<float>(jsecs, nsec, maxn, JV, st);
         // the kept factor that joins a block is re-orthonormalised in FP64 afterwards
-        block_jacobi32(use_qr ? xs : ss, jsecs, JW, JV, jmaxp, maxn, max_sweeps, drot.as<int>(), bar, jerr,
+        block_jacobi32(use_qr ? xs : ss, jsecs, JW, JV, jmaxp, max_sweeps, drot.as<int>(), jerr,
                        dflops.as<unsigned long long>(), st);
         if (use_qr) {
             DBuf dWo;
@@ -1959,12 +1956,12 @@ std::vector<SplitResult> svd_split_batch(const std::vector<SplitReq>& reqs, bool
         }
         const double tol = 4.0 * DBL_EPSILON;   // per sector: times sqrt(p)
         if (g_svd_qr && woff > 0)
-            fp64_precondition(ss, dsecs.as<SvdSec>(), dW, dV.as<double>(), woff, voff, maxp, maxn, bar, jerr, st);
+            fp64_precondition(ss, dsecs.as<SvdSec>(), dW, dV.as<double>(), woff, voff, maxp, maxn, jerr, st);
         else
             launch_svd_init_v<double>(dsecs.as<SvdSec>(), nsec, maxn, dV.as<double>(), st);
         int passes = 0;
         if (g_svd_qr && woff > 0 &&
-            polish64(ss, dsecs.as<SvdSec>(), dW, dV, woff, voff, soff, bar, jerr, &passes, st))
+            polish64(ss, dsecs.as<SvdSec>(), dW, dV, woff, voff, soff, jerr, &passes, st))
             PD_CK(cudaMemcpyAsync(drot.as<int>() + max_sweeps, &passes, sizeof(int), cudaMemcpyHostToDevice, st));
         else
             launch_jacobi<double>(dsecs.as<SvdSec>(), nsec, dpairs.as<int>(), npairs, maxnpad, max_sweeps,
