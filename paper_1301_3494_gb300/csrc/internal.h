@@ -195,21 +195,26 @@ inline std::vector<int2> make_chunks(const std::vector<long long>& elems) {
     return c;
 }
 
-// Davidson helpers (all FP64, vectors of length n, basis rows of stride ldv)
+// out[i] = V_i . y, i < k (rows of stride ldv, FP64)
 void launch_dots(const double* V, long long ldv, int k, const double* y, long long n,
                  double* partial, int nchunks, double* out, cudaStream_t st);
-void launch_ritz(const double* V, const double* AV, long long ldv, int k, const double* yth,
-                 long long n, double* u, double* Au, double* r, double* partial, int nchunks,
-                 double* norms, cudaStream_t st);
-void launch_precond(const double* r, const double* diag, const double* theta, double floor_,
-                    long long n, double* t, cudaStream_t st);
-void launch_subtract(const double* V, long long ldv, int k, const double* c, long long n,
-                     double* t, cudaStream_t st);
-void launch_scale(const double* x, const double* nrm2, long long n, double* y, int invert_sqrt,
-                  cudaStream_t st);
-void launch_small_eig(const double* G, int k, int ldg, double* yth, cudaStream_t st);
-void launch_nrm2(const double* x, long long n, double* partial, int nchunks, double* out,
-                 cudaStream_t st);
+
+// Davidson's vector work (FP64; vectors of length n, basis V and its images AV in rows of n).  partial:
+// 2 kmax * dav_grid(n) doubles of scratch; ctr: a zeroed word, zero again after each launch.
+int dav_grid(long long n);
+// column and row k of the kmax x kmax matrix G; eig: then yth[0] = lowest eigenvalue of its leading
+// (k + 1) x (k + 1) part, yth[1..k+1] = its vector
+void launch_dav_gram(const double* V, const double* AV, long long n, int k, int kmax, double* G, double* partial,
+                     unsigned* ctr, bool eig, double* yth, cudaStream_t st);
+// u = V y, Au = AV y, r = Au - theta u, norms = |r|^2, |u|^2
+void launch_dav_ritz(const double* V, const double* AV, long long n, int k, const double* yth, double* u, double* Au,
+                     double* r, double* partial, unsigned* ctr, double* norms, cudaStream_t st);
+// t = r / (theta - diag), twice orthogonalised against V's k rows (k >= 1); c1, c2: k words each
+void launch_dav_correct(const double* V, long long n, int k, const double* r, const double* diag, const double* theta,
+                        double fl, double* t, double* c1, double* c2, double* partial, unsigned* ctr, double* nrm2,
+                        cudaStream_t st);
+void launch_dav_norm(double* x, long long n, double* partial, unsigned* ctr, double* nrm2, cudaStream_t st);
+void launch_dav_unit(const double* x, const double* nrm2, double floor_, long long n, double* y, cudaStream_t st);
 void launch_finite_check(const double* x, long long n, unsigned* err, cudaStream_t st);
 
 // One-sided Jacobi SVD over a batch of column-major matrices W_s (p_s x n_s, n_s <= p_s)

@@ -495,7 +495,7 @@ __global__ void __launch_bounds__(256) k_convert(const Tin* __restrict__ src, To
 }
 
 // ------------------------------------------------------------------------------------------
-// Davidson vector kernels (FP64, deterministic two-pass reductions)
+// Dot product (FP64, deterministic two-pass reduction)
 // ------------------------------------------------------------------------------------------
 __global__ void k_dots_partial(const double* __restrict__ V, long long ldv, const double* __restrict__ y,
                                long long n, double* __restrict__ partial) {
@@ -516,63 +516,6 @@ __global__ void k_reduce_rows(const double* __restrict__ partial, int nchunks, d
     if (threadIdx.x == 0) out[i] = s;
 }
 
-// yth[0] = theta, yth[1..k] = Ritz coefficients.  norms[0] = |r|^2, norms[1] = |u|^2.
-__global__ void k_ritz(const double* __restrict__ V, const double* __restrict__ AV, long long ldv,
-                       int k, const double* __restrict__ yth, long long n, double* __restrict__ u,
-                       double* __restrict__ Au, double* __restrict__ r, double* __restrict__ partial) {
-    const int chunk = blockIdx.x, nchunks = gridDim.x;
-    const long long per = (n + nchunks - 1) / nchunks;
-    const long long b = chunk * per, e = min(n, b + per);
-    const double th = yth[0];
-    double sr = 0.0, su = 0.0;
-    for (long long x = b + threadIdx.x; x < e; x += blockDim.x) {
-        double uu = 0.0, aa = 0.0;
-        for (int i = 0; i < k; ++i) {
-            double yi = yth[1 + i];
-            uu = fma(yi, V[i * ldv + x], uu);
-            aa = fma(yi, AV[i * ldv + x], aa);
-        }
-        double rr = aa - th * uu;
-        u[x] = uu;
-        Au[x] = aa;
-        r[x] = rr;
-        sr = fma(rr, rr, sr);
-        su = fma(uu, uu, su);
-    }
-    sr = block_sum(sr);
-    su = block_sum(su);
-    if (threadIdx.x == 0) {
-        partial[chunk] = sr;
-        partial[nchunks + chunk] = su;
-    }
-}
-
-__global__ void k_precond(const double* __restrict__ r, const double* __restrict__ diag,
-                          const double* __restrict__ theta, double fl, long long n, double* __restrict__ t) {
-    const double th = theta[0];
-    for (long long x = (long long)blockIdx.x * blockDim.x + threadIdx.x; x < n; x += (long long)gridDim.x * blockDim.x) {
-        double den = th - diag[x];
-        if (fabs(den) < fl) den = den >= 0.0 ? fl : -fl;
-        t[x] = r[x] / den;
-    }
-}
-
-__global__ void k_subtract(const double* __restrict__ V, long long ldv, int k, const double* __restrict__ c,
-                           long long n, double* __restrict__ t) {
-    for (long long x = (long long)blockIdx.x * blockDim.x + threadIdx.x; x < n; x += (long long)gridDim.x * blockDim.x) {
-        double v = t[x];
-        for (int i = 0; i < k; ++i) v = fma(-c[i], V[i * ldv + x], v);
-        t[x] = v;
-    }
-}
-
-__global__ void k_scale(const double* __restrict__ x, const double* __restrict__ nrm2, long long n,
-                        double* __restrict__ y, int invert_sqrt) {
-    const double s = invert_sqrt ? 1.0 / sqrt(nrm2[0]) : nrm2[0];
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        y[i] = x[i] * s;
-}
-
 __global__ void k_finite(const double* __restrict__ x, long long n, unsigned* err) {
     bool bad = false;
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
@@ -581,9 +524,10 @@ __global__ void k_finite(const double* __restrict__ x, long long n, unsigned* er
 }
 
 // Lowest eigenpair of a small symmetric matrix (k <= 32) by cyclic Jacobi in FP64, one thread: the
-// general form, for matrices whose lowest eigenvalues the FP32 basis of k_small_eig cannot tell apart.
-__device__ __noinline__ void small_eig_serial(const double* __restrict__ G, int k, int ldg, double* __restrict__ yth) {
-    double a[32][32], v[32][32];
+// general form, for matrices whose lowest eigenvalues the FP32 basis of small_eig cannot tell apart.
+// (a, v: shared memory -- as local arrays they would reserve 16 KB for every resident thread of the GPU)
+__device__ __noinline__ void small_eig_serial(const double* G, int k, int ldg, double* yth, double (*a)[33],
+                                              double (*v)[33]) {
     for (int i = 0; i < k; ++i)
         for (int j = 0; j < k; ++j) {
             a[i][j] = 0.5 * (G[i * ldg + j] + G[j * ldg + i]);
@@ -635,13 +579,13 @@ __device__ __noinline__ void small_eig_serial(const double* __restrict__ G, int 
 // y <- y - sum_m q_m (q_m.r) / (lambda_m - theta), the sum in FP32 since it only has to be right to a
 // few digits.  The residual falls by ~1e-6 a pass; passes go on while it falls, and the pair is
 // accepted at |r| <= 32 eps |G|_F (the serial Jacobi's own backward error), else -- a cluster at the
-// bottom, or non-finite entries -- the serial form runs.  One call at k = 6: 300 -> about 10 us.
-__global__ void k_small_eig(const double* __restrict__ G, int k, int ldg, double* __restrict__ yth) {
+// bottom, or non-finite entries -- the serial form runs.  One call at k = 4-8, cold caches: 300 -> about 18 us.
+__device__ void small_eig(const double* G, int k, int ldg, double* yth) {
     constexpr unsigned ALL = 0xffffffffu;
-    __shared__ double A[32][33];
+    __shared__ double A[32][33], S[32][33];
     __shared__ float F[32][33], Q[32][33], cs[16], sn[16], rf[32], wf[32];
     __shared__ double ys[32];
-    const int lane = threadIdx.x;
+    const int lane = threadIdx.x & 31;
     double amax = 0.0, fro = 0.0;
     for (int i = 0; i < k; ++i)
         if (lane < k) {
@@ -671,6 +615,9 @@ __global__ void k_small_eig(const double* __restrict__ G, int k, int ldg, double
     double y = 0.0, theta = 0.0;
     if (ok) {
         const int kp = k + (k & 1), np = kp / 2;
+        // this lane's first 2 x 2 block (bi, bj) of F and first column pair rb of row rr of Q; 32 on,
+        // both move by the same step
+        const int bi0 = lane / np, bj0 = lane - bi0 * np, di = 32 / np, dj = 32 - di * np;
         for (int sweep = 0; sweep < 12 && k > 1; ++sweep) {
             float off = 0.f, dia = 0.f;
             for (int i = 0; i < k; ++i)
@@ -685,25 +632,30 @@ __global__ void k_small_eig(const double* __restrict__ G, int k, int ldg, double
             }
             if (off <= 1e-13f * dia) break;
             for (int round = 0; round < kp - 1; ++round) {
-                auto player = [&](int pos) { return pos == 0 ? 0 : ((pos - 1 + round) % (kp - 1)) + 1; };
+                auto player = [&](int pos) {       // pos - 1 + round modulo kp - 1, plus 1; 0 stays
+                    const int x = pos + round;
+                    return pos == 0 ? 0 : (x > kp - 1 ? x - (kp - 1) : x);
+                };
                 if (lane < np) {
                     const int p = player(lane), q = player(kp - 1 - lane);
                     float c = 1.f, s = 0.f;
                     if (p < k && q < k) {
-                        const float g = F[p][q];
-                        if (g != 0.f) {
-                            const float z = (F[q][q] - F[p][p]) / (2.f * g);
-                            const float t = copysignf(1.f, z) / (fabsf(z) + sqrtf(fmaf(z, z, 1.f)));
-                            c = 1.f / sqrtf(fmaf(t, t, 1.f));
-                            s = c * t;
+                        // cos 2t = |d| / sqrt(d^2 + h^2), c^2 = (1 + cos 2t) / 2: two reciprocal roots
+                        // (entries are at most 1; below 1e-18 nothing is left to turn, or to underflow)
+                        const float h = 2.f * F[p][q], d = F[q][q] - F[p][p];
+                        if (fabsf(h) > 1e-18f) {
+                            const float r = rsqrtf(fmaf(d, d, h * h));
+                            const float i = rsqrtf(fmaf(0.5f * fabsf(d), r, 0.5f));
+                            c = fmaf(0.5f * fabsf(d), r, 0.5f) * i;
+                            s = (d >= 0.f ? 0.5f : -0.5f) * h * r * i;
                         }
                     }
                     cs[lane] = c;
                     sn[lane] = s;
                 }
                 __syncwarp();
-                for (int e = lane; e < np * np; e += 32) {     // 2 x 2 blocks: they partition F
-                    const int bi = e / np, bj = e % np;
+                // (bj < np, so one carry a step) 2 x 2 blocks: they partition F
+                for (int bi = bi0, bj = bj0; bi < np;) {
                     const int p0 = player(bi), q0 = player(kp - 1 - bi), p1 = player(bj), q1 = player(kp - 1 - bj);
                     const float ci = cs[bi], si = sn[bi], cj = cs[bj], sj = sn[bj];
                     const float a = p0 < k && p1 < k ? F[p0][p1] : 0.f, b = p0 < k && q1 < k ? F[p0][q1] : 0.f;
@@ -713,13 +665,25 @@ __global__ void k_small_eig(const double* __restrict__ G, int k, int ldg, double
                     if (q0 < k && p1 < k) F[q0][p1] = si * a1 + ci * c1;
                     if (p0 < k && q1 < k) F[p0][q1] = ci * b1 - si * d1;
                     if (q0 < k && q1 < k) F[q0][q1] = si * b1 + ci * d1;
+                    bi += di;
+                    bj += dj;
+                    if (bj >= np) {
+                        bj -= np;
+                        ++bi;
+                    }
                 }
-                for (int e = lane; e < k * np; e += 32) {
-                    const int r = e / np, b = e % np, p = player(b), q = player(kp - 1 - b);
+                for (int r = bi0, b = bj0; r < k;) {
+                    const int p = player(b), q = player(kp - 1 - b);
                     if (p < k && q < k) {
                         const float x = Q[r][p], z = Q[r][q];
                         Q[r][p] = cs[b] * x - sn[b] * z;
                         Q[r][q] = sn[b] * x + cs[b] * z;
+                    }
+                    r += di;
+                    b += dj;
+                    if (b >= np) {
+                        b -= np;
+                        ++r;
                     }
                 }
                 __syncwarp();
@@ -778,11 +742,219 @@ __global__ void k_small_eig(const double* __restrict__ G, int k, int ldg, double
         }
     }
     if (!ok) {
-        if (lane == 0) small_eig_serial(G, k, ldg, yth);
+        __syncwarp();
+        if (lane == 0) small_eig_serial(G, k, ldg, yth, A, S);
         return;
     }
     if (lane == 0) yth[0] = ldexp(theta, ex);
     if (lane < k) yth[1 + lane] = y;
+}
+
+// ------------------------------------------------------------------------------------------
+// Davidson's vector work between two matvecs, six launches (FP64, deterministic).
+// Up to a few 10^4 elements these are launches of a few microseconds whose cost is the chain of them:
+// as single operations -- dots, row sums, place, eigenpair, Ritz, row sums, preconditioner, two
+// Gram-Schmidt passes of three, norm, scale: 18 launches and three host waits, 120 us a step with cold
+// caches against 60 here (chain m = 64; FP64 sweep over 16 sites 147 -> 115 ms).  Each launch ends in a
+// sum over all elements, and the CTA that arrives last adds up the CTAs' partial sums (in a fixed
+// order) and does what follows on k numbers.
+// Above, memory bounds them: V is read once a launch (three times in the correction, four before).
+// A CTA has 128 threads: the FP64 units take a warp instruction every 64 clocks a scheduler, so few
+// elements a CTA and a transposed warp reduction (9 additions for 8 sums instead of 40).
+// ------------------------------------------------------------------------------------------
+constexpr int DAV_THREADS = 128, DAV_GROUP = 8;
+
+// Sum of v[j] over the CTA in thread j < 8 (any value in others).
+__device__ __forceinline__ double dav_cta_sum(double (&v)[DAV_GROUP]) {
+    constexpr unsigned ALL = 0xffffffffu;
+    __shared__ double red[DAV_THREADS / 32][DAV_GROUP];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+#pragma unroll
+    for (int h = DAV_GROUP / 2, o = 16; h >= 1; h /= 2, o /= 2)       // halve the sums, double the lanes
+#pragma unroll
+        for (int j = 0; j < h; ++j) {
+            const bool up = lane & o;
+            v[j] = (up ? v[j + h] : v[j]) + __shfl_xor_sync(ALL, up ? v[j] : v[j + h], o);
+        }
+    v[0] += __shfl_xor_sync(ALL, v[0], 2);
+    v[0] += __shfl_xor_sync(ALL, v[0], 1);
+    __syncthreads();                                                   // red's last readers
+    if ((lane & 3) == 0) red[w][lane >> 2] = v[0];                     // bits 16, 8, 4 of the lane: j's bits
+    __syncthreads();
+    double s = 0.0;
+    if (threadIdx.x < DAV_GROUP)
+        s = (red[0][threadIdx.x] + red[1][threadIdx.x]) + (red[2][threadIdx.x] + red[3][threadIdx.x]);
+    return s;
+}
+// True in every thread of the CTA that arrives last (with every CTA's earlier writes visible);
+// *ctr is zero before and after a launch.
+__device__ __forceinline__ bool dav_last(unsigned* ctr) {
+    __shared__ unsigned last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(ctr, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!last) return false;
+    if (threadIdx.x == 0) *ctr = 0u;
+    __threadfence();
+    return true;
+}
+// Sum of a row of partial sums, one warp.
+__device__ __forceinline__ double dav_row(const double* partial, int row) {
+    const double* p = partial + (long long)row * gridDim.x;
+    double s = 0.0;
+    for (int c = threadIdx.x & 31; c < gridDim.x; c += 32) s += __ldcg(p + c);
+    return warp_sum(s);
+}
+#define DAV_FOR(x) \
+    for (long long x = (long long)blockIdx.x * DAV_THREADS + threadIdx.x; x < n; x += (long long)gridDim.x * DAV_THREADS)
+
+// G's new column k (V_i . AV_k, i <= k) and row (V_k . AV_i, i < k); eig: then the lowest pair of the
+// (k + 1) x (k + 1) matrix into yth (theta, coefficients).
+__global__ void __launch_bounds__(DAV_THREADS) k_dav_gram(const double* __restrict__ V, const double* __restrict__ AV,
+                                                          long long n, int k, int ldg, double* G, double* partial,
+                                                          unsigned* ctr, int eig, double* yth) {
+    const double* vk = V + k * n;
+    const double* ak = AV + k * n;
+    for (int i0 = 0; i0 <= k; i0 += DAV_GROUP / 2) {
+        double acc[DAV_GROUP] = {};
+        DAV_FOR(x) {
+            const double a = ak[x], v = vk[x];
+#pragma unroll
+            for (int j = 0; j < DAV_GROUP / 2; ++j) {
+                const long long o = (i0 + j) * n + x;
+                if (i0 + j <= k) acc[j] = fma(V[o], a, acc[j]);
+                if (i0 + j < k) acc[DAV_GROUP / 2 + j] = fma(AV[o], v, acc[DAV_GROUP / 2 + j]);
+            }
+        }
+        const double s = dav_cta_sum(acc);
+        const int j = threadIdx.x & (DAV_GROUP / 2 - 1);
+        if (threadIdx.x < DAV_GROUP && i0 + j <= k)
+            partial[(long long)(threadIdx.x < DAV_GROUP / 2 ? i0 + j : ldg + i0 + j) * gridDim.x + blockIdx.x] = s;
+    }
+    if (!dav_last(ctr)) return;
+    for (int i = threadIdx.x >> 5; i <= 2 * k; i += DAV_THREADS / 32) {     // k + 1 of the column, k of the row
+        const double s = dav_row(partial, i <= k ? i : ldg + i - k - 1);
+        if ((threadIdx.x & 31) == 0) G[i <= k ? (long long)i * ldg + k : (long long)k * ldg + i - k - 1] = s;
+    }
+    __syncthreads();
+    if (eig && threadIdx.x < 32) small_eig(G, k + 1, ldg, yth);
+}
+
+// u = V y, Au = AV y, r = Au - theta u; norms[0] = |r|^2, norms[1] = |u|^2.
+__global__ void __launch_bounds__(DAV_THREADS) k_dav_ritz(const double* __restrict__ V, const double* __restrict__ AV,
+                                                          long long n, int k, const double* __restrict__ yth,
+                                                          double* __restrict__ u, double* __restrict__ Au,
+                                                          double* __restrict__ r, double* partial, unsigned* ctr,
+                                                          double* __restrict__ norms) {
+    __shared__ double y[33];
+    if (threadIdx.x <= k) y[threadIdx.x] = yth[threadIdx.x];
+    __syncthreads();
+    double acc[DAV_GROUP] = {};
+    DAV_FOR(x) {
+        double uu = 0.0, aa = 0.0;
+#pragma unroll 4
+        for (int i = 0; i < k; ++i) {
+            uu = fma(y[1 + i], V[i * n + x], uu);
+            aa = fma(y[1 + i], AV[i * n + x], aa);
+        }
+        const double rr = aa - y[0] * uu;
+        u[x] = uu;
+        Au[x] = aa;
+        r[x] = rr;
+        acc[0] = fma(rr, rr, acc[0]);
+        acc[1] = fma(uu, uu, acc[1]);
+    }
+    const double s = dav_cta_sum(acc);
+    if (threadIdx.x < 2) partial[(long long)threadIdx.x * gridDim.x + blockIdx.x] = s;
+    if (!dav_last(ctr)) return;
+    if (threadIdx.x < 64) {
+        const double t = dav_row(partial, threadIdx.x >> 5);
+        if ((threadIdx.x & 31) == 0) norms[threadIdx.x >> 5] = t;
+    }
+}
+
+// Gram-Schmidt of the correction t against V_0 .. V_{k-1}, one pass per launch.  FIRST: t = r / (theta -
+// diag) (the denominator at least fl in size); else t -= V c.  Then c_out = V^T t.
+template <bool FIRST>
+__global__ void __launch_bounds__(DAV_THREADS) k_dav_correct(const double* __restrict__ V, long long n, int k,
+                                                             const double* __restrict__ r,
+                                                             const double* __restrict__ diag,
+                                                             const double* __restrict__ theta, double fl,
+                                                             const double* __restrict__ c, double* t, double* partial,
+                                                             unsigned* ctr, double* __restrict__ c_out) {
+    __shared__ double cs[32];
+    if (!FIRST && threadIdx.x < k) cs[threadIdx.x] = c[threadIdx.x];
+    __syncthreads();
+    const double th = FIRST ? theta[0] : 0.0;
+    for (int i0 = 0; i0 < k; i0 += DAV_GROUP) {
+        const int g = min(DAV_GROUP, k - i0);
+        double acc[DAV_GROUP] = {};
+        DAV_FOR(x) {
+            double v[DAV_GROUP], tx;
+#pragma unroll
+            for (int j = 0; j < DAV_GROUP; ++j) v[j] = j < g ? V[(i0 + j) * n + x] : 0.0;
+            if (i0 == 0) {
+                if (FIRST) {
+                    double den = th - diag[x];
+                    if (fabs(den) < fl) den = den >= 0.0 ? fl : -fl;
+                    tx = r[x] / den;
+                } else {
+                    tx = t[x];
+#pragma unroll
+                    for (int j = 0; j < DAV_GROUP; ++j)
+                        if (j < g) tx = fma(-cs[j], v[j], tx);
+                    for (int i = DAV_GROUP; i < k; ++i) tx = fma(-cs[i], V[i * n + x], tx);
+                }
+                t[x] = tx;
+            } else {
+                tx = t[x];                          // this thread's own write
+            }
+#pragma unroll
+            for (int j = 0; j < DAV_GROUP; ++j)
+                if (j < g) acc[j] = fma(v[j], tx, acc[j]);
+        }
+        const double s = dav_cta_sum(acc);
+        if (threadIdx.x < g) partial[(long long)(i0 + threadIdx.x) * gridDim.x + blockIdx.x] = s;
+    }
+    if (!dav_last(ctr)) return;
+    for (int i = threadIdx.x >> 5; i < k; i += DAV_THREADS / 32) {
+        const double s = dav_row(partial, i);
+        if ((threadIdx.x & 31) == 0) c_out[i] = s;
+    }
+}
+
+// t -= V c (k vectors; none: t is left), *nrm2 = |t|^2.
+__global__ void __launch_bounds__(DAV_THREADS) k_dav_norm(const double* __restrict__ V, long long n, int k,
+                                                          const double* __restrict__ c, double* t, double* partial,
+                                                          unsigned* ctr, double* __restrict__ nrm2) {
+    __shared__ double cs[32];
+    if (threadIdx.x < k) cs[threadIdx.x] = c[threadIdx.x];
+    __syncthreads();
+    double acc[DAV_GROUP] = {};
+    DAV_FOR(x) {
+        double tx = t[x];
+#pragma unroll 8
+        for (int i = 0; i < k; ++i) tx = fma(-cs[i], V[i * n + x], tx);
+        if (k > 0) t[x] = tx;
+        acc[0] = fma(tx, tx, acc[0]);
+    }
+    const double s = dav_cta_sum(acc);
+    if (threadIdx.x == 0) partial[blockIdx.x] = s;
+    if (!dav_last(ctr)) return;
+    if (threadIdx.x < 32) {
+        const double v = dav_row(partial, 0);
+        if (threadIdx.x == 0) *nrm2 = v;
+    }
+}
+
+// y = x / sqrt(*nrm2); zero where that root is below `floor_` (the caller stops there).
+__global__ void __launch_bounds__(256) k_dav_unit(const double* __restrict__ x, const double* __restrict__ nrm2,
+                                                  double floor_, long long n, double* __restrict__ y) {
+    const double root = sqrt(nrm2[0]);
+    const double s = root < floor_ ? 0.0 : 1.0 / root;
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
+        y[i] = s == 0.0 ? 0.0 : x[i] * s;
 }
 
 // ------------------------------------------------------------------------------------------
@@ -1197,39 +1369,43 @@ void launch_dots(const double* V, long long ldv, int k, const double* y, long lo
     PD_LAUNCHED();
 }
 
-void launch_ritz(const double* V, const double* AV, long long ldv, int k, const double* yth, long long n,
-                 double* u, double* Au, double* r, double* partial, int nchunks, double* norms, cudaStream_t st) {
-    k_ritz<<<nchunks, 256, 0, st>>>(V, AV, ldv, k, yth, n, u, Au, r, partial);
-    PD_LAUNCHED();
-    k_reduce_rows<<<2, 256, 0, st>>>(partial, nchunks, norms);
+int dav_grid(long long n) {
+    return (int)std::max<long long>(1, std::min<long long>((n + DAV_THREADS - 1) / DAV_THREADS, 152 * 4));
+}
+
+void launch_dav_gram(const double* V, const double* AV, long long n, int k, int kmax, double* G, double* partial,
+                     unsigned* ctr, bool eig, double* yth, cudaStream_t st) {
+    PD_REQUIRE(k >= 0 && k < kmax && kmax <= 32, DMRG_ERR_CAPACITY, "Davidson subspace larger than 32");
+    k_dav_gram<<<dav_grid(n), DAV_THREADS, 0, st>>>(V, AV, n, k, kmax, G, partial, ctr, eig ? 1 : 0, yth);
     PD_LAUNCHED();
 }
 
-void launch_precond(const double* r, const double* diag, const double* theta, double fl, long long n,
-                    double* t, cudaStream_t st) {
-    k_precond<<<grid_for(n), 256, 0, st>>>(r, diag, theta, fl, n, t);
+void launch_dav_ritz(const double* V, const double* AV, long long n, int k, const double* yth, double* u, double* Au,
+                     double* r, double* partial, unsigned* ctr, double* norms, cudaStream_t st) {
+    k_dav_ritz<<<dav_grid(n), DAV_THREADS, 0, st>>>(V, AV, n, k, yth, u, Au, r, partial, ctr, norms);
     PD_LAUNCHED();
 }
 
-void launch_subtract(const double* V, long long ldv, int k, const double* c, long long n, double* t,
-                     cudaStream_t st) {
-    k_subtract<<<grid_for(n), 256, 0, st>>>(V, ldv, k, c, n, t);
+void launch_dav_correct(const double* V, long long n, int k, const double* r, const double* diag, const double* theta,
+                        double fl, double* t, double* c1, double* c2, double* partial, unsigned* ctr, double* nrm2,
+                        cudaStream_t st) {
+    k_dav_correct<true><<<dav_grid(n), DAV_THREADS, 0, st>>>(V, n, k, r, diag, theta, fl, nullptr, t, partial, ctr, c1);
+    PD_LAUNCHED();
+    k_dav_correct<false>
+        <<<dav_grid(n), DAV_THREADS, 0, st>>>(V, n, k, nullptr, nullptr, nullptr, 0.0, c1, t, partial, ctr, c2);
+    PD_LAUNCHED();
+    k_dav_norm<<<dav_grid(n), DAV_THREADS, 0, st>>>(V, n, k, c2, t, partial, ctr, nrm2);
     PD_LAUNCHED();
 }
 
-void launch_scale(const double* x, const double* nrm2, long long n, double* y, int invert_sqrt, cudaStream_t st) {
-    k_scale<<<grid_for(n), 256, 0, st>>>(x, nrm2, n, y, invert_sqrt);
+void launch_dav_norm(double* x, long long n, double* partial, unsigned* ctr, double* nrm2, cudaStream_t st) {
+    k_dav_norm<<<dav_grid(n), DAV_THREADS, 0, st>>>(nullptr, n, 0, nullptr, x, partial, ctr, nrm2);
     PD_LAUNCHED();
 }
 
-void launch_small_eig(const double* G, int k, int ldg, double* yth, cudaStream_t st) {
-    PD_REQUIRE(k >= 1 && k <= 32, DMRG_ERR_CAPACITY, "Davidson subspace larger than 32");
-    k_small_eig<<<1, 32, 0, st>>>(G, k, ldg, yth);
+void launch_dav_unit(const double* x, const double* nrm2, double floor_, long long n, double* y, cudaStream_t st) {
+    k_dav_unit<<<grid_for(n), 256, 0, st>>>(x, nrm2, floor_, n, y);
     PD_LAUNCHED();
-}
-
-void launch_nrm2(const double* x, long long n, double* partial, int nchunks, double* out, cudaStream_t st) {
-    launch_dots(x, 0, 1, x, n, partial, nchunks, out, st);
 }
 
 void launch_finite_check(const double* x, long long n, unsigned* err, cudaStream_t st) {

@@ -298,14 +298,6 @@ __global__ void k_lam_out(const LamJob* jobs, int njobs, const double* sig, cons
     }
 }
 
-__global__ void k_place(double* G, int ldg, int k, const double* col, const double* row) {
-    // G[i*ldg + k] = col[i] (i <= k);  G[k*ldg + i] = row[i] (i < k)
-    for (int i = threadIdx.x; i <= k; i += blockDim.x) {
-        G[(long long)i * ldg + k] = col[i];
-        if (i < k) G[(long long)k * ldg + i] = row[i];
-    }
-}
-
 inline int gridn(long long n, int cap = 2048) {
     long long g = (n + 255) / 256;
     return (int)std::max<long long>(1, std::min<long long>(g, cap));
@@ -2150,35 +2142,51 @@ DavResult davidson(HeffPlan& P, const EnvSlab& L, const EnvSlab& R, double* x, i
     const long long n = P.psi.size;
     PD_REQUIRE(kmax >= 2 && kmax <= 32, DMRG_ERR_ARG, "Davidson kmax must be in [2, 32]");
     DavResult res;
-    const int nch = (int)std::max<long long>(1, std::min<long long>(512, (n + 4095) / 4096));
-    DBuf dV, dAV, dG, dyth, dpart, dd1, dd2, dnrm, du, dAu, dr, dt, ddg;
+    DBuf dV, dAV, dG, dyth, dpart, dc, dnrm, du, dAu, dr, dt, ddg, dctr;
     dV.ensure((size_t)kmax * n * 8, st);
     dAV.ensure((size_t)kmax * n * 8, st);
     dG.ensure((size_t)kmax * kmax * 8, st);
     dyth.ensure((kmax + 1) * 8, st);
-    dpart.ensure((size_t)std::max(2, kmax) * nch * 8, st);
-    dd1.ensure((kmax + 1) * 8, st);
-    dd2.ensure((kmax + 1) * 8, st);
-    dnrm.ensure(4 * 8, st);
+    dpart.ensure((size_t)2 * kmax * dav_grid(n) * 8, st);
+    dc.ensure(2 * kmax * 8, st);
+    dnrm.ensure(4 * 8, st);                     // |r|^2, |u|^2, |t|^2, |x|^2
+    dctr.ensure(sizeof(unsigned), st);
     du.ensure(n * 8, st);
     dAu.ensure(n * 8, st);
     dr.ensure(n * 8, st);
     dt.ensure(n * 8, st);
     ddg.ensure(n * 8, st);
+    PD_CK(cudaMemsetAsync(dctr.p, 0, sizeof(unsigned), st));
     double* V = dV.as<double>();
     double* AV = dAV.as<double>();
     double* G = dG.as<double>();
-    cudaEvent_t e0, e1;
-    PD_CK(cudaEventCreate(&e0));
-    PD_CK(cudaEventCreate(&e1));
+    double* part = dpart.as<double>();
+    double* nrm = dnrm.as<double>();
+    unsigned* ctr = dctr.as<unsigned>();
+    double* hn = reinterpret_cast<double*>(sweep_flags_host(64));   // pinned: |r|^2, |u|^2, |t|^2, theta
+    constexpr double kFloor = 1e-14;            // a correction this small is rounding
+    struct Events {
+        cudaEvent_t e[4] = {};
+        Events() {
+            for (int i = 0; i < 4; ++i)
+                PD_CK(i < 2 ? cudaEventCreate(&e[i]) : cudaEventCreateWithFlags(&e[i], cudaEventDisableTiming));
+        }
+        ~Events() {
+            for (auto x : e)
+                if (x) cudaEventDestroy(x);
+        }
+    } ev;
     HeffPlan* cur = &P;
+    // matvec timed by a pair of events, which is read at the next wait (the stream does not stop for it)
     auto mv = [&](const double* in, double* out) {
-        PD_CK(cudaEventRecord(e0, st));
+        PD_CK(cudaEventRecord(ev.e[0], st));
         heff_apply(*cur, L, R, in, out, err, st);
-        PD_CK(cudaEventRecord(e1, st));
-        PD_CK(cudaEventSynchronize(e1));
+        PD_CK(cudaEventRecord(ev.e[1], st));
+    };
+    auto mv_done = [&]() {
         float ms = 0.f;
-        PD_CK(cudaEventElapsedTime(&ms, e0, e1));
+        PD_CK(cudaEventSynchronize(ev.e[1]));
+        PD_CK(cudaEventElapsedTime(&ms, ev.e[0], ev.e[1]));
         if (cur == &P) {
             res.mv_ms += ms;
             res.matvecs++;
@@ -2188,60 +2196,50 @@ DavResult davidson(HeffPlan& P, const EnvSlab& L, const EnvSlab& R, double* x, i
         }
     };
     heff_diag(P, L, R, ddg.as<double>(), st);
-    double hn[4];
-    // one Davidson run from the normalised vector in x; leaves the Ritz vector in du (|u|^2 in dnrm[1])
+    // One Davidson run from the vector in x; leaves the Ritz vector in du (|u|^2 in nrm[1]).  The host
+    // queues ahead of the stream: the correction vector is made before the residual's norm is read, and
+    // the matvec before the correction's norm is (what a stop makes superfluous is a few vector launches
+    // or, with an exhausted subspace, a matvec of the zero vector, which is not counted).
     auto run = [&](int iters) {
-        launch_nrm2(x, n, dpart.as<double>(), nch, dnrm.as<double>(), st);
-        launch_scale(x, dnrm.as<double>(), n, V, 1, st);
+        launch_dav_norm(x, n, part, ctr, nrm + 3, st);
+        launch_dav_unit(x, nrm + 3, 0.0, n, V, st);
         mv(V, AV);
         int k = 1;
-        launch_dots(V, n, 1, AV, n, dpart.as<double>(), nch, dd1.as<double>(), st);
-        k_place<<<1, 32, 0, st>>>(G, kmax, 0, dd1.as<double>(), dd1.as<double>());
-        PD_LAUNCHED();
         for (int it = 1; it <= iters; ++it) {
             res.iters++;
-            launch_small_eig(G, k, kmax, dyth.as<double>(), st);
-            launch_ritz(V, AV, n, k, dyth.as<double>(), n, du.as<double>(), dAu.as<double>(), dr.as<double>(),
-                        dpart.as<double>(), nch, dnrm.as<double>(), st);
-            PD_CK(cudaMemcpyAsync(hn, dnrm.p, 16, cudaMemcpyDeviceToHost, st));
-            PD_CK(cudaMemcpyAsync(hn + 2, dyth.p, 8, cudaMemcpyDeviceToHost, st));
-            PD_CK(cudaStreamSynchronize(st));
-            res.theta = hn[2];
+            launch_dav_gram(V, AV, n, k - 1, kmax, G, part, ctr, true, dyth.as<double>(), st);
+            launch_dav_ritz(V, AV, n, k, dyth.as<double>(), du.as<double>(), dAu.as<double>(), dr.as<double>(), part, ctr,
+                            nrm, st);
+            PD_CK(cudaMemcpyAsync(hn, nrm, 16, cudaMemcpyDeviceToHost, st));
+            PD_CK(cudaMemcpyAsync(hn + 3, dyth.p, 8, cudaMemcpyDeviceToHost, st));
+            PD_CK(cudaEventRecord(ev.e[2], st));
+            if (it < iters) {
+                if (k >= kmax) {   // restart from the Ritz vector
+                    launch_dav_unit(du.as<double>(), nrm + 1, 0.0, n, V, st);
+                    launch_dav_unit(dAu.as<double>(), nrm + 1, 0.0, n, AV, st);
+                    k = 1;
+                    launch_dav_gram(V, AV, n, 0, kmax, G, part, ctr, false, nullptr, st);
+                }
+                launch_dav_correct(V, n, k, dr.as<double>(), ddg.as<double>(), dyth.as<double>(), 1e-4, dt.as<double>(),
+                                   dc.as<double>(), dc.as<double>() + kmax, part, ctr, nrm + 2, st);
+                launch_dav_unit(dt.as<double>(), nrm + 2, kFloor, n, V + (size_t)k * n, st);
+                PD_CK(cudaMemcpyAsync(hn + 2, nrm + 2, 8, cudaMemcpyDeviceToHost, st));
+                PD_CK(cudaEventRecord(ev.e[3], st));
+            }
+            mv_done();
+            PD_CK(cudaEventSynchronize(ev.e[2]));
+            res.theta = hn[3];
             res.rnorm = std::sqrt(std::max(0.0, hn[0]));
             PD_REQUIRE(std::isfinite(res.theta) && std::isfinite(res.rnorm), DMRG_ERR_NUMERIC,
                        "non-finite Ritz value in Davidson");
             if (res.rnorm <= tol * std::max(1.0, std::fabs(res.theta)) || it == iters) break;
-            launch_precond(dr.as<double>(), ddg.as<double>(), dyth.as<double>(), 1e-4, n, dt.as<double>(), st);
-            if (k >= kmax) {   // restart from the Ritz vector
-                launch_scale(du.as<double>(), dnrm.as<double>() + 1, n, V, 1, st);
-                launch_scale(dAu.as<double>(), dnrm.as<double>() + 1, n, AV, 1, st);
-                k = 1;
-                launch_dots(V, n, 1, AV, n, dpart.as<double>(), nch, dd1.as<double>(), st);
-                k_place<<<1, 32, 0, st>>>(G, kmax, 0, dd1.as<double>(), dd1.as<double>());
-                PD_LAUNCHED();
-            }
-            for (int pass = 0; pass < 2; ++pass) {
-                launch_dots(V, n, k, dt.as<double>(), n, dpart.as<double>(), nch, dd1.as<double>(), st);
-                launch_subtract(V, n, k, dd1.as<double>(), n, dt.as<double>(), st);
-            }
-            launch_nrm2(dt.as<double>(), n, dpart.as<double>(), nch, dnrm.as<double>() + 2, st);
-            double tn2 = 0.0;
-            PD_CK(cudaMemcpyAsync(&tn2, dnrm.as<double>() + 2, 8, cudaMemcpyDeviceToHost, st));
-            PD_CK(cudaStreamSynchronize(st));
-            if (std::sqrt(tn2) < 1e-14) break;
-            double* vk = V + (size_t)k * n;
-            double* avk = AV + (size_t)k * n;
-            launch_scale(dt.as<double>(), dnrm.as<double>() + 2, n, vk, 1, st);
-            mv(vk, avk);
-            // new column k: G[i][k] = V_i . AV_k (i <= k); new row: G[k][i] = V_k . AV_i (i < k)
-            launch_dots(V, n, k + 1, avk, n, dpart.as<double>(), nch, dd1.as<double>(), st);
-            launch_dots(AV, n, k, vk, n, dpart.as<double>(), nch, dd2.as<double>(), st);
-            k_place<<<1, 32, 0, st>>>(G, kmax, k, dd1.as<double>(), dd2.as<double>());
-            PD_LAUNCHED();
+            mv(V + (size_t)k * n, AV + (size_t)k * n);
+            PD_CK(cudaEventSynchronize(ev.e[3]));
+            if (std::sqrt(hn[2]) < kFloor) break;
             ++k;
         }
         // x = u / |u|
-        launch_scale(du.as<double>(), dnrm.as<double>() + 1, n, x, 1, st);
+        launch_dav_unit(du.as<double>(), nrm + 1, 0.0, n, x, st);
     };
     run(max_iter);
     if (acc && refine_iters > 0) {
@@ -2250,8 +2248,6 @@ DavResult davidson(HeffPlan& P, const EnvSlab& L, const EnvSlab& R, double* x, i
         run(refine_iters);
     }
     PD_CK(cudaStreamSynchronize(st));
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
     return res;
 }
 
