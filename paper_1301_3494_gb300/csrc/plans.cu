@@ -353,54 +353,163 @@ __global__ void k_ns_prep(const NsJob* jobs, const double* G, double* T) {
         T[j.off + e] = (r == c ? 1.5 : 0.0) - 0.5 * gram_at(G, j, r, c);
     }
 }
-// dev[s] = max |G - I| of block s (zeroed before; non-negative doubles order like their bits).  CTAs
-// share a block: one CTA each took 1.2 ms for the blocks of an m = 2000 bond.
-__global__ void k_gram_dev(const NsJob* jobs, const double* G, unsigned long long* dev) {
+// E_j = G_j - I (both triangles), T_j = I - E_j / 2
+__global__ void k_ns_start(const NsJob* jobs, const double* G, double* E, double* T) {
     const NsJob j = jobs[blockIdx.y];
-    unsigned long long m = 0;
+    const int total = j.k * j.k;
+    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < total; e += gridDim.x * blockDim.x) {
+        const int c = e / j.k, r = e - c * j.k;
+        const double one = r == c ? 1.0 : 0.0, d = gram_at(G, j, r, c) - one;
+        E[j.off + e] = d;
+        T[j.off + e] = fma(-0.5, d, one);
+    }
+}
+// S_j's upper triangle from its lower one; E_j <- 3/8 I - 5/16 E_j + 35/128 S_j
+__global__ void k_ns_quintic(const NsJob* jobs, double* S, double* E) {
+    const NsJob j = jobs[blockIdx.y];
+    const int total = j.k * j.k;
+    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < total; e += gridDim.x * blockDim.x) {
+        const int c = e / j.k, r = e - c * j.k;
+        const double s = gram_at(S, j, r, c);
+        if (r < c) S[j.off + e] = s;
+        E[j.off + e] = fma(0.2734375, s, fma(-0.3125, E[j.off + e], r == c ? 0.375 : 0.0));
+    }
+}
+// T_j's upper triangle from its lower one
+__global__ void k_mirror(const NsJob* jobs, double* T) {
+    const NsJob j = jobs[blockIdx.y];
+    const int total = j.k * j.k;
+    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < total; e += gridDim.x * blockDim.x) {
+        const int c = e / j.k, r = e - c * j.k;
+        if (r < c) T[j.off + e] = T[j.off + c + (long long)r * j.k];
+    }
+}
+// dev[2 x] = max |G - I|, dev[2 x + 1] = sum of (G - I)^2 over CTA x's columns of block s (x = s gridDim.x +
+// blockIdx.x).  CTAs share a block: one CTA each took 1.2 ms for the blocks of an m = 2000 bond.
+__global__ void __launch_bounds__(128) k_gram_dev(const NsJob* jobs, const double* G, float* dev) {
+    const NsJob j = jobs[blockIdx.y];
+    float m = 0.f, f = 0.f;
     for (int c = blockIdx.x; c < j.k; c += gridDim.x)
         for (int r = c + threadIdx.x; r < j.k; r += blockDim.x) {
-            const double d = fabs(G[j.off + r + (long long)c * j.k] - (r == c ? 1.0 : 0.0));
-            const unsigned long long b = (unsigned long long)__double_as_longlong(d);
-            if (d == d && b > m) m = b;
+            const float d = fabsf((float)(G[j.off + r + (long long)c * j.k] - (r == c ? 1.0 : 0.0)));
+            m = fmaxf(m, d);                                   // (NaN is passed over)
+            f = fmaf(r == c ? d : 2.f * d, d, f);
         }
     for (int o = 16; o > 0; o >>= 1) {
-        const unsigned long long w = __shfl_xor_sync(0xffffffffu, m, o);
-        m = w > m ? w : m;
+        m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+        f += __shfl_xor_sync(0xffffffffu, f, o);
     }
-    if ((threadIdx.x & 31) == 0 && m) atomicMax(dev + blockIdx.y, m);
+    __shared__ float sm[4], sf[4];
+    if ((threadIdx.x & 31) == 0) {
+        sm[threadIdx.x >> 5] = m;
+        sf[threadIdx.x >> 5] = f;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        float* o = dev + 2 * ((long long)blockIdx.y * gridDim.x + blockIdx.x);
+        o[0] = fmaxf(fmaxf(sm[0], sm[1]), fmaxf(sm[2], sm[3]));
+        o[1] = (sf[0] + sf[1]) + (sf[2] + sf[3]);
+    }
 }
 
-// max |G - I| over all blocks, on the host.
-double gram_deviation(const DBuf& djobs, const std::vector<NsJob>& jobs, const DBuf& G, DBuf& dev, cudaStream_t st) {
+// Over all blocks, on the host: max |G - I|, and the largest Frobenius norm of a block's G - I.
+struct GramDev { double max, fro; };
+GramDev gram_deviation(const DBuf& djobs, const std::vector<NsJob>& jobs, const DBuf& G, DBuf& dev, cudaStream_t st) {
     const int n = (int)jobs.size();
     int kmax = 1;
     for (const NsJob& j : jobs) kmax = std::max(kmax, j.k);
-    dev.ensure((size_t)n * 8, st);
-    PD_CK(cudaMemsetAsync(dev.p, 0, (size_t)n * 8, st));
-    k_gram_dev<<<dim3(std::min(kmax, 32), (unsigned)n), 128, 0, st>>>(djobs.as<NsJob>(), G.as<double>(),
-                                                                      dev.as<unsigned long long>());
+    const int ctas = std::min(kmax, 32);
+    std::vector<float> h((size_t)2 * n * ctas);
+    dev.ensure(h.size() * 4, st);
+    k_gram_dev<<<dim3(ctas, (unsigned)n), 128, 0, st>>>(djobs.as<NsJob>(), G.as<double>(), dev.as<float>());
     PD_LAUNCHED();
-    std::vector<double> h(n);
-    PD_CK(cudaMemcpyAsync(h.data(), dev.p, (size_t)n * 8, cudaMemcpyDeviceToHost, st));
+    PD_CK(cudaMemcpyAsync(h.data(), dev.p, h.size() * 4, cudaMemcpyDeviceToHost, st));
     PD_CK(cudaStreamSynchronize(st));
-    double worst = 0.0;
-    for (double v : h) worst = std::max(worst, v);
-    return worst;
+    GramDev d{0.0, 0.0};
+    for (int s = 0; s < n; ++s) {
+        double f = 0.0;
+        for (int x = 0; x < ctas; ++x) {
+            d.max = std::max(d.max, (double)h[2 * ((size_t)s * ctas + x)]);
+            f += h[2 * ((size_t)s * ctas + x) + 1];
+        }
+        // (a sum that overflowed, or NaN, settles nothing)
+        d.fro = f <= 1e30 ? std::max(d.fro, std::sqrt(f)) : 1e30;
+    }
+    return d;
 }
 
 // Adds to g the lower triangle of the k x k Gram block at c_off, 64 columns at a time: half the work of
 // the square.  Column i of segment s starts at segs[s].a_off + i sam; strides as for GemmBatch::add.
-void add_gram(GemmBatch& g, int k, long long c_off, int sam, int sak, const std::vector<GSeg>& segs, int accumulate = 0) {
+void add_gram(GemmBatch& g, int k, long long c_off, int sam, int sak, const std::vector<GSeg>& segs, int accumulate = 0,
+              double alpha = 1.0) {
     for (int j0 = 0; j0 < k; j0 += 64) {
         std::vector<GSeg> sg = segs;
         for (GSeg& x : sg) {
             x.a_off += (long long)j0 * sam;
             x.b_off = x.a_off;
         }
-        g.add(k - j0, std::min(64, k - j0), c_off + j0 + (long long)j0 * k, sam, sak, sam, sak, 1, k, sg, accumulate);
+        g.add(k - j0, std::min(64, k - j0), c_off + j0 + (long long)j0 * k, sam, sak, sam, sak, 1, k, sg, accumulate, alpha);
     }
 }
+
+// T ~ G^(-1/2), so that X T has orthonormal columns to `goal` where that is in reach.  With E = G - I,
+// the series of (1 + E)^(-1/2) cut after
+//   - E / 2 (a Newton-Schulz step)               leaves |X'^T X' - I| <= 3/4 |E|^2,
+//   3/8 E^2                                      5/8 |E|^3,
+//   E^2 (3/8 - 5/16 E + 35/128 E^2)              63/128 |E|^5
+// (spectral norms; the Frobenius norm bounds them).  The shortest whose bound meets the goal is the last
+// step: the Gram matrix is not formed again to see it.  From an FP32 Jacobi's rotations (1e-6 to 1e-4 an
+// element) that is one Gram matrix, one or two triangular products and one product instead of three Gram
+// matrices and two products, and one host wait instead of three: FP64 split of the 512-state chain bond
+// 20.3 -> 18.5 ms, accurate split of the cylinder's m = 1000 bond 36.3 -> 31.3, four mixed splits at m =
+// 2000 40.1 -> 37.4, a 16-site FP64 sweep at m = 64 115 -> 98.
+struct NsStep {
+    const DBuf& dj;
+    const std::vector<NsJob>& jobs;
+    DBuf E, S;
+    GemmBatch gT, gS, gP;                 // T += 3/8 E E;  S = E E;  T += S P (lower triangles)
+    int mx = 1;
+    long long size = 0;
+    NsStep(const DBuf& dj_, const std::vector<NsJob>& jobs_) : dj(dj_), jobs(jobs_) {
+        for (const NsJob& j : jobs) {
+            mx = std::max(mx, j.k * j.k);
+            size = std::max(size, j.off + (long long)j.k * j.k);
+        }
+    }
+    void products(GemmBatch& g, int accumulate, double alpha) {
+        if (!g.probs.empty()) return;
+        for (const NsJob& j : jobs) add_gram(g, j.k, j.off, j.k, 1, {GSeg{j.off, j.off, j.k, 0}}, accumulate, alpha);
+    }
+    // Returns whether this step was the last one needed.
+    bool make(const GramDev& d, double goal, const DBuf& G, DBuf& T, cudaStream_t st) {
+        const dim3 grid(gridn(mx, 256), (unsigned)jobs.size());
+        const double f = d.fro, f2 = f * f;
+        const bool square = 0.75 * f2 <= goal, cubic = 0.625 * f * f2 <= goal, quintic = 63.0 / 128.0 * f * f2 * f2 <= goal;
+        if (square || !quintic) {
+            k_ns_prep<<<grid, 256, 0, st>>>(dj.as<NsJob>(), G.as<double>(), T.as<double>());
+            PD_LAUNCHED();
+            return square;
+        }
+        E.ensure(size * 8, st);
+        k_ns_start<<<grid, 256, 0, st>>>(dj.as<NsJob>(), G.as<double>(), E.as<double>(), T.as<double>());
+        PD_LAUNCHED();
+        if (cubic) {
+            products(gT, 1, 0.375);
+            run_gemm64(gT, E.as<double>(), E.as<double>(), T.as<double>(), st);
+        } else {
+            products(gS, 0, 1.0);
+            products(gP, 1, 1.0);
+            S.ensure(size * 8, st);
+            run_gemm64(gS, E.as<double>(), E.as<double>(), S.as<double>(), st);
+            k_ns_quintic<<<grid, 256, 0, st>>>(dj.as<NsJob>(), S.as<double>(), E.as<double>());
+            PD_LAUNCHED();
+            run_gemm64(gP, S.as<double>(), E.as<double>(), T.as<double>(), st);
+        }
+        k_mirror<<<grid, 256, 0, st>>>(dj.as<NsJob>(), T.as<double>());
+        PD_LAUNCHED();
+        return true;
+    }
+};
 }  // namespace
 
 void orthonormalize_factor(const Sec& bl, const Sec& br, const std::vector<int>& qn, double* X, bool left,
@@ -414,11 +523,7 @@ void orthonormalize_factor(const Sec& bl, const Sec& br, const std::vector<int>&
     T.ensure(std::max<long long>(1, goff.back()) * 8, st);
     out.ensure(std::max<long long>(1, S.size) * 8, st);
     std::vector<NsJob> jobs;
-    int mx = 1;
-    for (int j = 0; j < mid.n(); ++j) {
-        jobs.push_back({goff[j], mid.m[j], 0});
-        mx = std::max(mx, mid.m[j] * mid.m[j]);
-    }
+    for (int j = 0; j < mid.n(); ++j) jobs.push_back({goff[j], mid.m[j], 0});
     upload(dj, jobs, st);
     GemmBatch gA;
     for (const auto& b : S.blk) {
@@ -447,21 +552,22 @@ void orthonormalize_factor(const Sec& bl, const Sec& br, const std::vector<int>&
             add_gram(gG[t], b.rows, goff[b.i], b.cols, 1, {GSeg{b.off, b.off, b.cols, 0}}, t > 0);
         }
     }
+    NsStep ns(dj, jobs);
     for (int iter = 0; iter < 6; ++iter) {
         PD_CK(cudaMemsetAsync(G.p, 0, std::max<long long>(1, goff.back()) * 8, st));
         for (auto& g1 : gG) run_gemm64(g1, X, X, G.as<double>(), st);
-        const double worst = gram_deviation(dj, jobs, G, dev, st);
+        const GramDev d = gram_deviation(dj, jobs, G, dev, st);
+        const double worst = d.max;
         PD_REQUIRE(std::isfinite(worst) && worst < 0.9, DMRG_ERR_NUMERIC,
                    "kept singular vectors too far from orthonormal for the FP64 re-orthonormalisation (|I - X^T X| = " +
                        std::to_string(worst) + " at iteration " + std::to_string(iter) + ")");
         if (worst < 1e-13 || iter == 5) break;
-        // X <- X (3I - G)/2 (left) or (3I - G)/2 X (right): one Newton-Schulz step
-        k_ns_prep<<<dim3(gridn(mx, 256), (unsigned)jobs.size()), 256, 0, st>>>(dj.as<NsJob>(), G.as<double>(),
-                                                                               T.as<double>());
-        PD_LAUNCHED();
+        // X <- X T (left) or T X (right)
+        const bool last = ns.make(d, 1e-13, G, T, st);
         if (left) run_gemm64(gA, T.as<double>(), X, out.as<double>(), st);
         else run_gemm64(gA, X, T.as<double>(), out.as<double>(), st);
         PD_CK(cudaMemcpyAsync(X, out.p, S.size * 8, cudaMemcpyDeviceToDevice, st));
+        if (last) break;
     }
     PD_CK(cudaStreamSynchronize(st));
 }
@@ -482,13 +588,13 @@ void convert_flat(const void* src, Num in, void* dst, Num out, long long n, cuda
 void orthonormalize_square(const std::vector<SvdSec>& ss, double* V, cudaStream_t st, int max_iter) {
     std::vector<NsJob> jobs;
     GemmBatch gG, gX;
-    long long tot = 0;
-    int mx = 1;
+    long long tot = 0, first = 0, sum = 0;
     for (const auto& x : ss) {
         if (x.n <= 0) continue;
         const int n = x.n;
+        if (jobs.empty()) first = x.v_off;
         jobs.push_back({x.v_off, n, 0});
-        mx = std::max(mx, n * n);
+        sum += (long long)n * n;
         // G = V^T V:  G(i, j) = sum_k V(k, i) V(k, j), V column-major (V(r, c) = V[off + r + c n])
         add_gram(gG, n, x.v_off, n, 1, {GSeg{x.v_off, x.v_off, n, 0}});
         // V' = V T:   V'(r, c) = sum_u V(r, u) T(u, c), T symmetric
@@ -496,24 +602,26 @@ void orthonormalize_square(const std::vector<SvdSec>& ss, double* V, cudaStream_
         tot = std::max(tot, x.v_off + (long long)n * n);
     }
     if (jobs.empty()) return;
+    PD_REQUIRE(sum == tot - first, DMRG_ERR_STATE, "sector matrices are not contiguous");
     DBuf G, T, out, dev, dj;
     G.ensure(tot * 8, st);
     T.ensure(tot * 8, st);
     out.ensure(tot * 8, st);
     upload(dj, jobs, st);
+    NsStep ns(dj, jobs);
     for (int iter = 0; iter < max_iter; ++iter) {
         run_gemm64(gG, V, V, G.as<double>(), st);
-        const double worst = gram_deviation(dj, jobs, G, dev, st);
+        const GramDev d = gram_deviation(dj, jobs, G, dev, st);
+        const double worst = d.max;
         PD_REQUIRE(std::isfinite(worst) && worst < 0.5, DMRG_ERR_NUMERIC,
                    "FP32 Jacobi rotations too far from orthogonal for the FP64 polish (|V^T V - I| = " +
                        std::to_string(worst) + " at iteration " + std::to_string(iter) + ")");
         if (worst < 1e-14) return;
-        k_ns_prep<<<dim3(gridn(mx, 256), (unsigned)jobs.size()), 256, 0, st>>>(dj.as<NsJob>(), G.as<double>(),
-                                                                               T.as<double>());
-        PD_LAUNCHED();
+        const bool last = ns.make(d, 1e-14, G, T, st);
         run_gemm64(gX, V, T.as<double>(), out.as<double>(), st);
-        for (const auto& j : jobs)
-            PD_CK(cudaMemcpyAsync(V + j.off, out.as<double>() + j.off, (size_t)j.k * j.k * 8, cudaMemcpyDeviceToDevice, st));
+        // the matrices follow each other without gaps
+        PD_CK(cudaMemcpyAsync(V + first, out.as<double>() + first, (size_t)(tot - first) * 8, cudaMemcpyDeviceToDevice, st));
+        if (last) return;
     }
     PD_REQUIRE(max_iter <= 8, DMRG_ERR_NUMERIC, "Newton-Schulz orthonormalisation did not converge");
 }
@@ -1401,7 +1509,7 @@ void fp64_precondition(const std::vector<SvdSec>& ss, const SvdSec* dsecs, DBuf&
 // Columns below about 1e-6 of the largest are not resolved by FP32 at all.  The first pass frees them
 // of the large columns (those angles are small) and leaves the angles among themselves, which a second
 // FP32 block Jacobi on these columns alone, scaled to order one, then makes small.
-// Whole splits: 512-state chain bond 96 -> 31 ms, accurate split at the 24x8 cylinder's m = 1000 bond
+// Whole splits, at this step: 512-state chain bond 96 -> 31 ms, accurate at the 24x8 cylinder's m = 1000 bond
 // 164 -> 52 ms, and closer to 64 bits than the scalar Jacobi's (2.8e-15 against 1.8e-14).
 // ------------------------------------------------------------------------------------------
 constexpr int kPolishPasses = 16;
