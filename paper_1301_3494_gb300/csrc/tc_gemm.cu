@@ -6,11 +6,19 @@
 // stored at C[c_off + m + n*ldc].  A and B are row slabs with a uniform leading dimension, rows
 // zero-padded to a multiple of 64 elements, so every k-block is a full 128-byte TMA box.
 //
-// Kernel: persistent, one CTA per SM, 6 warps:
+// Kernel: persistent, one CTA per SM, 18 warps:
 //   warp 0      TMA producer (one lane): 2D tiled loads, SWIZZLE_128B, S-stage mbarrier ring
 //   warp 1      TMEM owner + MMA issuer (one lane): tcgen05.mma 128 x BN x (32 bytes of K)
-//   warps 2..5  epilogue: tcgen05.ld 32x32b from the accumulator, coalesced stores along m
+//   warps 2..17 epilogue: tcgen05.ld 32x32b from the accumulator, coalesced stores along m; four warps
+//               a lane quarter, each a quarter of the columns
 // Two accumulators of BN columns each in TMEM, so the epilogue of tile i overlaps tile i+1.
+// Charge blocks make short tiles (four k-blocks of 64 on average at m = 2000, 0.6 us of MMA), so what
+// bounds a batch is what happens once a tile: with four epilogue warps, one per scheduler, a tile took
+// 5.7 us whatever its K, most of it single-warp issue latency over 128 columns of address arithmetic;
+// the rest was the chain tile -> problem -> segment of dependent loads and 64-bit divisions in the two
+// issuing lanes.  Hence the sixteen epilogue warps and TileFeed, which loads these records a tile ahead:
+// the three launches of an m = 2000 H_eff application took 51 + 135 + 72 us and take 24 + 50 + 67 (long K, the
+// last, is bound by the 128 bytes/ns an SM draws from L2 and by 206 tiles on 152 SMs).
 // Every mbarrier wait is bounded by %globaltimer; on expiry the kernel sets ERRBIT_TIMEOUT,
 // drains its own asynchronous work with bounded waits, frees TMEM and returns.
 #include <cuda.h>
@@ -30,7 +38,8 @@ namespace pd {
 namespace {
 
 constexpr int BM = TC_TILE_M;
-constexpr int THREADS = 192;
+constexpr int EPI_WARPS = 16;
+constexpr int THREADS = 64 + 32 * EPI_WARPS;
 constexpr uint64_t WAIT_NS = 2000000000ull;      // 2 s per wait before giving up
 constexpr uint64_t DRAIN_NS = 500000000ull;
 
@@ -123,6 +132,66 @@ __device__ __forceinline__ void tc_ld32(uint32_t taddr, uint32_t (&r)[32]) {
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
+__device__ __forceinline__ void tc_ld(uint32_t taddr, uint32_t (&r)[32]) { tc_ld32(taddr, r); }
+__device__ __forceinline__ void tc_ld(uint32_t taddr, uint32_t (&r)[16]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
+        "%15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr));
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+
+// A CTA's successive tiles with their problem and first segment.  Each record's address comes from the
+// one before it, three round trips to L2 a tile; they are loaded three, two and one tile ahead (indices
+// past the end repeat the last tile).
+template <bool SEGS>
+struct TileFeed {
+    const GTile* tiles;
+    const GProb* probs;
+    const GSeg* segs;
+    int last, step, t;
+    GTile tile, tile1, tile2;
+    GProb prob, prob1;
+    GSeg seg;
+    __device__ __forceinline__ TileFeed(const GTile* tiles_, const GProb* probs_, const GSeg* segs_, int ntiles)
+        : tiles(tiles_), probs(probs_), segs(segs_), last(ntiles - 1), step(gridDim.x), t(blockIdx.x) {
+        if (!more()) return;
+        tile = tiles[t];
+        tile1 = tiles[min(t + step, last)];
+        tile2 = tiles[min(t + 2 * step, last)];
+        prob = probs[tile.prob];
+        prob1 = probs[tile1.prob];
+        if (SEGS) seg = segs[prob.seg0];
+    }
+    __device__ __forceinline__ bool more() const { return t <= last; }
+    // the loads for the tiles to come, before this tile's work; next() after it
+    GTile tile3;
+    GProb prob2;
+    GSeg seg1;
+    __device__ __forceinline__ void ahead() {
+        tile3 = tiles[min(t + 3 * step, last)];
+        prob2 = probs[tile2.prob];
+        if (SEGS) seg1 = segs[prob1.seg0];
+    }
+    __device__ __forceinline__ void next() {
+        t += step;
+        tile = tile1;
+        tile1 = tile2;
+        tile2 = tile3;
+        prob = prob1;
+        prob1 = prob2;
+        if (SEGS) seg = seg1;
+    }
+};
+
+// a / d for a multiple or not of d, by the reciprocal magic = floor((2^64 - 1) / d) + 1: exact while
+// a d < 2^64 (a < 2^31 rows of d)
+__device__ __forceinline__ int row_of(long long a, unsigned long long magic) {
+    return (int)__umul64hi((unsigned long long)a, magic);
+}
+
 // Shared-memory matrix descriptor: K-major, 128-byte swizzle, 8-row atoms 1024 bytes apart.
 __device__ __forceinline__ uint64_t sdesc(uint32_t saddr) {
     uint64_t d = 0;
@@ -144,7 +213,8 @@ template <int KIND, int BN, int STAGES, class OutT>
 __global__ void __launch_bounds__(THREADS, 1)
     k_tc_gemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
               const GProb* __restrict__ probs, const GSeg* __restrict__ segs, const GTile* __restrict__ tiles,
-              int ntiles, int lda, int ldb, OutT* __restrict__ C, unsigned* __restrict__ err) {
+              int ntiles, unsigned long long lda_magic, unsigned long long ldb_magic, OutT* __restrict__ C,
+              unsigned* __restrict__ err) {
     constexpr int ESIZE = KIND == 0 ? 2 : 4;
     constexpr int BK = 128 / ESIZE;            // elements of K per stage (one 128-byte row)
     constexpr int A_BYTES = BM * 128;
@@ -171,7 +241,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         }
         for (int s = 0; s < 2; ++s) {
             mbar_init(smem_u32(&bar_tfull[s]), 1);
-            mbar_init(smem_u32(&bar_tempty[s]), 4);
+            mbar_init(smem_u32(&bar_tempty[s]), EPI_WARPS);
         }
         mbar_init(smem_u32(&bar_drain), 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -198,13 +268,15 @@ __global__ void __launch_bounds__(THREADS, 1)
             uint32_t issued_phase[STAGES];
             for (int s = 0; s < STAGES; ++s) issued[s] = 0, issued_phase[s] = 0;
             bool ok = true;
-            for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
-                const GTile tl = tiles[t];
-                const GProb p = probs[tl.prob];
-                for (int sgi = 0; sgi < p.nseg && ok; ++sgi) {
-                    const GSeg sg = segs[p.seg0 + sgi];
-                    const int ya = (int)(sg.a_off / lda) + tl.m0;
-                    const int yb = (int)(sg.b_off / ldb) + tl.n0;
+            TileFeed<true> feed(tiles, probs, segs, ntiles);
+            for (; feed.more() && ok; feed.next()) {
+                feed.ahead();
+                const int m0 = feed.tile.m0, n0 = feed.tile.n0, seg0 = feed.prob.seg0, nseg = feed.prob.nseg;
+                GSeg sg = feed.seg, sg1;
+                for (int sgi = 0; sgi < nseg && ok; ++sgi, sg = sg1) {
+                    sg1 = segs[seg0 + min(sgi + 1, nseg - 1)];
+                    const int ya = row_of(sg.a_off, lda_magic) + m0;
+                    const int yb = row_of(sg.b_off, ldb_magic) + n0;
                     const int nkb = (sg.K + BK - 1) / BK;
                     for (int kb = 0; kb < nkb; ++kb) {
                         if (!mbar_wait(smem_u32(&bar_empty[stage]), phase ^ 1u, &abort_flag, err)) { ok = false; break; }
@@ -233,16 +305,18 @@ __global__ void __launch_bounds__(THREADS, 1)
             int acc = 0;
             uint32_t acc_phase = 0;
             bool ok = true, any = false;
-            for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
-                const GTile tl = tiles[t];
-                const GProb p = probs[tl.prob];
+            TileFeed<true> feed(tiles, probs, segs, ntiles);
+            for (; feed.more() && ok; feed.next()) {
+                feed.ahead();
+                const int seg0 = feed.prob.seg0, nseg = feed.prob.nseg;
                 if (!mbar_wait(smem_u32(&bar_tempty[acc]), acc_phase ^ 1u, &abort_flag, err)) { ok = false; break; }
                 tc_fence_after();
                 const uint32_t dt = tmem + (uint32_t)(acc * BN);
                 uint32_t accumulate = 0;
-                for (int sgi = 0; sgi < p.nseg && ok; ++sgi) {
-                    const GSeg sg = segs[p.seg0 + sgi];
-                    const int nkb = (sg.K + BK - 1) / BK;
+                int K = feed.seg.K, K1;
+                for (int sgi = 0; sgi < nseg && ok; ++sgi, K = K1) {
+                    K1 = segs[seg0 + min(sgi + 1, nseg - 1)].K;
+                    const int nkb = (K + BK - 1) / BK;
                     for (int kb = 0; kb < nkb; ++kb) {
                         if (!mbar_wait(smem_u32(&bar_full[stage]), phase, &abort_flag, err)) { ok = false; break; }
                         tc_fence_after();
@@ -269,45 +343,45 @@ __global__ void __launch_bounds__(THREADS, 1)
             }
         }
     } else {
-        // ---------------- epilogue (warps 2..5) ----------------
-        const int quarter = warp & 3;
+        // ---------------- epilogue (warps 2..17) ----------------
+        constexpr int CW = BN / 4 < 32 ? BN / 4 : 32;          // columns a load
+        const int quarter = warp & 3, part = (warp - 2) >> 2;  // TMEM lanes, columns from part * BN / 4
         int acc = 0;
         uint32_t acc_phase = 0;
-        for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
-            const GTile tl = tiles[t];
-            const GProb p = probs[tl.prob];
+        TileFeed<false> feed(tiles, probs, segs, ntiles);
+        for (; feed.more(); feed.next()) {
+            feed.ahead();
             const bool ok = mbar_wait(smem_u32(&bar_tfull[acc]), acc_phase, &abort_flag, err);
             if (!__all_sync(0xffffffffu, ok)) break;
             tc_fence_after();
-            const int m = tl.m0 + quarter * 32 + lane;
+            const int m = feed.tile.m0 + quarter * 32 + lane, M = feed.prob.M, n0 = feed.tile.n0;
+            const int scn = feed.prob.scn, ncols = min(BN, feed.prob.N - n0);
             const uint32_t trow = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * BN);
-            const int ncols = min(BN, p.N - tl.n0);
             // FP32 arithmetic only (FP64 issue rate is low on this part); one conversion for FP64 output
-            const float alpha = (float)p.alpha;
-            const bool scale = alpha != 1.0f;
-            const bool accum = p.accumulate != 0;
-            OutT* crow = C + p.c_off + (long long)m * p.scm;
-            const int nlim = p.N - tl.n0;
-            for (int c0 = 0; c0 < ncols; c0 += 32) {
-                uint32_t r[32];
-                tc_ld32(trow + (uint32_t)c0, r);
-                if (m < p.M) {
+            const float alpha = (float)feed.prob.alpha;
+            const bool accum = feed.prob.accumulate != 0;
 #pragma unroll
-                    for (int j = 0; j < 32; ++j) {
-                        const int n = c0 + j;
-                        if (n < nlim) {
-                            OutT* dst = crow + (long long)(tl.n0 + n) * p.scn;
-                            float v = __uint_as_float(r[j]);
-                            if (scale) v *= alpha;
-                            if constexpr (std::is_same<OutT, double>::value) {
-                                *dst = accum ? *dst + (double)v : (double)v;
-                            } else {
-                                if (accum) v += (float)*dst;
-                                *dst = (OutT)v;
-                            }
+            for (int c0 = part * (BN / 4); c0 < (part + 1) * (BN / 4); c0 += CW) {
+                if (c0 >= ncols || feed.tile.m0 + quarter * 32 >= M) break;      // (uniform)
+                uint32_t r[CW];
+                tc_ld(trow + (uint32_t)c0, r);
+                if (m < M) {
+                    OutT* dst = C + feed.prob.c_off + m + (long long)(n0 + c0) * scn;
+                    const int lim = ncols - c0;
+                    if (lim >= CW && !accum) {
+#pragma unroll
+                        for (int j = 0; j < CW; ++j, dst += scn) *dst = (OutT)(__uint_as_float(r[j]) * alpha);
+                    } else {
+#pragma unroll
+                        for (int j = 0; j < CW; ++j, dst += scn) {
+                            if (j >= lim) break;
+                            const float v = __uint_as_float(r[j]) * alpha;
+                            if constexpr (std::is_same<OutT, double>::value) *dst = accum ? *dst + (double)v : (double)v;
+                            else *dst = (OutT)(accum ? v + (float)*dst : v);
                         }
                     }
                 }
+                __syncwarp();                                                    // (the next load is warp-wide)
             }
             tc_fence_before();
             __syncwarp();
@@ -382,7 +456,7 @@ void launch_tc(GemmBatch& g, const CUtensorMap& ma, const CUtensorMap& mb, int l
     int grid = std::min(g.ntiles, sm_share(sm_count()));
     void* tok = prof_on() ? prof_start(st) : nullptr;
     kern<<<grid, THREADS, SMEM, st>>>(ma, mb, g.dprobs.as<GProb>(), g.dsegs.as<GSeg>(), g.dtiles.as<GTile>(), g.ntiles,
-                                      lda, ldb, (OutT*)C, err);
+                                      ~0ull / (unsigned)lda + 1, ~0ull / (unsigned)ldb + 1, (OutT*)C, err);
     PD_LAUNCHED();
     if (tok) prof_stop(tok, st, g_prof_class, g.flops);
 }
