@@ -684,7 +684,7 @@ def rooflines(precision, fp64_emulation, prof, rates, pk, pk_kind):
             peak_note += ("; emulated GEMMs are counted in FP64-equivalent flops, so frac > 1 is a rate beyond "
                           "what the FP64 units can deliver")
         else:
-            gemm_kernel = "k_gemm_simt<double>: every FP64 grouped GEMM of the step"
+            gemm_kernel = "k_gemm_f64: every FP64 grouped GEMM of the step"
     else:
         gemm_kernel = "k_tc_gemm (matvec L and R stages)"
         g_ms, g_fl, g_n = prof["mv_gemm_ms"], prof["mv_gemm_flops"], prof["mv_gemm_launches"]

@@ -235,7 +235,8 @@ __global__ void __launch_bounds__(KS == 1 ? 128 : 32 * KS)
 // are zero up to a multiple of 16 in k (the tensor-core layout): they come in as float4 along k, one
 // chunk of 16 ahead in registers, and are stored k-major into a double buffer -- one barrier a chunk.
 // Each value is one chain of FMA in k order, as in the 4 x 4 kernel before: the same bits.
-// FP32 environment update at the 24x8 cylinder's m = 2000 bond, its two GEMMs: see launch_gemm_f32.
+// FP32 environment update at the 24x8 cylinder's m = 2000 bond, its two GEMMs (23 GFLOP): 1125 us with 4 x 4
+// values a thread, 603 now (38 TFLOP/s of the 78.5 measured; the rest is blocks' edges).
 // ------------------------------------------------------------------------------------------
 constexpr int F32_T = 64, F32_K = 16, F32_LD = F32_T + 4;
 __global__ void __launch_bounds__(64) k_gemm_f32(const GProb* __restrict__ probs, const GSeg* __restrict__ segs,
@@ -380,8 +381,9 @@ struct ElemWalk {
 };
 // Elements a thread has in flight in the block kernels.  They are bound by memory latency (a chunk is a
 // chain of list, job and data reads), so each thread issues its loads together; a chunk of 4096
-// elements is two such groups.  Packing the 24x8 cylinder's m = 2000 environments (2 x 138 MB), one
-// load at a time and a division an element before: see launch_copy.
+// elements is two such groups.  Packing for one bf16 H_eff application of the 24x8 cylinder's m = 2000 bond
+// (210 MB in all), with one load at a time and a division an element before: 162 -> 69 us; the mix of an
+// environment update 81 -> 59.
 constexpr int EW = 8;
 
 template <class Tin, class Tout>
