@@ -206,13 +206,14 @@ int dav_grid(long long n);
 // (k + 1) x (k + 1) part, yth[1..k+1] = its vector
 void launch_dav_gram(const double* V, const double* AV, long long n, int k, int kmax, double* G, double* partial,
                      unsigned* ctr, bool eig, double* yth, cudaStream_t st);
-// u = V y, Au = AV y, r = Au - theta u, norms = |r|^2, |u|^2
+// u = V y, Au = AV y, r = Au - theta u, norms = |r|^2, |u|^2; host (pinned) = |r|^2, |u|^2, theta
 void launch_dav_ritz(const double* V, const double* AV, long long n, int k, const double* yth, double* u, double* Au,
-                     double* r, double* partial, unsigned* ctr, double* norms, cudaStream_t st);
-// t = r / (theta - diag), twice orthogonalised against V's k rows (k >= 1); c1, c2: k words each
+                     double* r, double* partial, unsigned* ctr, double* norms, double* host, cudaStream_t st);
+// t = r / (theta - diag), twice orthogonalised against V's k rows (k >= 1); c1, c2: k words each; nrm2 and
+// host (pinned) = |t|^2
 void launch_dav_correct(const double* V, long long n, int k, const double* r, const double* diag, const double* theta,
                         double fl, double* t, double* c1, double* c2, double* partial, unsigned* ctr, double* nrm2,
-                        cudaStream_t st);
+                        double* host, cudaStream_t st);
 void launch_dav_norm(double* x, long long n, double* partial, unsigned* ctr, double* nrm2, cudaStream_t st);
 void launch_dav_unit(const double* x, const double* nrm2, double floor_, long long n, double* y, cudaStream_t st);
 void launch_finite_check(const double* x, long long n, unsigned* err, cudaStream_t st);

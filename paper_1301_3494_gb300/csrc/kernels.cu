@@ -843,12 +843,14 @@ __global__ void __launch_bounds__(DAV_THREADS) k_dav_gram(const double* __restri
     if (eig && threadIdx.x < 32) small_eig(G, k + 1, ldg, yth);
 }
 
-// u = V y, Au = AV y, r = Au - theta u; norms[0] = |r|^2, norms[1] = |u|^2.
+// u = V y, Au = AV y, r = Au - theta u; norms[0] = |r|^2, norms[1] = |u|^2; host[0..2] = |r|^2, |u|^2, theta
+// (pinned memory that the host reads after an event; as copies in the stream, three an iteration: 16-site
+// FP64 sweep at m = 64 96.3 ms, 89.7 this way; four bf16 regions at m = 128 83.7, 79.8).
 __global__ void __launch_bounds__(DAV_THREADS) k_dav_ritz(const double* __restrict__ V, const double* __restrict__ AV,
                                                           long long n, int k, const double* __restrict__ yth,
                                                           double* __restrict__ u, double* __restrict__ Au,
                                                           double* __restrict__ r, double* partial, unsigned* ctr,
-                                                          double* __restrict__ norms) {
+                                                          double* __restrict__ norms, double* __restrict__ host) {
     __shared__ double y[33];
     if (threadIdx.x <= k) y[threadIdx.x] = yth[threadIdx.x];
     __syncthreads();
@@ -872,8 +874,9 @@ __global__ void __launch_bounds__(DAV_THREADS) k_dav_ritz(const double* __restri
     if (!dav_last(ctr)) return;
     if (threadIdx.x < 64) {
         const double t = dav_row(partial, threadIdx.x >> 5);
-        if ((threadIdx.x & 31) == 0) norms[threadIdx.x >> 5] = t;
+        if ((threadIdx.x & 31) == 0) norms[threadIdx.x >> 5] = host[threadIdx.x >> 5] = t;
     }
+    if (threadIdx.x == 64) host[2] = y[0];
 }
 
 // Gram-Schmidt of the correction t against V_0 .. V_{k-1}, one pass per launch.  FIRST: t = r / (theta -
@@ -926,10 +929,11 @@ __global__ void __launch_bounds__(DAV_THREADS) k_dav_correct(const double* __res
     }
 }
 
-// t -= V c (k vectors; none: t is left), *nrm2 = |t|^2.
+// t -= V c (k vectors; none: t is left), *nrm2 = *host = |t|^2 (host: pinned memory or null).
 __global__ void __launch_bounds__(DAV_THREADS) k_dav_norm(const double* __restrict__ V, long long n, int k,
                                                           const double* __restrict__ c, double* t, double* partial,
-                                                          unsigned* ctr, double* __restrict__ nrm2) {
+                                                          unsigned* ctr, double* __restrict__ nrm2,
+                                                          double* __restrict__ host) {
     __shared__ double cs[32];
     if (threadIdx.x < k) cs[threadIdx.x] = c[threadIdx.x];
     __syncthreads();
@@ -946,7 +950,10 @@ __global__ void __launch_bounds__(DAV_THREADS) k_dav_norm(const double* __restri
     if (!dav_last(ctr)) return;
     if (threadIdx.x < 32) {
         const double v = dav_row(partial, 0);
-        if (threadIdx.x == 0) *nrm2 = v;
+        if (threadIdx.x == 0) {
+            *nrm2 = v;
+            if (host) *host = v;
+        }
     }
 }
 
@@ -1383,25 +1390,25 @@ void launch_dav_gram(const double* V, const double* AV, long long n, int k, int 
 }
 
 void launch_dav_ritz(const double* V, const double* AV, long long n, int k, const double* yth, double* u, double* Au,
-                     double* r, double* partial, unsigned* ctr, double* norms, cudaStream_t st) {
-    k_dav_ritz<<<dav_grid(n), DAV_THREADS, 0, st>>>(V, AV, n, k, yth, u, Au, r, partial, ctr, norms);
+                     double* r, double* partial, unsigned* ctr, double* norms, double* host, cudaStream_t st) {
+    k_dav_ritz<<<dav_grid(n), DAV_THREADS, 0, st>>>(V, AV, n, k, yth, u, Au, r, partial, ctr, norms, host);
     PD_LAUNCHED();
 }
 
 void launch_dav_correct(const double* V, long long n, int k, const double* r, const double* diag, const double* theta,
                         double fl, double* t, double* c1, double* c2, double* partial, unsigned* ctr, double* nrm2,
-                        cudaStream_t st) {
+                        double* host, cudaStream_t st) {
     k_dav_correct<true><<<dav_grid(n), DAV_THREADS, 0, st>>>(V, n, k, r, diag, theta, fl, nullptr, t, partial, ctr, c1);
     PD_LAUNCHED();
     k_dav_correct<false>
         <<<dav_grid(n), DAV_THREADS, 0, st>>>(V, n, k, nullptr, nullptr, nullptr, 0.0, c1, t, partial, ctr, c2);
     PD_LAUNCHED();
-    k_dav_norm<<<dav_grid(n), DAV_THREADS, 0, st>>>(V, n, k, c2, t, partial, ctr, nrm2);
+    k_dav_norm<<<dav_grid(n), DAV_THREADS, 0, st>>>(V, n, k, c2, t, partial, ctr, nrm2, host);
     PD_LAUNCHED();
 }
 
 void launch_dav_norm(double* x, long long n, double* partial, unsigned* ctr, double* nrm2, cudaStream_t st) {
-    k_dav_norm<<<dav_grid(n), DAV_THREADS, 0, st>>>(nullptr, n, 0, nullptr, x, partial, ctr, nrm2);
+    k_dav_norm<<<dav_grid(n), DAV_THREADS, 0, st>>>(nullptr, n, 0, nullptr, x, partial, ctr, nrm2, nullptr);
     PD_LAUNCHED();
 }
 

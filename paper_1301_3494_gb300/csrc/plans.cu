@@ -2271,19 +2271,22 @@ DavResult davidson(HeffPlan& P, const EnvSlab& L, const EnvSlab& R, double* x, i
     double* part = dpart.as<double>();
     double* nrm = dnrm.as<double>();
     unsigned* ctr = dctr.as<unsigned>();
-    double* hn = reinterpret_cast<double*>(sweep_flags_host(64));   // pinned: |r|^2, |u|^2, |t|^2, theta
+    // pinned, written by kernels: |r|^2, |u|^2, theta, |t|^2
+    double* hn = reinterpret_cast<double*>(sweep_flags_host(64));
     constexpr double kFloor = 1e-14;            // a correction this small is rounding
     struct Events {
+        cudaStream_t st;
         cudaEvent_t e[4] = {};
-        Events() {
+        explicit Events(cudaStream_t st_) : st(st_) {
             for (int i = 0; i < 4; ++i)
                 PD_CK(i < 2 ? cudaEventCreate(&e[i]) : cudaEventCreateWithFlags(&e[i], cudaEventDisableTiming));
         }
         ~Events() {
+            cudaStreamSynchronize(st);           // no kernel writes to hn once this call has left, by throw or return
             for (auto x : e)
                 if (x) cudaEventDestroy(x);
         }
-    } ev;
+    } ev(st);
     HeffPlan* cur = &P;
     // matvec timed by a pair of events, which is read at the next wait (the stream does not stop for it)
     auto mv = [&](const double* in, double* out) {
@@ -2317,9 +2320,7 @@ DavResult davidson(HeffPlan& P, const EnvSlab& L, const EnvSlab& R, double* x, i
             res.iters++;
             launch_dav_gram(V, AV, n, k - 1, kmax, G, part, ctr, true, dyth.as<double>(), st);
             launch_dav_ritz(V, AV, n, k, dyth.as<double>(), du.as<double>(), dAu.as<double>(), dr.as<double>(), part, ctr,
-                            nrm, st);
-            PD_CK(cudaMemcpyAsync(hn, nrm, 16, cudaMemcpyDeviceToHost, st));
-            PD_CK(cudaMemcpyAsync(hn + 3, dyth.p, 8, cudaMemcpyDeviceToHost, st));
+                            nrm, hn, st);
             PD_CK(cudaEventRecord(ev.e[2], st));
             if (it < iters) {
                 if (k >= kmax) {   // restart from the Ritz vector
@@ -2329,21 +2330,20 @@ DavResult davidson(HeffPlan& P, const EnvSlab& L, const EnvSlab& R, double* x, i
                     launch_dav_gram(V, AV, n, 0, kmax, G, part, ctr, false, nullptr, st);
                 }
                 launch_dav_correct(V, n, k, dr.as<double>(), ddg.as<double>(), dyth.as<double>(), 1e-4, dt.as<double>(),
-                                   dc.as<double>(), dc.as<double>() + kmax, part, ctr, nrm + 2, st);
+                                   dc.as<double>(), dc.as<double>() + kmax, part, ctr, nrm + 2, hn + 3, st);
                 launch_dav_unit(dt.as<double>(), nrm + 2, kFloor, n, V + (size_t)k * n, st);
-                PD_CK(cudaMemcpyAsync(hn + 2, nrm + 2, 8, cudaMemcpyDeviceToHost, st));
                 PD_CK(cudaEventRecord(ev.e[3], st));
             }
             mv_done();
             PD_CK(cudaEventSynchronize(ev.e[2]));
-            res.theta = hn[3];
+            res.theta = hn[2];
             res.rnorm = std::sqrt(std::max(0.0, hn[0]));
             PD_REQUIRE(std::isfinite(res.theta) && std::isfinite(res.rnorm), DMRG_ERR_NUMERIC,
                        "non-finite Ritz value in Davidson");
             if (res.rnorm <= tol * std::max(1.0, std::fabs(res.theta)) || it == iters) break;
             mv(V + (size_t)k * n, AV + (size_t)k * n);
             PD_CK(cudaEventSynchronize(ev.e[3]));
-            if (std::sqrt(hn[2]) < kFloor) break;
+            if (std::sqrt(hn[3]) < kFloor) break;
             ++k;
         }
         // x = u / |u|
