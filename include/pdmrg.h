@@ -101,8 +101,11 @@ typedef struct {
                                environment updates, wavefunction formation, gauge moves, local
                                measurements) run FP64-accurate on the bf16 tensor cores
                                (dmrg_gemm64 mode 1); batches outside its K limit, and those too
-                               small to gain from it (below about 1 GFLOP), stay on the FP64
-                               units.  0 = FP64 units throughout.                               */
+                               small to gain from it, stay on the FP64 units: below 1 GFLOP
+                               where a plan is run many times (a Davidson's matvec, the
+                               measurements of one state), below 6 GFLOP elsewhere.  2 = every
+                               batch inside the K limit, whatever its size.  0 = FP64 units
+                               throughout.                                                      */
     int svd_plain_jacobi;   /* 1 = every split's one-sided Jacobi runs on the sector matrix W
                                itself; 0 (default) = on R^T from a Householder QR W = QR (a
                                few sweeps instead of many; sectors taller than the QR panel's
@@ -334,6 +337,7 @@ typedef struct {
                                     R-SVD with U and V, 4 p n^2 + 22 n^3 per p x n sector         */
     double svd_block_alg_bytes;  /* FP32 splits: the sector matrices read once, U and V written
                                     once (FP32), 4 (2 p n + n^2) per sector                      */
+    long long emu_batches;       /* FP64 GEMM batches run emulated on the bf16 tensor cores       */
 } dmrg_profile;
 
 void dmrg_profile_enable(int on);

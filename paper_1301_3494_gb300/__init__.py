@@ -45,7 +45,7 @@ class Profile(C.Structure):
                 ("svd_fp64_fallbacks", C.c_longlong), ("svd_block_flops", C.c_double),
                 ("svd_rot_hist", C.c_longlong * 48), ("emu_fallbacks", C.c_longlong), ("tune_classes", C.c_longlong),
                 ("tune_changed", C.c_longlong), ("svd_bonds", C.c_longlong), ("svd_block_alg_flops", C.c_double),
-                ("svd_block_alg_bytes", C.c_double)]
+                ("svd_block_alg_bytes", C.c_double), ("emu_batches", C.c_longlong)]
 
     def as_dict(self):
         d = {k: getattr(self, k) for k, _ in self._fields_}
@@ -324,7 +324,8 @@ class Engine:
         self._wshapes = [(int(D_[j]), len(q_), len(q_), int(D_[j + 1])) for j in range(self.L)]
         desc = MpoDesc(self.L, len(q_), _ptr(q_, _ip), _ptr(D_, _ip), _ptr(f_, _ip), _ptr(W_, _dp), int(qtot))
         prec = PRECISIONS[precision] if isinstance(precision, str) else int(precision)
-        cfg = Config(prec, int(kmax), C.c_void_p(stream), int(bool(svd_fp64)), int(bool(fp64_emulation)),
+        cfg = Config(prec, int(kmax), C.c_void_p(stream), int(bool(svd_fp64)),
+                     2 if fp64_emulation == 2 else int(bool(fp64_emulation)),
                      int(bool(svd_plain_jacobi)), int(bool(env_fp64)), int(accurate_edges))
         h = C.c_void_p()
         _check(lib().dmrg_init_mpo(C.byref(h), C.byref(desc), C.byref(cfg)))

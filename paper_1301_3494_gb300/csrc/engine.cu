@@ -102,7 +102,7 @@ struct dmrg_ctx {
     std::vector<std::unique_ptr<TwoSiteMPO>> w12;   // per bond (j, j+1), lazily built
     int prec = DMRG_FP64, kmax = 8;
     bool svd_fp64 = false;       // mixed modes: FP64 splits on ordinary bonds too
-    bool emu = false;            // FP64 grouped GEMMs on the bf16 tensor cores (ozaki.cu)
+    int emu = 0;                 // FP64 grouped GEMMs on the bf16 tensor cores (g_gemm64_emu)
     bool svd_plain = false;      // splits by the plain Jacobi on W (no QR preconditioning)
     bool env64 = false;          // mixed modes: FP64-accurate environments (PREC_ENV64)
     int acc_edges = 0;           // mixed modes: FP64 solves next to region boundaries (2: FP64 splits there too)
@@ -814,7 +814,7 @@ StepStats region_sweep(dmrg_ctx* c, const dmrg_sweep_params* p) {
 struct EmuGuard {
     int saved, saved_qr;
     explicit EmuGuard(const dmrg_ctx* c) : saved(g_gemm64_emu), saved_qr(g_svd_qr) {
-        g_gemm64_emu = (c && c->emu) ? 1 : 0;
+        g_gemm64_emu = c ? c->emu : 0;
         g_svd_qr = (c && c->svd_plain) ? 0 : 1;
     }
     ~EmuGuard() {
@@ -857,7 +857,7 @@ dmrg_status dmrg_init_mpo(dmrg_ctx** out, const dmrg_mpo_desc* mpo, const dmrg_c
     C->prec = cfg->precision;
     C->kmax = cfg->kmax > 0 ? cfg->kmax : 8;
     C->svd_fp64 = cfg->svd_fp64 != 0;
-    C->emu = cfg->fp64_emulation != 0;
+    C->emu = cfg->fp64_emulation == 2 ? 2 : (cfg->fp64_emulation != 0 ? 1 : 0);
     C->svd_plain = cfg->svd_plain_jacobi != 0;
     C->env64 = cfg->env_fp64 != 0;
     C->acc_edges = std::max(0, std::min(2, cfg->accurate_edges));

@@ -337,6 +337,7 @@ static std::unique_ptr<MeasPlan> make_meas_plan(const ICMPS& ic, const std::vect
     if (with2) {
         M->P.ensure(std::max<long long>(1, M->p_size) * 8, st);
         M->Th.ensure(std::max<long long>(1, M->th_size) * 8, st);
+        M->theta.repeated = true;
         M->theta.upload_f64(st);
     }
     return M;

@@ -70,6 +70,7 @@ void prof_svd(int sweeps, double ms, int kind, int max_rows, double flops, const
 void prof_fallback();
 // An emulated FP64 GEMM batch sent to the FP64 units by its scale guard (counted always).
 void prof_emu_fallback();
+void prof_emu_batch();
 
 // Persistent and cooperative grids are sized to the SMs of the device; while R regions run
 // concurrently (one host thread each), each thread caps its grids at sms / R so that the regions

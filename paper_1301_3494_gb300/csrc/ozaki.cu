@@ -541,6 +541,7 @@ bool run_gemm64_emu(GemmBatch& g, const double* A, const double* B, double* C, c
     PD_LAUNCHED();
     if (tok) prof_stop(tok, st, cls, g.flops);
     check_err_word(P.err.as<unsigned>(), st);
+    prof_emu_batch();
     return true;
 }
 

@@ -163,18 +163,19 @@ void GemmBatch::stage_f64(ListPack& pk) {
     stage(pk, f64.tile, f64.tile);
 }
 
-// Whether a batch gains from the emulation.  Its plan is built on the host (one to several ms for the
-// batches of a bond) and a run is seven launches and two host waits around the slice products, so it
-// only pays for large batches, or from its third use on for middling ones.  Measured, FP64 units
-// against a first emulated run / a repeated one:
+// Whether a batch runs emulated.  Its plan is built on the host (one to several ms for the batches of a
+// bond) and a run is seven launches and two host waits around the slice products, so it only pays for
+// large batches, or for middling ones whose plan is run many times.  Size and that hint (a Davidson's
+// matvec, a kept measurement plan) decide, never the history of a batch: the two arithmetics round
+// differently, and one operator must not change between its applications.  Measured, FP64 units against
+// a first emulated run / a repeated one:
 //   17 of 320 x 320 x 640 (2.2 GFLOP)        2.1 ms,  2.0 / 1.0 ms
 //   68 of 80 x 80, 20 x K = 80 (1.4 GFLOP)   1.5 ms,  4.5 / 1.3 ms
 //   68 of 150 x 150, 26 x K = 150 (12)       10 ms,   13 / 5.0 ms
 //   2000^3 (16)                              13 ms,   4.3 / 1.8 ms
 //   34 of 80 x 80 x 80 (0.035)               0.05 ms, 0.5 / 0.2 ms
-static bool worth_emulating(GemmBatch& g) {
-    const int use = g.uses++;
-    return g.flops >= 6e9 || (g.flops >= 1e9 && use >= 2);
+static bool emulated(const GemmBatch& g) {
+    return g_gemm64_emu == 2 || (g_gemm64_emu && g.flops >= (g.repeated ? 1e9 : 6e9));
 }
 
 F64Shape GemmBatch::upload_f64(cudaStream_t st) {
@@ -185,7 +186,7 @@ F64Shape GemmBatch::upload_f64(cudaStream_t st) {
 
 void run_gemm64(GemmBatch& g, const double* A, const double* B, double* C, cudaStream_t st) {
     if (g.empty()) return;
-    if (g_gemm64_emu && worth_emulating(g) && run_gemm64_emu(g, A, B, C, st)) return;
+    if (emulated(g) && run_gemm64_emu(g, A, B, C, st)) return;
     const F64Shape shape = g.upload_f64(st);
     void* tok = prof_on() ? prof_start(st) : nullptr;
     launch_gemm_f64(g.dprobs.as<GProb>(), g.dsegs.as<GSeg>(), g.dtiles.as<GTile>(), g.ntiles, shape.tile, shape, A, B, C,
@@ -823,6 +824,7 @@ std::unique_ptr<HeffPlan> make_heff_plan(const Sec& bl, const Sec& br, const std
         P->diag_chunks = (int)c.size();
         pk.add(P->ddc, c);
         auto stage = [&](GemmBatch& g, Num cnum) {
+            g.repeated = true;
             if (prec == DMRG_FP64) g.stage_f64(pk);
             else if (prec == PREC_F32) g.stage(pk, 64, 64);
             else {

@@ -182,7 +182,8 @@ inline Num env_num(int prec) { return (prec == DMRG_FP64 || prec == PREC_ENV64) 
 // Grouped GEMM batch (host list -> device arrays -> FP64 SIMT or tcgen05 launch)
 // ------------------------------------------------------------------------------------------
 struct EmuPlan;
-// FP64 GEMMs through the bf16 tensor cores (ozaki.cu) when set on the calling thread.
+// FP64 GEMMs through the bf16 tensor cores (ozaki.cu) when set on the calling thread: 1 where they gain
+// from it, 2 wherever the emulation can run them.
 extern thread_local int g_gemm64_emu;
 struct GemmBatch {
     std::vector<GProb> probs;
@@ -193,7 +194,7 @@ struct GemmBatch {
     int ntiles = 0;
     int tile_m = 0, tile_n = 0;         // shape of the uploaded tile list
     F64Shape f64{0, 0};                 // FP64 tile shape (0: not chosen yet)
-    int uses = 0;                       // runs so far with FP64 emulation on
+    bool repeated = false;              // run many times with one plan (see run_gemm64)
     int bn_choice = 0;                  // tensor-core tile width chosen for this batch (0: not yet)
     long long a_rows = 0, b_rows = 0;   // slab extents (tensor-core path)
     int lda = 0, ldb = 0;
