@@ -256,6 +256,9 @@ void launch_bjacobi(const SvdSec* secs, const BjSec* bsecs, const int* task_sec,
                     int max_sweeps, float* W, float* V, float noise_c, float* gmax, int* bmod, int* pchk, int* border,
                     int nblk, int* rot, int* sweeps, unsigned* err, unsigned long long* flops, const int2* items,
                     int per_sweep, int nsec, int nact, int* qstate, cudaStream_t st);
+// sig[s_off + i] = norm of column i of sector s; and the columns' order by decreasing norm.
+template <class T>
+void launch_svd_norms(const SvdSec* secs, int nsec, int max_n, const T* W, double* sig, cudaStream_t st);
 template <class T>
 void launch_svd_finish(const SvdSec* secs, int nsec, int max_n, const T* W, double* sig, int* order, cudaStream_t st);
 

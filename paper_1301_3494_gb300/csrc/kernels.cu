@@ -1501,12 +1501,18 @@ template void launch_jacobi<float>(const SvdSec*, int, const int*, int, int, int
                                    double*, int*, int*, unsigned*, unsigned*, cudaStream_t);
 
 template <class T>
+void launch_svd_norms(const SvdSec* secs, int nsec, int max_n, const T* W, double* sig, cudaStream_t st) {
+    if (nsec <= 0 || max_n <= 0) return;
+    k_svd_norms<T><<<dim3((max_n + 7) / 8, nsec), 256, 0, st>>>(secs, W, sig);
+    PD_LAUNCHED();
+}
+template void launch_svd_norms<double>(const SvdSec*, int, int, const double*, double*, cudaStream_t);
+
+template <class T>
 void launch_svd_finish(const SvdSec* secs, int nsec, int max_n, const T* W, double* sig, int* order, cudaStream_t st) {
     if (nsec <= 0 || max_n <= 0) return;
-    const dim3 grid((max_n + 7) / 8, nsec);
-    k_svd_norms<T><<<grid, 256, 0, st>>>(secs, W, sig);
-    PD_LAUNCHED();
-    k_svd_order<<<grid, 256, 0, st>>>(secs, sig, order);
+    launch_svd_norms<T>(secs, nsec, max_n, W, sig, st);
+    k_svd_order<<<dim3((max_n + 7) / 8, nsec), 256, 0, st>>>(secs, sig, order);
     PD_LAUNCHED();
 }
 template void launch_svd_finish<double>(const SvdSec*, int, int, const double*, double*, int*, cudaStream_t);

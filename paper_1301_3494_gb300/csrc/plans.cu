@@ -1511,10 +1511,18 @@ void fp64_precondition(const std::vector<SvdSec>& ss, const SvdSec* dsecs, DBuf&
 // Columns below about 1e-6 of the largest are not resolved by FP32 at all.  The first pass frees them
 // of the large columns (those angles are small) and leaves the angles among themselves, which a second
 // FP32 block Jacobi on these columns alone, scaled to order one, then makes small.
+// Columns below kNull of the sector's largest are finished: W V was formed in FP64, so a column that is
+// not zero in exact arithmetic does not come out below rounding, 1e-16 of the largest, and one that is (an
+// exactly low-rank matrix: its columns are multiples of each other, bit for bit) falls by that factor in
+// every pass without ever being orthogonal to its like.  Splits drop such values at 1e-12, gauge moves
+// absorb the columns unnormalised.  Without the floor an all-ones 200 x 200 matrix took 95 ms (four passes
+// and 60 sweeps of the scalar Jacobi, which has the same floor now), 21 by the scalar Jacobi alone, 1.8 with
+// it; integers of rank 3, 200 x 200: 252, 244 and 12 ms.
 // Whole splits, at this step: 512-state chain bond 96 -> 31 ms, accurate at the 24x8 cylinder's m = 1000 bond
 // 164 -> 52 ms, and closer to 64 bits than the scalar Jacobi's (2.8e-15 against 1.8e-14).
 // ------------------------------------------------------------------------------------------
 constexpr int kPolishPasses = 16;
+constexpr double kNull = 0x1p-80;             // 8e-25, in column norms
 
 // One CTA per column j of a sector: E(:, j) from the lower triangle of G (rows i >= 64 (j / 64)),
 // rotations by at most tan = 0.6, and none between two columns at or after cut[sector].  stat, four
@@ -1525,7 +1533,7 @@ struct PolCol {
 };
 __global__ void k_polish_angles(const SvdSec* __restrict__ secs, const PolCol* __restrict__ cols,
                                 const double* __restrict__ G, double* __restrict__ E, const int* __restrict__ cut,
-                                double* __restrict__ diag, unsigned* __restrict__ stat) {
+                                unsigned* __restrict__ stat) {
     const PolCol pc = cols[blockIdx.x];
     const SvdSec s = secs[pc.sec];
     const int j = pc.j, n = s.n;
@@ -1534,6 +1542,14 @@ __global__ void k_polish_angles(const SvdSec* __restrict__ secs, const PolCol* _
     const double gjj = Gs[j + (long long)j * n];
     const double tol = 4.0 * DBL_EPSILON * sqrt((double)s.p);
     const int from = cut[pc.sec];
+    // squared norms are not negative: they order like their bits (NaN above all, and no floor then)
+    __shared__ long long tops[4];
+    long long top = 0;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) top = max(top, __double_as_longlong(Gs[i + (long long)i * n]));
+    for (int o = 16; o > 0; o >>= 1) top = max(top, __shfl_xor_sync(0xffffffffu, top, o));
+    if ((threadIdx.x & 31) == 0) tops[threadIdx.x >> 5] = top;
+    __syncthreads();
+    const double null2 = kNull * kNull * __longlong_as_double(max(max(tops[0], tops[1]), max(tops[2], tops[3])));
     float sum = 0.f;
     int above = 0, first = n;
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
@@ -1541,7 +1557,7 @@ __global__ void k_polish_angles(const SvdSec* __restrict__ secs, const PolCol* _
         const double g = Gs[hi + (long long)lo * n], gii = Gs[i + (long long)i * n];
         double t = 0.0;
         const double size = sqrt(gii * gjj);
-        if (i != j && fabs(g) > 0.1 * tol * size) {
+        if (i != j && fabs(g) > 0.1 * tol * size && !(fmin(gii, gjj) <= null2)) {
             above |= fabs(g) > tol * size;
             const double zeta = (gjj - gii) / (2.0 * g);
             t = 1.0 / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
@@ -1552,7 +1568,6 @@ __global__ void k_polish_angles(const SvdSec* __restrict__ secs, const PolCol* _
         }
         Ej[i] = t;
     }
-    if (threadIdx.x == 0) diag[s.s_off + j] = gjj;
     for (int o = 16; o > 0; o >>= 1) {
         sum += __shfl_xor_sync(0xffffffffu, sum, o);
         first = min(first, __shfl_xor_sync(0xffffffffu, first, o));
@@ -1594,20 +1609,22 @@ bool polish64(const std::vector<SvdSec>& ss, const SvdSec* dsecs, DBuf& dW, DBuf
     }
     *passes = 0;
     if (cols.empty()) return true;
-    DBuf dcols, G, E, X, Wn, Vn, diag, stat;
+    DBuf dcols, G, E, X, Wn, Vn, norms, stat;
     upload(dcols, cols, st);
     G.ensure(voff * 8, st);
     E.ensure(voff * 8, st);
     X.ensure(voff * 8, st);
     Wn.ensure(woff * 8, st);
     Vn.ensure(voff * 8, st);
-    diag.ensure(soff * 8, st);
+    norms.ensure(soff * 8, st);
     stat.ensure((size_t)nsec * 16, st);
     std::vector<unsigned> hs((size_t)nsec * 4);
     std::vector<double> hd(soff);
     const unsigned nc = (unsigned)cols.size();
     std::vector<int> cut(nsec);
     DBuf dcut;
+    int maxn = 1;
+    for (const SvdSec& x : ss) maxn = std::max(maxn, x.n);
     int large = 0;                        // passes in a row with large angles
     int stages = 3;                       // FP32 passes over unresolved columns still allowed
     for (int pass = 0; pass < kPolishPasses; ++pass) {
@@ -1616,10 +1633,9 @@ bool polish64(const std::vector<SvdSec>& ss, const SvdSec* dsecs, DBuf& dW, DBuf
             upload(dcut, cut, st);
             PD_CK(cudaMemsetAsync(stat.p, 0, (size_t)nsec * 16, st));
             k_polish_angles<<<nc, 128, 0, st>>>(dsecs, dcols.as<PolCol>(), G.as<double>(), E.as<double>(),
-                                                dcut.as<int>(), diag.as<double>(), stat.as<unsigned>());
+                                                dcut.as<int>(), stat.as<unsigned>());
             PD_LAUNCHED();
             PD_CK(cudaMemcpyAsync(hs.data(), stat.p, (size_t)nsec * 16, cudaMemcpyDeviceToHost, st));
-            PD_CK(cudaMemcpyAsync(hd.data(), diag.p, (size_t)soff * 8, cudaMemcpyDeviceToHost, st));
             PD_CK(cudaStreamSynchronize(st));
         };
         for (int s = 0; s < nsec; ++s) cut[s] = ss[s].n;
@@ -1675,6 +1691,9 @@ bool polish64(const std::vector<SvdSec>& ss, const SvdSec* dsecs, DBuf& dW, DBuf
         // rotations against the resolved columns have become small
         if (!unresolved || norm > 0.05f) continue;
         --stages;
+        launch_svd_norms<double>(dsecs, nsec, maxn, dW.as<double>(), norms.as<double>(), st);
+        PD_CK(cudaMemcpyAsync(hd.data(), norms.p, (size_t)soff * 8, cudaMemcpyDeviceToHost, st));
+        PD_CK(cudaStreamSynchronize(st));
         std::vector<SvdSec> sub;
         CopyList down;
         GemmBatch gw, gv;
@@ -1694,7 +1713,7 @@ bool polish64(const std::vector<SvdSec>& ss, const SvdSec* dsecs, DBuf& dW, DBuf
             CopyJob j{};
             j.src = x.w_off + (long long)cut[s] * x.p; j.dst = wo; j.rows = y.n; j.cols = x.p;
             j.srs = x.p; j.scs = 1; j.drs = x.p; j.dcs = 1; j.zero_to = 0;
-            j.scale = top > 0.0 ? std::ldexp(1.0, -std::ilogb(std::sqrt(top))) : 1.0;
+            j.scale = top > 0.0 && std::isfinite(top) ? std::ldexp(1.0, -std::max(-1000, std::ilogb(top))) : 1.0;
             down.add(j);
             const long long wc = x.w_off + (long long)cut[s] * x.p, vc = x.v_off + (long long)cut[s] * x.n;
             gw.add(x.p, y.n, wc, 1, x.p, y.n, 1, 1, x.p, {GSeg{wc, vo, y.n, 0}});
@@ -1706,7 +1725,8 @@ bool polish64(const std::vector<SvdSec>& ss, const SvdSec* dsecs, DBuf& dW, DBuf
             sub.push_back(y);
         }
         const int max_sweeps = 60;
-        DBuf w32, v32, v64, rot32, fl, dsub;
+        DBuf w64, w32, v32, v64, rot32, fl, dsub;
+        w64.ensure(wo * 8, st);
         w32.ensure(wo * 4, st);
         v32.ensure(vo * 4, st);
         v64.ensure(vo * 8, st);
@@ -1715,7 +1735,9 @@ bool polish64(const std::vector<SvdSec>& ss, const SvdSec* dsecs, DBuf& dW, DBuf
         upload(dsub, sub, st);
         down.up(st);
         PD_CK(cudaMemsetAsync(rot32.p, 0, (max_sweeps + 1) * 4, st));
-        run_copy<double>(down, dW.as<double>(), w32.p, Num::F32, st);
+        // scaled before the conversion: the columns may lie below what FP32 can hold
+        run_copy<double>(down, dW.as<double>(), w64.p, Num::F64, st);
+        convert_flat(w64.p, Num::F64, w32.p, Num::F32, wo, st);
         launch_svd_init_v<float>(dsub.as<SvdSec>(), (int)sub.size(), mn, v32.as<float>(), st);
         block_jacobi32(sub, dsub.as<SvdSec>(), w32.as<float>(), v32.as<float>(), mp, max_sweeps, rot32.as<int>(), err,
                        fl.as<unsigned long long>(), st, 0.0f);
@@ -1729,6 +1751,25 @@ bool polish64(const std::vector<SvdSec>& ss, const SvdSec* dsecs, DBuf& dW, DBuf
         std::swap(dV, Vn);
     }
     return false;
+}
+
+// The FP64 one-sided Jacobi of W from V on (after fp64_precondition, or from the identity in the plain mode):
+// the polish where it settles, else the scalar sweeps.  rot: max_sweeps + 1 zeroed ints, the last of which
+// gets the passes or sweeps taken; pairs: the sectors' column pairs.
+void jacobi64_finish(const std::vector<SvdSec>& ss, const SvdSec* dsecs, const DBuf& pairs, int npairs, int maxnpad,
+                     int max_sweeps, DBuf& dW, DBuf& dV, long long woff, long long voff, long long soff, int* rot,
+                     unsigned* bar, unsigned* err, cudaStream_t st) {
+    const bool polish = g_svd_qr && woff > 0;
+    int passes = 0;
+    if (polish && polish64(ss, dsecs, dW, dV, woff, voff, soff, err, &passes, st)) {
+        PD_CK(cudaMemcpyAsync(rot + max_sweeps, &passes, sizeof(int), cudaMemcpyHostToDevice, st));
+        return;
+    }
+    DBuf floor2;
+    if (polish) floor2.ensure(std::max<size_t>(1, ss.size()) * 8, st);
+    launch_jacobi<double>(dsecs, (int)ss.size(), pairs.as<int>(), npairs, maxnpad, max_sweeps, dW.as<double>(),
+                          dV.as<double>(), 4.0 * DBL_EPSILON, polish ? kNull : 0.0, floor2.as<double>(), rot,
+                          rot + max_sweeps, bar, err, st);
 }
 
 void jacobi64(std::vector<SvdSec>& ss, DBuf& dWbuf, DBuf& dsecs, DBuf& dV, DBuf& dsig, DBuf& dord, cudaStream_t st) {
@@ -1766,12 +1807,8 @@ void jacobi64(std::vector<SvdSec>& ss, DBuf& dWbuf, DBuf& dsecs, DBuf& dV, DBuf&
         fp64_precondition(ss, dsecs.as<SvdSec>(), dWbuf, dV.as<double>(), woff, voff, maxp, maxn, bar + 3, st);
     else
         launch_svd_init_v<double>(dsecs.as<SvdSec>(), nsec, maxn, dV.as<double>(), st);
-    int passes = 0;
-    if (!(g_svd_qr && woff > 0 &&
-          polish64(ss, dsecs.as<SvdSec>(), dWbuf, dV, woff, voff, soff, bar + 3, &passes, st)))
-        launch_jacobi<double>(dsecs.as<SvdSec>(), nsec, dpairs.as<int>(), (int)pair_sec.size(), maxnpad, max_sweeps,
-                              dWbuf.as<double>(), dV.as<double>(), 4.0 * DBL_EPSILON, 0.0, nullptr, drot.as<int>(),
-                              drot.as<int>() + max_sweeps, bar, bar + 3, st);
+    jacobi64_finish(ss, dsecs.as<SvdSec>(), dpairs, (int)pair_sec.size(), maxnpad, max_sweeps, dWbuf, dV, woff, voff, soff,
+                    drot.as<int>(), bar, bar + 3, st);
     double* W = dWbuf.as<double>();
     launch_svd_finish<double>(dsecs.as<SvdSec>(), nsec, maxn, W, dsig.as<double>(), dord.as<int>(), st);
     unsigned err = 0;
@@ -2056,19 +2093,12 @@ std::vector<SplitResult> svd_split_batch(const std::vector<SplitReq>& reqs, bool
             dM.ensure(woff * 8, st);
             PD_CK(cudaMemcpyAsync(dM.p, dW.p, woff * 8, cudaMemcpyDeviceToDevice, st));
         }
-        const double tol = 4.0 * DBL_EPSILON;   // per sector: times sqrt(p)
         if (g_svd_qr && woff > 0)
             fp64_precondition(ss, dsecs.as<SvdSec>(), dW, dV.as<double>(), woff, voff, maxp, maxn, jerr, st);
         else
             launch_svd_init_v<double>(dsecs.as<SvdSec>(), nsec, maxn, dV.as<double>(), st);
-        int passes = 0;
-        if (g_svd_qr && woff > 0 &&
-            polish64(ss, dsecs.as<SvdSec>(), dW, dV, woff, voff, soff, jerr, &passes, st))
-            PD_CK(cudaMemcpyAsync(drot.as<int>() + max_sweeps, &passes, sizeof(int), cudaMemcpyHostToDevice, st));
-        else
-            launch_jacobi<double>(dsecs.as<SvdSec>(), nsec, dpairs.as<int>(), npairs, maxnpad, max_sweeps,
-                                  dW.as<double>(), dV.as<double>(), tol, 0.0, nullptr, drot.as<int>(),
-                                  drot.as<int>() + max_sweeps, bar, jerr, st);
+        jacobi64_finish(ss, dsecs.as<SvdSec>(), dpairs, npairs, maxnpad, max_sweeps, dW, dV, woff, voff, soff, drot.as<int>(),
+                        bar, jerr, st);
         launch_svd_finish<double>(dsecs.as<SvdSec>(), nsec, maxn, dW.as<double>(), dsig.as<double>(), dord.as<int>(), st);
         if (accurate && woff > 0)
             accurate_refine(ss, dsecs.as<SvdSec>(), dW.as<double>(), dV.as<double>(), dsig.as<double>(),
