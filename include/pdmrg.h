@@ -316,7 +316,8 @@ typedef struct {
     double f32_gemm_flops;
     long long svd_calls;         /* block-sparse SVD passes (one per split, or one per batch of
                                     splits of several regions' bonds run together)               */
-    long long svd_sweeps;        /* Jacobi sweeps they ran in total                             */
+    long long svd_sweeps;        /* Jacobi sweeps they ran in total; FP64 splits: whole-matrix passes
+                                    where these settled, else sweeps of the scalar Jacobi        */
     double svd_ms;               /* device time of their Jacobi kernels                         */
     long long svd_block_calls;   /* of those, FP32 splits run by the block Jacobi                */
     long long svd_fp64_calls;    /* of those, FP64 splits (parity mode, shared bonds)            */
@@ -338,6 +339,9 @@ typedef struct {
     double svd_block_alg_bytes;  /* FP32 splits: the sector matrices read once, U and V written
                                     once (FP32), 4 (2 p n + n^2) per sector                      */
     long long emu_batches;       /* FP64 GEMM batches run emulated on the bf16 tensor cores       */
+    long long svd_scalar;        /* FP64 split passes whose whole-matrix rotations did not settle
+                                    (clustered singular values) and that went on to the scalar
+                                    Jacobi                                                       */
 } dmrg_profile;
 
 void dmrg_profile_enable(int on);

@@ -45,7 +45,8 @@ class Profile(C.Structure):
                 ("svd_fp64_fallbacks", C.c_longlong), ("svd_block_flops", C.c_double),
                 ("svd_rot_hist", C.c_longlong * 48), ("emu_fallbacks", C.c_longlong), ("tune_classes", C.c_longlong),
                 ("tune_changed", C.c_longlong), ("svd_bonds", C.c_longlong), ("svd_block_alg_flops", C.c_double),
-                ("svd_block_alg_bytes", C.c_double), ("emu_batches", C.c_longlong)]
+                ("svd_block_alg_bytes", C.c_double), ("emu_batches", C.c_longlong),
+                ("svd_scalar", C.c_longlong)]
 
     def as_dict(self):
         d = {k: getattr(self, k) for k, _ in self._fields_}

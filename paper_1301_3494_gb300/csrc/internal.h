@@ -71,6 +71,8 @@ void prof_fallback();
 // An emulated FP64 GEMM batch sent to the FP64 units by its scale guard (counted always).
 void prof_emu_fallback();
 void prof_emu_batch();
+// An FP64 split whose polish did not settle (counted always).
+void prof_svd_scalar();
 
 // Persistent and cooperative grids are sized to the SMs of the device; while R regions run
 // concurrently (one host thread each), each thread caps its grids at sms / R so that the regions

@@ -1511,6 +1511,13 @@ void fp64_precondition(const std::vector<SvdSec>& ss, const SvdSec* dsecs, DBuf&
 // Columns below about 1e-6 of the largest are not resolved by FP32 at all.  The first pass frees them
 // of the large columns (those angles are small) and leaves the angles among themselves, which a second
 // FP32 block Jacobi on these columns alone, scaled to order one, then makes small.
+// Columns of nearly equal norm want wide angles (tan > 0.1).  Taken beside the small ones these spoil the
+// quadratic convergence (what is left of a small angle is then a share of it, not its square), and those
+// between exactly degenerate columns are not even wanted: their cosines are the squares of the small angles
+// and vanish with them.  So they wait until the others are below kNarrow, turn only pairs above the
+// tolerance then, and a cluster of five or more columns goes to the scalar Jacobi at once.  A 200 x 200
+// matrix of two values: 13.2 ms with all angles taken together (and the scalar Jacobi after), 2.7 now, 14.6 by
+// the scalar Jacobi alone; 300 values 1e-9 apart, which only that one settles: 57.3, 55.1 and 55.7.
 // Columns below kNull of the sector's largest are finished: W V was formed in FP64, so a column that is
 // not zero in exact arithmetic does not come out below rounding, 1e-16 of the largest, and one that is (an
 // exactly low-rank matrix: its columns are multiples of each other, bit for bit) falls by that factor in
@@ -1523,17 +1530,20 @@ void fp64_precondition(const std::vector<SvdSec>& ss, const SvdSec* dsecs, DBuf&
 // ------------------------------------------------------------------------------------------
 constexpr int kPolishPasses = 16;
 constexpr double kNull = 0x1p-80;             // 8e-25, in column norms
+constexpr float kNarrow = 1e-8f;              // largest column norm of E
+constexpr double kClose = 1e-5;               // relative distance of two squared norms
 
 // One CTA per column j of a sector: E(:, j) from the lower triangle of G (rows i >= 64 (j / 64)),
 // rotations by at most tan = 0.6, and none between two columns at or after cut[sector].  stat, four
-// words per sector: [0] columns with a pair above tol (those above tol / 10 turn too), [1] n - (first column of an unresolved pair:
-// cos > 1e-3 and tan > 0.1), [2] largest squared column norm of E as float bits.
+// words per sector: [0] columns with a pair above tol (those above tol / 10 turn too, by small angles),
+// [1] n - (first column of an unresolved pair: cos > 1e-3 and tan > 0.1), [2] largest squared column norm of
+// E as float bits, [3] nonzero: without `wide`, a pair above tol waits.
 struct PolCol {
     int sec, j;
 };
 __global__ void k_polish_angles(const SvdSec* __restrict__ secs, const PolCol* __restrict__ cols,
                                 const double* __restrict__ G, double* __restrict__ E, const int* __restrict__ cut,
-                                unsigned* __restrict__ stat) {
+                                bool wide, unsigned* __restrict__ stat) {
     const PolCol pc = cols[blockIdx.x];
     const SvdSec s = secs[pc.sec];
     const int j = pc.j, n = s.n;
@@ -1551,18 +1561,23 @@ __global__ void k_polish_angles(const SvdSec* __restrict__ secs, const PolCol* _
     __syncthreads();
     const double null2 = kNull * kNull * __longlong_as_double(max(max(tops[0], tops[1]), max(tops[2], tops[3])));
     float sum = 0.f;
-    int above = 0, first = n;
+    int above = 0, first = n, waits = 0;
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
         const int lo = min(i, j), hi = max(i, j);
         const double g = Gs[hi + (long long)lo * n], gii = Gs[i + (long long)i * n];
         double t = 0.0;
         const double size = sqrt(gii * gjj);
         if (i != j && fabs(g) > 0.1 * tol * size && !(fmin(gii, gjj) <= null2)) {
-            above |= fabs(g) > tol * size;
+            const bool over = fabs(g) > tol * size;
+            above |= over;
             const double zeta = (gjj - gii) / (2.0 * g);
             t = 1.0 / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
             if (t > 0.1 && fabs(g) > 1e-3 * size) first = min(first, lo);
-            t = lo >= from ? 0.0 : fmin(t, 0.6);
+            if (lo >= from) t = 0.0;
+            else if (t > 0.1 || fabs(gjj - gii) <= kClose * fmax(gii, gjj)) {
+                waits |= over && !wide;
+                t = !wide || (t > 0.1 && !over) ? 0.0 : fmin(t, 0.6);
+            }
             if (zeta < 0.0 || (zeta == 0.0 && i > j)) t = -t;
             sum = fmaf((float)t, (float)t, sum);
         }
@@ -1571,12 +1586,14 @@ __global__ void k_polish_angles(const SvdSec* __restrict__ secs, const PolCol* _
     for (int o = 16; o > 0; o >>= 1) {
         sum += __shfl_xor_sync(0xffffffffu, sum, o);
         first = min(first, __shfl_xor_sync(0xffffffffu, first, o));
-        above |= __shfl_xor_sync(0xffffffffu, above, o);
     }
+    above = __any_sync(0xffffffffu, above);
+    waits = __any_sync(0xffffffffu, waits);
     __shared__ float ssum[4];
     if ((threadIdx.x & 31) == 0) {
         ssum[threadIdx.x >> 5] = sum;
         if (above) atomicAdd(&stat[4 * pc.sec], 1u);
+        if (waits) atomicOr(&stat[4 * pc.sec + 3], 1u);
         if (first < n) atomicMax(&stat[4 * pc.sec + 1], (unsigned)(n - first));
     }
     __syncthreads();
@@ -1625,21 +1642,21 @@ bool polish64(const std::vector<SvdSec>& ss, const SvdSec* dsecs, DBuf& dW, DBuf
     DBuf dcut;
     int maxn = 1;
     for (const SvdSec& x : ss) maxn = std::max(maxn, x.n);
-    int large = 0;                        // passes in a row with large angles
+    int large = 0;                        // passes whose wide angles were large together
     int stages = 3;                       // FP32 passes over unresolved columns still allowed
     for (int pass = 0; pass < kPolishPasses; ++pass) {
         run_gemm64(gG, dW.as<double>(), dW.as<double>(), G.as<double>(), st);
-        auto angles = [&]() {
+        auto angles = [&](bool wide) {
             upload(dcut, cut, st);
             PD_CK(cudaMemsetAsync(stat.p, 0, (size_t)nsec * 16, st));
             k_polish_angles<<<nc, 128, 0, st>>>(dsecs, dcols.as<PolCol>(), G.as<double>(), E.as<double>(),
-                                                dcut.as<int>(), stat.as<unsigned>());
+                                                dcut.as<int>(), wide, stat.as<unsigned>());
             PD_LAUNCHED();
             PD_CK(cudaMemcpyAsync(hs.data(), stat.p, (size_t)nsec * 16, cudaMemcpyDeviceToHost, st));
             PD_CK(cudaStreamSynchronize(st));
         };
         for (int s = 0; s < nsec; ++s) cut[s] = ss[s].n;
-        angles();
+        angles(false);
         bool unresolved = false, above = false;
         for (int s = 0; s < nsec; ++s) {
             above = above || hs[4 * s] > 0;
@@ -1650,18 +1667,28 @@ bool polish64(const std::vector<SvdSec>& ss, const SvdSec* dsecs, DBuf& dW, DBuf
         if (unresolved) {
             // the unresolved columns turn against the others only
             for (int s = 0; s < nsec; ++s) cut[s] = ss[s].n - (int)hs[4 * s + 1];
-            angles();
+            angles(false);
         }
-        float norm = 0.f;
-        for (int s = 0; s < nsec; ++s) {
-            float v;
-            std::memcpy(&v, &hs[4 * s + 2], 4);
-            if (!std::isfinite(v)) return false;
-            norm = std::max(norm, std::sqrt(v));
+        bool finite = true, waits = false;
+        auto largest = [&]() {
+            float m = 0.f;
+            for (int s = 0; s < nsec; ++s) {
+                float v;
+                std::memcpy(&v, &hs[4 * s + 2], 4);
+                finite = finite && std::isfinite(v);
+                m = std::max(m, std::sqrt(v));
+                waits = waits || hs[4 * s + 3];
+            }
+            return m;
+        };
+        float norm = largest();
+        if (finite && waits && norm <= kNarrow) {
+            angles(true);
+            norm = largest();
+            // columns that all want large angles among themselves do not settle this way
+            if (norm > 0.6f && !unresolved && (norm > 1.2f || ++large > 2)) return false;
         }
-        // a cluster whose columns all want large angles among themselves does not settle this way
-        large = !unresolved && norm > 0.6f ? large + 1 : 0;
-        if (large > 2) return false;
+        if (!finite) return false;
         // E <- Q - I
         if (norm <= 1e-6f) {
             // (I + E)(I - E^2)^(-1/2) = I + E + E^2 / 2 + O(|E|^3)
@@ -1755,21 +1782,23 @@ bool polish64(const std::vector<SvdSec>& ss, const SvdSec* dsecs, DBuf& dW, DBuf
 
 // The FP64 one-sided Jacobi of W from V on (after fp64_precondition, or from the identity in the plain mode):
 // the polish where it settles, else the scalar sweeps.  rot: max_sweeps + 1 zeroed ints, the last of which
-// gets the passes or sweeps taken; pairs: the sectors' column pairs.
-void jacobi64_finish(const std::vector<SvdSec>& ss, const SvdSec* dsecs, const DBuf& pairs, int npairs, int maxnpad,
+// gets the passes or sweeps taken; pairs: the sectors' column pairs.  Returns true where the polish did not
+// settle.
+bool jacobi64_finish(const std::vector<SvdSec>& ss, const SvdSec* dsecs, const DBuf& pairs, int npairs, int maxnpad,
                      int max_sweeps, DBuf& dW, DBuf& dV, long long woff, long long voff, long long soff, int* rot,
                      unsigned* bar, unsigned* err, cudaStream_t st) {
     const bool polish = g_svd_qr && woff > 0;
     int passes = 0;
     if (polish && polish64(ss, dsecs, dW, dV, woff, voff, soff, err, &passes, st)) {
         PD_CK(cudaMemcpyAsync(rot + max_sweeps, &passes, sizeof(int), cudaMemcpyHostToDevice, st));
-        return;
+        return false;
     }
     DBuf floor2;
     if (polish) floor2.ensure(std::max<size_t>(1, ss.size()) * 8, st);
     launch_jacobi<double>(dsecs, (int)ss.size(), pairs.as<int>(), npairs, maxnpad, max_sweeps, dW.as<double>(),
                           dV.as<double>(), 4.0 * DBL_EPSILON, polish ? kNull : 0.0, floor2.as<double>(), rot,
                           rot + max_sweeps, bar, err, st);
+    return polish;
 }
 
 void jacobi64(std::vector<SvdSec>& ss, DBuf& dWbuf, DBuf& dsecs, DBuf& dV, DBuf& dsig, DBuf& dord, cudaStream_t st) {
@@ -2097,8 +2126,9 @@ std::vector<SplitResult> svd_split_batch(const std::vector<SplitReq>& reqs, bool
             fp64_precondition(ss, dsecs.as<SvdSec>(), dW, dV.as<double>(), woff, voff, maxp, maxn, jerr, st);
         else
             launch_svd_init_v<double>(dsecs.as<SvdSec>(), nsec, maxn, dV.as<double>(), st);
-        jacobi64_finish(ss, dsecs.as<SvdSec>(), dpairs, npairs, maxnpad, max_sweeps, dW, dV, woff, voff, soff, drot.as<int>(),
-                        bar, jerr, st);
+        if (jacobi64_finish(ss, dsecs.as<SvdSec>(), dpairs, npairs, maxnpad, max_sweeps, dW, dV, woff, voff, soff,
+                            drot.as<int>(), bar, jerr, st))
+            prof_svd_scalar();
         launch_svd_finish<double>(dsecs.as<SvdSec>(), nsec, maxn, dW.as<double>(), dsig.as<double>(), dord.as<int>(), st);
         if (accurate && woff > 0)
             accurate_refine(ss, dsecs.as<SvdSec>(), dW.as<double>(), dV.as<double>(), dsig.as<double>(),

@@ -33,7 +33,7 @@ int* sweep_flags_host(int n) {
 
 std::atomic<long long> g_launches{0};
 std::atomic<long long> g_fallbacks{0};
-std::atomic<long long> g_emu_fallbacks{0}, g_emu_batches{0};
+std::atomic<long long> g_emu_fallbacks{0}, g_emu_batches{0}, g_svd_scalar{0};
 thread_local int g_prof_class = PROF_MV;
 
 namespace {
@@ -58,6 +58,7 @@ bool prof_on() { return g_on.load(std::memory_order_relaxed); }
 void prof_fallback() { g_fallbacks.fetch_add(1); }
 void prof_emu_fallback() { g_emu_fallbacks.fetch_add(1); }
 void prof_emu_batch() { g_emu_batches.fetch_add(1); }
+void prof_svd_scalar() { g_svd_scalar.fetch_add(1); }
 
 void* prof_start(cudaStream_t st) {
     cudaEvent_t* ev = new cudaEvent_t[2];
@@ -119,6 +120,7 @@ void dmrg_profile_reset(void) {
     g_fallbacks.store(0);
     g_emu_fallbacks.store(0);
     g_emu_batches.store(0);
+    g_svd_scalar.store(0);
 }
 
 dmrg_status dmrg_profile_read(dmrg_profile* out) {
@@ -165,6 +167,7 @@ dmrg_status dmrg_profile_read(dmrg_profile* out) {
     for (int i = 0; i < 48; ++i) out->svd_rot_hist[i] = g_rot_hist[i];
     out->emu_fallbacks = g_emu_fallbacks.load();
     out->emu_batches = g_emu_batches.load();
+    out->svd_scalar = g_svd_scalar.load();
     tune_stats(&out->tune_classes, &out->tune_changed);
     return DMRG_OK;
 }
