@@ -1560,13 +1560,14 @@ __global__ void k_polish_angles(const SvdSec* __restrict__ secs, const PolCol* _
     if ((threadIdx.x & 31) == 0) tops[threadIdx.x >> 5] = top;
     __syncthreads();
     const double null2 = kNull * kNull * __longlong_as_double(max(max(tops[0], tops[1]), max(tops[2], tops[3])));
+    const double rjj = sqrt(gjj);
     float sum = 0.f;
     int above = 0, first = n, waits = 0;
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
         const int lo = min(i, j), hi = max(i, j);
         const double g = Gs[hi + (long long)lo * n], gii = Gs[i + (long long)i * n];
         double t = 0.0;
-        const double size = sqrt(gii * gjj);
+        const double size = sqrt(gii) * rjj;
         if (i != j && fabs(g) > 0.1 * tol * size && !(fmin(gii, gjj) <= null2)) {
             const bool over = fabs(g) > tol * size;
             above |= over;
@@ -1851,10 +1852,13 @@ void jacobi64(std::vector<SvdSec>& ss, DBuf& dWbuf, DBuf& dsecs, DBuf& dV, DBuf&
 // lambda_1 >= ... >= lambda_n: p = the first index with lambda_p / lambda_1 < eps; if there is one,
 // X = U_p^T M V_p over the columns p..n, the same SVD and refinement recursively on X, then
 // U_p <- U_p U_X, V_p <- V_p V_X, lambda_p.. <- lambda_X.  Results written back into W, V, and
-// sig / ord recomputed.
+// sig / ord recomputed.  top: the largest singular value of the matrix each of ss descends from.  A
+// block at its rounding level holds nothing that the split keeps (its cutoff is 1e-12), and the
+// rounding noise of an exactly low-rank matrix is of low rank itself, level after level: it is not
+// refined (all-ones 200 x 200: 111 ms with all its levels).
 constexpr double ACC_EPS = 1e-4;
 void accurate_refine(const std::vector<SvdSec>& ss, const SvdSec* dsecs, double* W, double* V, double* sig, int* ord,
-                     const double* M, int depth, cudaStream_t st) {
+                     const double* M, int depth, cudaStream_t st, const std::vector<double>& top = {}) {
     const int nsec = (int)ss.size();
     long long total = 0;
     for (const auto& x : ss) total = std::max(total, x.s_off + x.n);
@@ -1869,21 +1873,24 @@ void accurate_refine(const std::vector<SvdSec>& ss, const SvdSec* dsecs, double*
         long long up, vp, x;
     };
     std::vector<Ref> refs;
+    std::vector<double> xtop;
     long long nup = 0, nvp = 0, nx = 0;
     for (int s = 0; s < nsec; ++s) {
         const SvdSec& S = ss[s];
         if (S.n <= 1) continue;
         const double l0 = hsig[S.s_off + hord[S.s_off]];
         if (!(l0 > 0.0)) continue;
+        const double l_top = depth > 0 ? top[s] : l0;
         int p = -1;
         for (int i = 1; i < S.n; ++i)
             if (hsig[S.s_off + hord[S.s_off + i]] / l0 < ACC_EPS) {
                 p = i;
                 break;
             }
-        if (p < 0) continue;
+        if (p < 0 || hsig[S.s_off + hord[S.s_off + p]] <= DBL_EPSILON * l_top) continue;
         const int q = S.n - p;
         refs.push_back({s, p, q, nup, nvp, nx});
+        xtop.push_back(l_top);
         nup += (long long)S.p * q;
         nvp += (long long)S.n * q;
         nx += (long long)q * q;
@@ -1928,7 +1935,7 @@ void accurate_refine(const std::vector<SvdSec>& ss, const SvdSec* dsecs, double*
     PD_CK(cudaMemcpyAsync(dXW.p, dX.p, nx * 8, cudaMemcpyDeviceToDevice, st));
     jacobi64(xs, dXW, dXsecs, dXV, dXsig, dXord, st);
     accurate_refine(xs, dXsecs.as<SvdSec>(), dXW.as<double>(), dXV.as<double>(), dXsig.as<double>(),
-                    dXord.as<int>(), dX.as<double>(), depth + 1, st);
+                    dXord.as<int>(), dX.as<double>(), depth + 1, st, xtop);
     std::vector<int> hxo(nx > 0 ? (size_t)std::max<long long>(1, xs.back().s_off + xs.back().n) : 1);
     PD_CK(cudaMemcpyAsync(hxo.data(), dXord.p, hxo.size() * 4, cudaMemcpyDeviceToHost, st));
     PD_CK(cudaStreamSynchronize(st));
