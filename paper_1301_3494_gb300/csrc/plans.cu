@@ -586,7 +586,7 @@ void convert_flat(const void* src, Num in, void* dst, Num out, long long n, cuda
     }
 }
 
-void orthonormalize_square(const std::vector<SvdSec>& ss, double* V, cudaStream_t st, int max_iter) {
+bool orthonormalize_square(const std::vector<SvdSec>& ss, double* V, cudaStream_t st, int steps) {
     std::vector<NsJob> jobs;
     GemmBatch gG, gX;
     long long tot = 0, first = 0, sum = 0;
@@ -602,7 +602,7 @@ void orthonormalize_square(const std::vector<SvdSec>& ss, double* V, cudaStream_
         gX.add(n, n, x.v_off, 1, n, n, 1, 1, n, {GSeg{x.v_off, x.v_off, n, 0}});
         tot = std::max(tot, x.v_off + (long long)n * n);
     }
-    if (jobs.empty()) return;
+    if (jobs.empty()) return true;
     PD_REQUIRE(sum == tot - first, DMRG_ERR_STATE, "sector matrices are not contiguous");
     DBuf G, T, out, dev, dj;
     G.ensure(tot * 8, st);
@@ -610,21 +610,21 @@ void orthonormalize_square(const std::vector<SvdSec>& ss, double* V, cudaStream_
     out.ensure(tot * 8, st);
     upload(dj, jobs, st);
     NsStep ns(dj, jobs);
-    for (int iter = 0; iter < max_iter; ++iter) {
+    for (int iter = 0; iter < steps; ++iter) {
         run_gemm64(gG, V, V, G.as<double>(), st);
         const GramDev d = gram_deviation(dj, jobs, G, dev, st);
         const double worst = d.max;
         PD_REQUIRE(std::isfinite(worst) && worst < 0.5, DMRG_ERR_NUMERIC,
                    "FP32 Jacobi rotations too far from orthogonal for the FP64 polish (|V^T V - I| = " +
                        std::to_string(worst) + " at iteration " + std::to_string(iter) + ")");
-        if (worst < 1e-14) return;
+        if (worst < 1e-14) return true;
         const bool last = ns.make(d, 1e-14, G, T, st);
         run_gemm64(gX, V, T.as<double>(), out.as<double>(), st);
         // the matrices follow each other without gaps
         PD_CK(cudaMemcpyAsync(V + first, out.as<double>() + first, (size_t)(tot - first) * 8, cudaMemcpyDeviceToDevice, st));
-        if (last) return;
+        if (last) return true;
     }
-    PD_REQUIRE(max_iter <= 8, DMRG_ERR_NUMERIC, "Newton-Schulz orthonormalisation did not converge");
+    return false;
 }
 
 void scale_vec(double* x, long long n, double s, cudaStream_t st) {
@@ -1483,7 +1483,7 @@ void fp64_precondition(const std::vector<SvdSec>& ss, const SvdSec* dsecs, DBuf&
     block_jacobi32(ss, dsecs, w32.as<float>(), v32.as<float>(), maxp, max_sweeps, rot32.as<int>(), err,
                    fl.as<unsigned long long>(), st);
     convert_flat(v32.p, Num::F32, V, Num::F64, voff, st);
-    orthonormalize_square(ss, V, st);
+    orthonormalize_square(ss, V, st, 8);          // (from FP32's 1e-4 two or three steps)
     GemmBatch gwq;
     for (const auto& x : ss)
         if (x.n > 0)   // W1(r, c) = sum_u W(r, u) V(u, c)
@@ -1645,6 +1645,15 @@ bool polish64(const std::vector<SvdSec>& ss, const SvdSec* dsecs, DBuf& dW, DBuf
     for (const SvdSec& x : ss) maxn = std::max(maxn, x.n);
     int large = 0;                        // passes whose wide angles were large together
     int stages = 3;                       // FP32 passes over unresolved columns still allowed
+    // false: too far from orthogonal; W and V are as before, for the scalar Jacobi to go on with
+    auto orthonormalized = [&](const std::vector<SvdSec>& of, DBuf& Q, int steps) {
+        try {
+            return orthonormalize_square(of, Q.as<double>(), st, steps);
+        } catch (const Error& e) {
+            if (e.st != DMRG_ERR_NUMERIC) throw;
+            return false;
+        }
+    };
     for (int pass = 0; pass < kPolishPasses; ++pass) {
         run_gemm64(gG, dW.as<double>(), dW.as<double>(), G.as<double>(), st);
         auto angles = [&](bool wide) {
@@ -1700,12 +1709,7 @@ bool polish64(const std::vector<SvdSec>& ss, const SvdSec* dsecs, DBuf& dW, DBuf
             k_polish_shift<<<nc, 128, 0, st>>>(dsecs, dcols.as<PolCol>(), E.as<double>(), norm > 0.6f ? 0.6 / norm : 1.0,
                                                1.0, X.as<double>());
             PD_LAUNCHED();
-            try {
-                orthonormalize_square(ss, X.as<double>(), st, 14);
-            } catch (const Error& e) {
-                if (e.st != DMRG_ERR_NUMERIC) throw;
-                return false;                 // angles too large to take together: W and V are as before
-            }
+            if (!orthonormalized(ss, X, 14)) return false;     // angles too large to take together
             k_polish_shift<<<nc, 128, 0, st>>>(dsecs, dcols.as<PolCol>(), X.as<double>(), 1.0, -1.0, E.as<double>());
             PD_LAUNCHED();
         }
@@ -1770,7 +1774,7 @@ bool polish64(const std::vector<SvdSec>& ss, const SvdSec* dsecs, DBuf& dW, DBuf
         block_jacobi32(sub, dsub.as<SvdSec>(), w32.as<float>(), v32.as<float>(), mp, max_sweeps, rot32.as<int>(), err,
                        fl.as<unsigned long long>(), st, 0.0f);
         convert_flat(v32.p, Num::F32, v64.p, Num::F64, vo, st);
-        orthonormalize_square(sub, v64.as<double>(), st);
+        if (!orthonormalized(sub, v64, 8)) return false;
         PD_CK(cudaMemcpyAsync(Wn.p, dW.p, woff * 8, cudaMemcpyDeviceToDevice, st));
         PD_CK(cudaMemcpyAsync(Vn.p, dV.p, voff * 8, cudaMemcpyDeviceToDevice, st));
         run_gemm64(gw, dW.as<double>(), v64.as<double>(), Wn.as<double>(), st);

@@ -449,10 +449,11 @@ void orthonormalize_factor(const Sec& bl, const Sec& br, const std::vector<int>&
                            cudaStream_t st);
 // Flat element-type conversion of n elements (FP64 or FP32 source), stream-ordered.
 void convert_flat(const void* src, Num in, void* dst, Num out, long long n, cudaStream_t st);
-// Newton-Schulz orthonormalisation in FP64 of the square n x n matrices at v_off (column-major) of
-// V, one per sector of ss, until |V^T V - I|_max < 1e-14.  Takes at most max_iter steps; above 8,
-// not having got there by then is DMRG_ERR_NUMERIC.
-void orthonormalize_square(const std::vector<SvdSec>& ss, double* V, cudaStream_t st, int max_iter = 8);
+// Orthonormalises in FP64 the square n x n matrices at v_off (column-major) of V, one per sector of ss: Newton-
+// Schulz steps, ended by a series whose truncation leaves |V^T V - I| below 1e-14 (the rounding of its
+// products, n eps and the like, comes on top and is not measured).  False: not there after `steps` steps.
+// |V^T V - I|_max of 0.5 or more, or not finite: DMRG_ERR_NUMERIC.
+bool orthonormalize_square(const std::vector<SvdSec>& ss, double* V, cudaStream_t st, int steps);
 // Worst-case (untruncated) element counts of the split's A and B outputs.
 void svd_split_bounds(const Sec& bl, const Sec& br, const std::vector<int>& qn1, const std::vector<int>& qn2,
                       long long* a_elems, long long* b_elems, long long* lam_elems);
