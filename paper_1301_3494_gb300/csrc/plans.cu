@@ -387,28 +387,30 @@ __global__ void k_mirror(const NsJob* jobs, double* T) {
 }
 // dev[2 x] = max |G - I|, dev[2 x + 1] = sum of (G - I)^2 over CTA x's columns of block s (x = s gridDim.x +
 // blockIdx.x).  CTAs share a block: one CTA each took 1.2 ms for the blocks of an m = 2000 bond.
-__global__ void __launch_bounds__(128) k_gram_dev(const NsJob* jobs, const double* G, float* dev) {
+__global__ void __launch_bounds__(128) k_gram_dev(const NsJob* jobs, const double* G, double* dev) {
     const NsJob j = jobs[blockIdx.y];
-    float m = 0.f, f = 0.f;
+    long long m = 0;                                           // magnitudes order like their bits
+    double f = 0.0;
     for (int c = blockIdx.x; c < j.k; c += gridDim.x)
         for (int r = c + threadIdx.x; r < j.k; r += blockDim.x) {
-            const float d = fabsf((float)(G[j.off + r + (long long)c * j.k] - (r == c ? 1.0 : 0.0)));
-            m = fmaxf(m, d);                                   // (NaN is passed over)
-            f = fmaf(r == c ? d : 2.f * d, d, f);
+            const double d = fabs(G[j.off + r + (long long)c * j.k] - (r == c ? 1.0 : 0.0));
+            if (d == d) m = max(m, __double_as_longlong(d));   // (NaN is passed over)
+            f = fma(r == c ? d : 2.0 * d, d, f);
         }
     for (int o = 16; o > 0; o >>= 1) {
-        m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+        m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
         f += __shfl_xor_sync(0xffffffffu, f, o);
     }
-    __shared__ float sm[4], sf[4];
+    __shared__ long long sm[4];
+    __shared__ double sf[4];
     if ((threadIdx.x & 31) == 0) {
         sm[threadIdx.x >> 5] = m;
         sf[threadIdx.x >> 5] = f;
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-        float* o = dev + 2 * ((long long)blockIdx.y * gridDim.x + blockIdx.x);
-        o[0] = fmaxf(fmaxf(sm[0], sm[1]), fmaxf(sm[2], sm[3]));
+        double* o = dev + 2 * ((long long)blockIdx.y * gridDim.x + blockIdx.x);
+        o[0] = __longlong_as_double(max(max(sm[0], sm[1]), max(sm[2], sm[3])));
         o[1] = (sf[0] + sf[1]) + (sf[2] + sf[3]);
     }
 }
@@ -420,17 +422,17 @@ GramDev gram_deviation(const DBuf& djobs, const std::vector<NsJob>& jobs, const 
     int kmax = 1;
     for (const NsJob& j : jobs) kmax = std::max(kmax, j.k);
     const int ctas = std::min(kmax, 32);
-    std::vector<float> h((size_t)2 * n * ctas);
-    dev.ensure(h.size() * 4, st);
-    k_gram_dev<<<dim3(ctas, (unsigned)n), 128, 0, st>>>(djobs.as<NsJob>(), G.as<double>(), dev.as<float>());
+    std::vector<double> h((size_t)2 * n * ctas);
+    dev.ensure(h.size() * 8, st);
+    k_gram_dev<<<dim3(ctas, (unsigned)n), 128, 0, st>>>(djobs.as<NsJob>(), G.as<double>(), dev.as<double>());
     PD_LAUNCHED();
-    PD_CK(cudaMemcpyAsync(h.data(), dev.p, h.size() * 4, cudaMemcpyDeviceToHost, st));
+    PD_CK(cudaMemcpyAsync(h.data(), dev.p, h.size() * 8, cudaMemcpyDeviceToHost, st));
     PD_CK(cudaStreamSynchronize(st));
     GramDev d{0.0, 0.0};
     for (int s = 0; s < n; ++s) {
         double f = 0.0;
         for (int x = 0; x < ctas; ++x) {
-            d.max = std::max(d.max, (double)h[2 * ((size_t)s * ctas + x)]);
+            d.max = std::max(d.max, h[2 * ((size_t)s * ctas + x)]);
             f += h[2 * ((size_t)s * ctas + x) + 1];
         }
         // (a sum that overflowed, or NaN, settles nothing)
