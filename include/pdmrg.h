@@ -286,7 +286,16 @@ dmrg_status dmrg_local_expectations(dmrg_ctx* ctx, int n_ops1, const double* ops
 /* Orthogonality-centre site of the serial state, or of region k in region mode. */
 dmrg_status dmrg_get_center(dmrg_ctx* ctx, int region, int* site_out);
 
+/* Releases the context and its device memory; the last one on a device also gives back what the
+ * library's memory pool kept. */
 dmrg_status dmrg_destroy(dmrg_ctx* ctx);
+
+/* The library allocates device memory from a stream-ordered pool of its own, which no other
+ * allocator of the process can draw on.  While a context lives the pool keeps all memory it has
+ * ever needed; between single operations without a context it keeps up to 2 GiB per device for the
+ * next one.  dmrg_trim synchronises the current device and gives back everything that is not in
+ * use, on every device the library has used. */
+dmrg_status dmrg_trim(void);
 
 /* Message of the last failure on this context (context-owned, valid until the next call). */
 const char* dmrg_last_error(const dmrg_ctx* ctx);

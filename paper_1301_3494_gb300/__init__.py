@@ -150,7 +150,8 @@ def lib():
                                      _dp, vp]
         L.dmrg_svd_split_batch.argtypes = [C.c_int, C.POINTER(BondDesc), C.POINTER(vp), _ip, C.c_int, C.POINTER(vp),
                                            C.POINTER(vp), C.POINTER(vp), C.c_int, _ip, _ip, _ip, _dp, vp]
-        for name in ("dmrg_init_mpo", "dmrg_set_mps", "dmrg_setup_regions", "dmrg_sweep", "dmrg_advance",
+        L.dmrg_trim.argtypes = []
+        for name in ("dmrg_init_mpo", "dmrg_set_mps", "dmrg_trim", "dmrg_setup_regions", "dmrg_sweep", "dmrg_advance",
                      "dmrg_profile_read", "dmrg_merge",
                      "dmrg_energy", "dmrg_get_bond", "dmrg_get_lambda", "dmrg_get_center", "dmrg_get_site",
                      "dmrg_energy_gradient", "dmrg_destroy", "dmrg_inverse_canonical", "dmrg_icmps_bond",
@@ -175,6 +176,11 @@ def profile_read():
     p = Profile()
     _check(lib().dmrg_profile_read(C.byref(p)))
     return p.as_dict()
+
+
+def trim():
+    """Give the device memory that the library keeps between operations back to the driver (dmrg_trim)."""
+    _check(lib().dmrg_trim())
 
 
 def probe(kind, stream=0):

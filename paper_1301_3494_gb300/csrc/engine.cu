@@ -1232,7 +1232,10 @@ dmrg_status dmrg_destroy(dmrg_ctx* c) {
     cudaStreamSynchronize(c->base);
     for (auto& r : c->reg)
         if (r->st) cudaStreamSynchronize(r->st);
+    const cudaStream_t base = c->base;
     delete c;   // buffers free on their streams, then the owned streams are destroyed
+    cudaStreamSynchronize(base);
+    pool_trim(true);
     return DMRG_OK;
 }
 

@@ -34,8 +34,10 @@ struct Error {
     } while (0)
 
 // Stream-ordered device memory from the library's pool on the current device (pool.cu); freed with
-// cudaFreeAsync.  A PoolHold makes the pool keep all freed memory while it lives.
+// cudaFreeAsync.  A PoolHold makes the pool keep all freed memory while it lives; pool_trim gives back
+// what is freed and not in use (idle_only: on devices without a PoolHold).
 void* pool_alloc(size_t bytes, cudaStream_t st);
+cudaError_t pool_trim(bool idle_only);
 struct PoolHold {
     int dev = 0;
     PoolHold();

@@ -3,10 +3,12 @@
 // Work buffers live for one call or one step, so a pool that hands freed memory back at every
 // synchronisation -- the default release threshold is 0 -- maps it again on the next call: a 64-state
 // matvec took 510 us after a synchronisation against 170 among other calls.  The pool is the
-// library's own, so its threshold touches no other user of the device's default pool.  It keeps up to
-// kIdleBytes between calls; while a context is alive, whose sweeps free and allocate gigabytes per
-// bond step, it keeps everything, and the last context gives the rest back.  All of it is safe
-// from several host threads and streams (the driver's pool is).
+// library's own, so its threshold touches no other user of the device's default pool -- and no other
+// allocator of the process can use what it keeps.  That is up to kIdleBytes between single operations
+// (those at the largest bonds take half a gigabyte and more, and free it, each call); everything while
+// a context is alive, whose sweeps free and allocate gigabytes per bond step; nothing after the last
+// context is destroyed or dmrg_trim is called.  All of it is safe from several host threads and streams
+// (the driver's pool is).
 #include <mutex>
 
 #include "internal.h"
@@ -81,7 +83,30 @@ PoolHold::~PoolHold() {
     if (--g_pools[dev].holders > 0) return;
     unsigned long long keep = kIdleBytes;
     cudaMemPoolSetAttribute(g_pools[dev].pool, cudaMemPoolAttrReleaseThreshold, &keep);
-    cudaMemPoolTrimTo(g_pools[dev].pool, kIdleBytes);
+}
+
+cudaError_t pool_trim(bool idle_only) {
+    std::lock_guard<std::mutex> lk(g_mu);
+    cudaError_t e = cudaSuccess;
+    for (const DevicePool& d : g_pools)
+        if (d.pool && !(idle_only && d.holders > 0)) {
+            const cudaError_t x = cudaMemPoolTrimTo(d.pool, 0);
+            if (x != cudaSuccess) e = x;
+        }
+    return e;
+}
+
+static bool pool_in_use() {
+    std::lock_guard<std::mutex> lk(g_mu);
+    for (const DevicePool& d : g_pools)
+        if (d.pool) return true;
+    return false;
 }
 
 }  // namespace pd
+
+extern "C" dmrg_status dmrg_trim(void) {
+    if (!pd::pool_in_use()) return DMRG_OK;          // (nothing allocated yet: no device call)
+    if (cudaDeviceSynchronize() != cudaSuccess) return DMRG_ERR_CUDA;
+    return pd::pool_trim(false) == cudaSuccess ? DMRG_OK : DMRG_ERR_CUDA;
+}
