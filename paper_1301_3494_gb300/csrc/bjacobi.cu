@@ -61,7 +61,6 @@ struct alignas(16) BjShared {
         float Q[2][BJ_K * BJ_QLD];             // accumulated rotation; its column-permuted copy
     };
     float G[2][BJ_K * BJ_GLD];                 // Gram matrix, one copy read and one written a round
-    float diag[BJ_K];
     int gcol[BJ_K];                            // sector column of staged column u (-1: padding)
     int pos[BJ_K];                             // pos[v] = position of eigenvector v
     float gmax;                                // largest squared column norm seen in the sector

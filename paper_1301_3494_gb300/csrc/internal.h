@@ -80,6 +80,8 @@ void prof_svd_scalar();
 // concurrently (one host thread each), each thread caps its grids at sms / R so that the regions
 // share the GPU spatially instead of queueing behind each other's resident grids.
 extern thread_local int g_sm_cap;   // 0: no cap
+// SMs of a GB300: grid sizes and tile rules are laid out for it (the kernels run on any number).
+constexpr int kSMs = 152;
 inline int sm_share(int sms) { return g_sm_cap > 0 ? std::max(1, std::min(sms, g_sm_cap)) : sms; }
 
 // Pinned host words (one per sweep, at least n) owned by the calling thread, for reading the

@@ -1288,14 +1288,21 @@ void launch_gemm_f32(const GProb* probs, const GSeg* segs, const GTile* tiles, i
 
 F64Shape f64_shape(const std::vector<GProb>& probs, const std::vector<GSeg>& segs) {
     // 16 x 16 tiles and their mean K decide.  A tile's chain is 8 K warp instructions of 64 clocks on
-    // one scheduler, and 608 schedulers (152 SMs) want several tiles each: with 16 or more (or a K
-    // too short to divide) a warp takes a tile alone, else four warps share one, and 16 where there
-    // are fewer tiles than schedulers and a long K.  Measured, one / four / sixteen warps a tile:
-    //   5000 of 15x15x15              74 /   92 /  346 us   (64 x 64 CTA tiles before: 541)
-    //     34 of 80x80x80              69 /   53 /  100      (98)
-    //     52 of 15x15, 98 x K = 15   468 /  133 /  112      (1625)
-    //     17 of 320x320x640         1964 / 1869 / 2300      (1957; 1.19 TFLOP/s of the 1.25 measured peak)
-    //    400 of 150x150x150         2300 / 2477 / 4583      (3859)
+    // one scheduler, and the 4 kSMs schedulers want several tiles each: with 16 or more (or a K too
+    // short to divide) a warp takes a tile alone, else four warps share one; eight where there are no
+    // more tiles than schedulers and K is at least 128, sixteen where there are no more than SMs and K is
+    // at least 256.  Measured, one / four / eight / sixteen warps a tile, in us:
+    //   5000 of 15x15x15 (5000 tiles)          76 /   89 /  199 /  342   (64 x 64 CTA tiles before: 541)
+    //    400 of 150x150x150 (40000)          2300 / 2476 / 3563 / 4583   (3859)
+    //     17 of 320x320x640 (6800)           1960 / 1868 / 2121 / 2297   (1957; 1.19 TFLOP/s of the 1.25 measured peak)
+    //     34 of 80x80x80 (850)                 65 /   47 /   70 /   94   (98)
+    //    320x320x640 (400)                    227 /  139 /  147 /  158
+    //     10 of 100x100x128 (490)              80 /   45 /   55 /   70
+    //    160x160x640 (100)                    226 /   64 /   54 /   58
+    //     52 of 15x15, 98 x K = 15 (52)       465 /  130 /  108 /  108   (1625)
+    // Below one tile an SM eight and sixteen win over four by a sixth; the line of the eight-warp shape was
+    // drawn against sixteen (R stage of the m = 500 matvec 578 -> 440 us): from 153 to 608 tiles four does as
+    // well or better (that call 1110 us with the rule, 1052 with four).
     long long tiles = 0, kt = 0;
     for (const GProb& p : probs) {
         const long long t = (long long)((p.M + 15) / 16) * ((p.N + 15) / 16);
@@ -1306,8 +1313,8 @@ F64Shape f64_shape(const std::vector<GProb>& probs, const std::vector<GSeg>& seg
     }
     const double kmean = tiles ? (double)kt / (double)tiles : 0.0;
     if (tiles >= 9728 || kmean < 16.0) return {32, 1};
-    if (tiles <= 152 && kmean >= 256.0) return {16, 16};
-    if (tiles <= 608 && kmean >= 128.0) return {16, 8};
+    if (tiles <= kSMs && kmean >= 256.0) return {16, 16};
+    if (tiles <= 4 * kSMs && kmean >= 128.0) return {16, 8};
     return {16, 4};
 }
 
@@ -1334,7 +1341,7 @@ void launch_copy(const CopyJob* jobs, const int2* chunks, int nchunks, const Tin
 template <class Tin, class Tout>
 void launch_convert(const Tin* src, Tout* dst, long long n, cudaStream_t st) {
     if (n <= 0) return;
-    k_convert<Tin, Tout><<<(unsigned)std::max<long long>(1, std::min<long long>((n + 2047) / 2048, 152 * 8)), 256, 0, st>>>(
+    k_convert<Tin, Tout><<<(unsigned)std::max<long long>(1, std::min<long long>((n + 2047) / 2048, 8 * kSMs)), 256, 0, st>>>(
         src, dst, n);
     PD_LAUNCHED();
 }
@@ -1381,7 +1388,7 @@ void launch_dots(const double* V, long long ldv, int k, const double* y, long lo
 }
 
 int dav_grid(long long n) {
-    return (int)std::max<long long>(1, std::min<long long>((n + DAV_THREADS - 1) / DAV_THREADS, 152 * 4));
+    return (int)std::max<long long>(1, std::min<long long>((n + DAV_THREADS - 1) / DAV_THREADS, 4 * kSMs));
 }
 
 void launch_dav_gram(const double* V, const double* AV, long long n, int k, int kmax, double* G, double* partial,

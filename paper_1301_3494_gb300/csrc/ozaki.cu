@@ -381,7 +381,7 @@ std::unique_ptr<EmuPlan> build_plan(const GemmBatch& g, cudaStream_t st) {
             if ((double)((1 << beta) - 1) * ((1 << beta) - 1) * (double)kmax_tot * per > lim) continue;
             const int pairs = s * (s + 1) / 2, groups = lv ? s : pairs;
             // tensor-core flops, FP32 partial results written and read back, per-tile overhead
-            const double ms = pairs * flops / 2.5e11 + groups * mn_tot * 8.0 / 5.0e9 + groups * tiles * 1.5e-3 / 152.0;
+            const double ms = pairs * flops / 2.5e11 + groups * mn_tot * 8.0 / 5.0e9 + groups * tiles * 1.5e-3 / kSMs;
             if (best.ms < 0 || ms < best.ms) best = {lv != 0, beta, s, groups, pairs, ms};
             break;
         }

@@ -786,7 +786,6 @@ std::unique_ptr<HeffPlan> make_heff_plan(const Sec& bl, const Sec& br, const std
                 for (int t = Y.t0; t < Y.t0 + Y.nt; ++t)
                     P->mix.terms.push_back({xs[yt[t].first].off, xs[yt[t].first].cols, 0, yt[t].second});
                 P->mix.jobs.push_back(mj);
-                P->mix.max_elems = std::max(P->mix.max_elems, mj.rows * std::max(mj.cols, mj.zero_to));
             }
             rs.push_back({R.blk[Y.rb].row * R.ld, Y.row * P->ld_y, x0.cols, 0});
         }
@@ -808,7 +807,6 @@ std::unique_ptr<HeffPlan> make_heff_plan(const Sec& bl, const Sec& br, const std
             ++j.nt;
         }
         P->djobs.push_back(j);
-        P->diag_max = std::max(P->diag_max, B.rows * B.cols);
     }
 
     P->flops = P->lstage.flops + P->ldirect.flops + P->rstage.flops + P->mix.flops;
@@ -1123,7 +1121,6 @@ void env_update_left(const Sec& ba, const Sec& bb, const std::vector<int>& qn, c
                 mj.dst = trow * ldT; mj.rows = x0->rows; mj.cols = x0->cols; mj.ldo = ldT;
                 mj.zero_to = kpad(x0->cols, prec); mj.t0 = first; mj.nt = (int)mx.terms.size() - first;
                 mx.jobs.push_back(mj);
-                mx.max_elems = std::max(mx.max_elems, mj.rows * std::max(mj.cols, mj.zero_to));
                 trow += x0->rows;
             }
         }
@@ -1243,7 +1240,6 @@ void env_update_right(const Sec& ba, const Sec& bc, const std::vector<int>& qn, 
                 mj.dst = trow * ldT; mj.rows = x0->rows; mj.cols = x0->cols; mj.ldo = ldT;
                 mj.zero_to = kpad(x0->cols, prec); mj.t0 = first; mj.nt = (int)mx.terms.size() - first;
                 mx.jobs.push_back(mj);
-                mx.max_elems = std::max(mx.max_elems, mj.rows * std::max(mj.cols, mj.zero_to));
                 trow += x0->rows;
             }
         }

@@ -256,11 +256,9 @@ struct CopyList {
     std::vector<long long> elems;
     DBuf d, dc;
     int nchunks = 0;
-    int max_elems = 0;
     void add(const CopyJob& j) {
         jobs.push_back(j);
         elems.push_back((long long)j.rows * std::max(j.cols, j.zero_to));
-        max_elems = std::max(max_elems, j.rows * std::max(j.cols, j.zero_to));
     }
     void up(cudaStream_t st) {
         upload(d, jobs, st);
@@ -280,7 +278,6 @@ struct MixList {
     std::vector<MixTerm> terms;
     DBuf dj, dt, dc;
     int nchunks = 0;
-    int max_elems = 0;
     double flops = 0.0;
     void up(cudaStream_t st) {
         upload(dj, jobs, st);
@@ -363,7 +360,7 @@ struct HeffPlan {
     std::vector<DiagJob> djobs;
     std::vector<DiagTerm> dterms;
     DBuf ddj, ddt, ddc;
-    int diag_max = 0, diag_chunks = 0;
+    int diag_chunks = 0;
     double flops = 0.0;
     DBuf lists;               // every list above, one allocation
     // scratch
