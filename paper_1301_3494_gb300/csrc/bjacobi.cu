@@ -227,12 +227,12 @@ __device__ __forceinline__ void bj_rotate_out(const float* __restrict__ X, int l
 // and s are normalised to c^2 + s^2 = 1 within rounding, since the accumulated rotations must stay
 // orthogonal.
 __device__ __forceinline__ void bj_rot(float gpp, float gqq, float gpq, float& c, float& s) {
-    float d = gqq - gpp, h = 2.f * gpq;
+    float d = gqq - gpp, h = gpq;
     const float m = fmaxf(fabsf(d), fabsf(h));
-    // 2^-exponent(m): its bits are 254 - e in the exponent field (m is a normal number below 2^127)
-    const float sc = __int_as_float(0x7f000000 - (__float_as_int(m) & 0x7f800000));
+    // 2^-exponent(m): its bits are 254 - e in the exponent field; 2^-126 from 2^126 on
+    const float sc = __int_as_float(max(0x7f000000 - (__float_as_int(m) & 0x7f800000), 0x00800000));
     d *= sc;
-    h *= sc;
+    h *= 2.f * sc;
     const float r = rsqrtf(fmaf(d, d, h * h));
     const float c2 = fmaf(0.5f * fabsf(d), r, 0.5f);
     const float y = rsqrtf(c2);
