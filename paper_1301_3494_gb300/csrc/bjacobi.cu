@@ -232,7 +232,8 @@ __device__ __forceinline__ void bj_rot(float gpp, float gqq, float gpq, float& c
     // 2^-exponent(m): its bits are 254 - e in the exponent field; 2^-126 from 2^126 on
     const float sc = __int_as_float(max(0x7f000000 - (__float_as_int(m) & 0x7f800000), 0x00800000));
     d *= sc;
-    h *= 2.f * sc;
+    h *= sc;                                           // (2 sc would overflow where m is not normal)
+    h += h;
     const float r = rsqrtf(fmaf(d, d, h * h));
     const float c2 = fmaf(0.5f * fabsf(d), r, 0.5f);
     const float y = rsqrtf(c2);
