@@ -1511,11 +1511,13 @@ void fp64_precondition(const std::vector<SvdSec>& ss, const SvdSec* dsecs, DBuf&
 // FP32 block Jacobi on these columns alone, scaled to order one, then makes small.
 // Columns of nearly equal norm want wide angles (tan > 0.1).  Taken beside the small ones these spoil the
 // quadratic convergence (what is left of a small angle is then a share of it, not its square), and those
-// between exactly degenerate columns are not even wanted: their cosines are the squares of the small angles
-// and vanish with them.  So they wait until the others are below kNarrow, turn only pairs above the
-// tolerance then, and a cluster of five or more columns goes to the scalar Jacobi at once.  A 200 x 200
-// matrix of two values: 13.2 ms with all angles taken together (and the scalar Jacobi after), 2.7 now, 14.6 by
-// the scalar Jacobi alone; 300 values 1e-9 apart, which only that one settles: 57.3, 55.1 and 55.7.
+// between exactly degenerate columns are not even wanted: their cosines are the products of those with the
+// other columns and vanish with them.  So a pair of nearly equal columns turns only where its cosine is
+// above the tolerance and above what the others explain (the root of the product of the two columns' sums of
+// squared cosines), and a cluster of five or more columns goes to the scalar Jacobi at once.  A 200 x 200 matrix of two values:
+// 13.2 ms with all angles taken together (and the scalar Jacobi after), 2.8 now, 14.6 by the scalar Jacobi
+// alone; 300 values 1e-9 apart, which only that one settles: 57.3, 55.1 and 55.7.  (Waiting for all small
+// angles instead costs passes where a few pairs are close: 7 to 15 for 5 or 6 at an FP64 m = 2000 bond.)
 // Columns below kNull of the sector's largest are finished: W V was formed in FP64, so a column that is
 // not zero in exact arithmetic does not come out below rounding, 1e-16 of the largest, and one that is (an
 // exactly low-rank matrix: its columns are multiples of each other, bit for bit) falls by that factor in
@@ -1528,20 +1530,20 @@ void fp64_precondition(const std::vector<SvdSec>& ss, const SvdSec* dsecs, DBuf&
 // ------------------------------------------------------------------------------------------
 constexpr int kPolishPasses = 16;
 constexpr double kNull = 0x1p-80;             // 8e-25, in column norms
-constexpr float kNarrow = 1e-8f;              // largest column norm of E
 constexpr double kClose = 1e-5;               // relative distance of two squared norms
 
 // One CTA per column j of a sector: E(:, j) from the lower triangle of G (rows i >= 64 (j / 64)),
-// rotations by at most tan = 0.6, and none between two columns at or after cut[sector].  stat, four
-// words per sector: [0] columns with a pair above tol (those above tol / 10 turn too, by small angles),
-// [1] n - (first column of an unresolved pair: cos > 1e-3 and tan > 0.1), [2] largest squared column norm of
-// E as float bits, [3] nonzero: without `wide`, a pair above tol waits.
+// rotations by at most tan = 0.6, and none between two columns at or after cut[sector].  Close pairs (see
+// above) turn only with `wide`, by the cosine sums cos2 that a call without it has left (one value a column).
+// stat, four words per sector: [0] columns with a pair above tol (those above tol / 10 turn too, by small
+// angles), [1] n - (first column of an unresolved pair: cos > 1e-3 and tan > 0.1), [2] largest squared column
+// norm of E as float bits, [3] nonzero: there are close pairs above tol.
 struct PolCol {
     int sec, j;
 };
 __global__ void k_polish_angles(const SvdSec* __restrict__ secs, const PolCol* __restrict__ cols,
                                 const double* __restrict__ G, double* __restrict__ E, const int* __restrict__ cut,
-                                bool wide, unsigned* __restrict__ stat) {
+                                float* cos2, bool wide, unsigned* __restrict__ stat) {
     const PolCol pc = cols[blockIdx.x];
     const SvdSec s = secs[pc.sec];
     const int j = pc.j, n = s.n;
@@ -1559,8 +1561,9 @@ __global__ void k_polish_angles(const SvdSec* __restrict__ secs, const PolCol* _
     __syncthreads();
     const double null2 = kNull * kNull * __longlong_as_double(max(max(tops[0], tops[1]), max(tops[2], tops[3])));
     const double rjj = sqrt(gjj);
-    float sum = 0.f;
-    int above = 0, first = n, waits = 0;
+    cos2 += s.s_off;
+    float sum = 0.f, csum = 0.f;
+    int above = 0, first = n, close = 0;
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
         const int lo = min(i, j), hi = max(i, j);
         const double g = Gs[hi + (long long)lo * n], gii = Gs[i + (long long)i * n];
@@ -1573,9 +1576,14 @@ __global__ void k_polish_angles(const SvdSec* __restrict__ secs, const PolCol* _
             t = 1.0 / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
             if (t > 0.1 && fabs(g) > 1e-3 * size) first = min(first, lo);
             if (lo >= from) t = 0.0;
-            else if (t > 0.1 || fabs(gjj - gii) <= kClose * fmax(gii, gjj)) {
-                waits |= over && !wide;
-                t = !wide || (t > 0.1 && !over) ? 0.0 : fmin(t, 0.6);
+            else {
+                const float c = (float)(fabs(g) / size);
+                if (t > 0.1 || fabs(gjj - gii) <= kClose * fmax(gii, gjj)) {
+                    close |= over;
+                    t = wide && over && c > 1.5f * sqrtf(cos2[i] * cos2[j]) ? fmin(t, 0.6) : 0.0;
+                } else {
+                    csum = fmaf(c, c, csum);
+                }
             }
             if (zeta < 0.0 || (zeta == 0.0 && i > j)) t = -t;
             sum = fmaf((float)t, (float)t, sum);
@@ -1584,20 +1592,24 @@ __global__ void k_polish_angles(const SvdSec* __restrict__ secs, const PolCol* _
     }
     for (int o = 16; o > 0; o >>= 1) {
         sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        csum += __shfl_xor_sync(0xffffffffu, csum, o);
         first = min(first, __shfl_xor_sync(0xffffffffu, first, o));
     }
     above = __any_sync(0xffffffffu, above);
-    waits = __any_sync(0xffffffffu, waits);
-    __shared__ float ssum[4];
+    close = __any_sync(0xffffffffu, close);
+    __shared__ float ssum[4], scos[4];
     if ((threadIdx.x & 31) == 0) {
         ssum[threadIdx.x >> 5] = sum;
+        scos[threadIdx.x >> 5] = csum;
         if (above) atomicAdd(&stat[4 * pc.sec], 1u);
-        if (waits) atomicOr(&stat[4 * pc.sec + 3], 1u);
         if (first < n) atomicMax(&stat[4 * pc.sec + 1], (unsigned)(n - first));
+        if (close) atomicOr(&stat[4 * pc.sec + 3], 1u);
     }
     __syncthreads();
-    if (threadIdx.x == 0)
+    if (threadIdx.x == 0) {
         atomicMax(&stat[4 * pc.sec + 2], __float_as_uint(ssum[0] + ssum[1] + ssum[2] + ssum[3]));
+        if (!wide) cos2[j] = scos[0] + scos[1] + scos[2] + scos[3];
+    }
 }
 
 // X = scale E + a I over the sectors' n x n matrices (X may be E).
@@ -1625,7 +1637,7 @@ bool polish64(const std::vector<SvdSec>& ss, const SvdSec* dsecs, DBuf& dW, DBuf
     }
     *passes = 0;
     if (cols.empty()) return true;
-    DBuf dcols, G, E, X, Wn, Vn, norms, stat;
+    DBuf dcols, G, E, X, Wn, Vn, norms, cos2, stat;
     upload(dcols, cols, st);
     G.ensure(voff * 8, st);
     E.ensure(voff * 8, st);
@@ -1633,11 +1645,12 @@ bool polish64(const std::vector<SvdSec>& ss, const SvdSec* dsecs, DBuf& dW, DBuf
     Wn.ensure(woff * 8, st);
     Vn.ensure(voff * 8, st);
     norms.ensure(soff * 8, st);
+    cos2.ensure(soff * 4, st);
     stat.ensure((size_t)nsec * 16, st);
     std::vector<unsigned> hs((size_t)nsec * 4);
     std::vector<double> hd(soff);
     const unsigned nc = (unsigned)cols.size();
-    std::vector<int> cut(nsec);
+    std::vector<int> cut(nsec), sent;     // (sent: what dcut holds)
     DBuf dcut;
     int maxn = 1;
     for (const SvdSec& x : ss) maxn = std::max(maxn, x.n);
@@ -1655,10 +1668,13 @@ bool polish64(const std::vector<SvdSec>& ss, const SvdSec* dsecs, DBuf& dW, DBuf
     for (int pass = 0; pass < kPolishPasses; ++pass) {
         run_gemm64(gG, dW.as<double>(), dW.as<double>(), G.as<double>(), st);
         auto angles = [&](bool wide) {
-            upload(dcut, cut, st);
+            if (cut != sent) {
+                upload(dcut, cut, st);
+                sent = cut;
+            }
             PD_CK(cudaMemsetAsync(stat.p, 0, (size_t)nsec * 16, st));
             k_polish_angles<<<nc, 128, 0, st>>>(dsecs, dcols.as<PolCol>(), G.as<double>(), E.as<double>(),
-                                                dcut.as<int>(), wide, stat.as<unsigned>());
+                                                dcut.as<int>(), cos2.as<float>(), wide, stat.as<unsigned>());
             PD_LAUNCHED();
             PD_CK(cudaMemcpyAsync(hs.data(), stat.p, (size_t)nsec * 16, cudaMemcpyDeviceToHost, st));
             PD_CK(cudaStreamSynchronize(st));
@@ -1677,7 +1693,7 @@ bool polish64(const std::vector<SvdSec>& ss, const SvdSec* dsecs, DBuf& dW, DBuf
             for (int s = 0; s < nsec; ++s) cut[s] = ss[s].n - (int)hs[4 * s + 1];
             angles(false);
         }
-        bool finite = true, waits = false;
+        bool finite = true, close = false;
         auto largest = [&]() {
             float m = 0.f;
             for (int s = 0; s < nsec; ++s) {
@@ -1685,12 +1701,13 @@ bool polish64(const std::vector<SvdSec>& ss, const SvdSec* dsecs, DBuf& dW, DBuf
                 std::memcpy(&v, &hs[4 * s + 2], 4);
                 finite = finite && std::isfinite(v);
                 m = std::max(m, std::sqrt(v));
-                waits = waits || hs[4 * s + 3];
+                close = close || hs[4 * s + 3];
             }
             return m;
         };
-        float norm = largest();
-        if (finite && waits && norm <= kNarrow) {
+        const float narrow = largest();
+        float norm = narrow;
+        if (finite && close) {
             angles(true);
             norm = largest();
             // columns that all want large angles among themselves do not settle this way
@@ -1719,7 +1736,7 @@ bool polish64(const std::vector<SvdSec>& ss, const SvdSec* dsecs, DBuf& dW, DBuf
         std::swap(dV, Vn);
         // FP32 block Jacobi on the columns from the cut of every sector that has unresolved pairs, once the
         // rotations against the resolved columns have become small
-        if (!unresolved || norm > 0.05f) continue;
+        if (!unresolved || narrow > 0.05f) continue;
         --stages;
         launch_svd_norms<double>(dsecs, nsec, maxn, dW.as<double>(), norms.as<double>(), st);
         PD_CK(cudaMemcpyAsync(hd.data(), norms.p, (size_t)soff * 8, cudaMemcpyDeviceToHost, st));
