@@ -1543,7 +1543,8 @@ struct PolCol {
 };
 __global__ void k_polish_angles(const SvdSec* __restrict__ secs, const PolCol* __restrict__ cols,
                                 const double* __restrict__ G, double* __restrict__ E, const int* __restrict__ cut,
-                                float* cos2, bool wide, unsigned* __restrict__ stat) {
+                                float* cos2, bool wide, unsigned* __restrict__ stat, int nshared) {
+    extern __shared__ double diag[];               // G's diagonal, for sectors of up to nshared columns
     const PolCol pc = cols[blockIdx.x];
     const SvdSec s = secs[pc.sec];
     const int j = pc.j, n = s.n;
@@ -1555,7 +1556,11 @@ __global__ void k_polish_angles(const SvdSec* __restrict__ secs, const PolCol* _
     // squared norms are not negative: they order like their bits (NaN above all, and no floor then)
     __shared__ long long tops[4];
     long long top = 0;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) top = max(top, __double_as_longlong(Gs[i + (long long)i * n]));
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        const double gii = Gs[i + (long long)i * n];
+        top = max(top, __double_as_longlong(gii));
+        if (n <= nshared) diag[i] = gii;
+    }
     for (int o = 16; o > 0; o >>= 1) top = max(top, __shfl_xor_sync(0xffffffffu, top, o));
     if ((threadIdx.x & 31) == 0) tops[threadIdx.x >> 5] = top;
     __syncthreads();
@@ -1566,7 +1571,7 @@ __global__ void k_polish_angles(const SvdSec* __restrict__ secs, const PolCol* _
     int above = 0, first = n, close = 0;
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
         const int lo = min(i, j), hi = max(i, j);
-        const double g = Gs[hi + (long long)lo * n], gii = Gs[i + (long long)i * n];
+        const double g = Gs[hi + (long long)lo * n], gii = n <= nshared ? diag[i] : Gs[i + (long long)i * n];
         double t = 0.0;
         const double size = sqrt(gii) * rjj;
         if (i != j && fabs(g) > 0.1 * tol * size && !(fmin(gii, gjj) <= null2)) {
@@ -1654,6 +1659,7 @@ bool polish64(const std::vector<SvdSec>& ss, const SvdSec* dsecs, DBuf& dW, DBuf
     DBuf dcut;
     int maxn = 1;
     for (const SvdSec& x : ss) maxn = std::max(maxn, x.n);
+    const int nshared = std::min(maxn, 4096);
     int large = 0;                        // passes whose wide angles were large together
     int stages = 3;                       // FP32 passes over unresolved columns still allowed
     // false: too far from orthogonal; W and V are as before, for the scalar Jacobi to go on with
@@ -1673,8 +1679,8 @@ bool polish64(const std::vector<SvdSec>& ss, const SvdSec* dsecs, DBuf& dW, DBuf
                 sent = cut;
             }
             PD_CK(cudaMemsetAsync(stat.p, 0, (size_t)nsec * 16, st));
-            k_polish_angles<<<nc, 128, 0, st>>>(dsecs, dcols.as<PolCol>(), G.as<double>(), E.as<double>(),
-                                                dcut.as<int>(), cos2.as<float>(), wide, stat.as<unsigned>());
+            k_polish_angles<<<nc, 128, (size_t)nshared * 8, st>>>(dsecs, dcols.as<PolCol>(), G.as<double>(), E.as<double>(),
+                                                dcut.as<int>(), cos2.as<float>(), wide, stat.as<unsigned>(), nshared);
             PD_LAUNCHED();
             PD_CK(cudaMemcpyAsync(hs.data(), stat.p, (size_t)nsec * 16, cudaMemcpyDeviceToHost, st));
             PD_CK(cudaStreamSynchronize(st));
