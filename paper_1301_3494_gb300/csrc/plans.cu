@@ -1532,18 +1532,20 @@ constexpr int kPolishPasses = 16;
 constexpr double kNull = 0x1p-80;             // 8e-25, in column norms
 constexpr double kClose = 1e-5;               // relative distance of two squared norms
 
-// One CTA per column j of a sector: E(:, j) from the lower triangle of G (rows i >= 64 (j / 64)),
-// rotations by at most tan = 0.6, and none between two columns at or after cut[sector].  Close pairs (see
-// above) turn only with `wide`, by the cosine sums cos2 that a call without it has left (one value a column).
-// stat, four words per sector: [0] columns with a pair above tol (those above tol / 10 turn too, by small
-// angles), [1] n - (first column of an unresolved pair: cos > 1e-3 and tan > 0.1), [2] largest squared column
-// norm of E as float bits, [3] nonzero: there are close pairs above tol.
+// One CTA per column j of a sector: E(:, j) from the lower triangle of G (rows i >= 64 (j / 64)).  Pairs above
+// tol / 10 turn, close ones (see above) only above tol, and those are left to k_polish_take, as sign (2 + t).
+// cos2: the column's sum of squared cosines with the columns not close to it.  stat, four words per sector:
+// [0] columns with a pair above tol, [1] n - (first column of an unresolved pair: cos > 1e-3 and tan > 0.1),
+// [2] largest squared norm of a column of E without the close pairs, as float bits, [3] nonzero: there are
+// close pairs above tol.
+// A pair costs two roots and three divisions on the FP64 units, 1 to 2 ms a launch at an m = 2000 bond:
+// what depends on its result (the cut, the close pairs) reads E instead of working it out again.
 struct PolCol {
     int sec, j;
 };
-__global__ void k_polish_angles(const SvdSec* __restrict__ secs, const PolCol* __restrict__ cols,
-                                const double* __restrict__ G, double* __restrict__ E, const int* __restrict__ cut,
-                                float* cos2, bool wide, unsigned* __restrict__ stat, int nshared) {
+__global__ void __launch_bounds__(128)
+    k_polish_angles(const SvdSec* __restrict__ secs, const PolCol* __restrict__ cols, const double* __restrict__ G,
+                    double* __restrict__ E, float* __restrict__ cos2, unsigned* __restrict__ stat, int nshared) {
     extern __shared__ double diag[];               // G's diagonal, for sectors of up to nshared columns
     const PolCol pc = cols[blockIdx.x];
     const SvdSec s = secs[pc.sec];
@@ -1552,7 +1554,6 @@ __global__ void k_polish_angles(const SvdSec* __restrict__ secs, const PolCol* _
     double* Ej = E + s.v_off + (long long)j * n;
     const double gjj = Gs[j + (long long)j * n];
     const double tol = 4.0 * DBL_EPSILON * sqrt((double)s.p);
-    const int from = cut[pc.sec];
     // squared norms are not negative: they order like their bits (NaN above all, and no floor then)
     __shared__ long long tops[4];
     long long top = 0;
@@ -1566,7 +1567,6 @@ __global__ void k_polish_angles(const SvdSec* __restrict__ secs, const PolCol* _
     __syncthreads();
     const double null2 = kNull * kNull * __longlong_as_double(max(max(tops[0], tops[1]), max(tops[2], tops[3])));
     const double rjj = sqrt(gjj);
-    cos2 += s.s_off;
     float sum = 0.f, csum = 0.f;
     int above = 0, first = n, close = 0;
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
@@ -1580,18 +1580,15 @@ __global__ void k_polish_angles(const SvdSec* __restrict__ secs, const PolCol* _
             const double zeta = (gjj - gii) / (2.0 * g);
             t = 1.0 / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
             if (t > 0.1 && fabs(g) > 1e-3 * size) first = min(first, lo);
-            if (lo >= from) t = 0.0;
-            else {
+            if (t > 0.1 || fabs(gjj - gii) <= kClose * fmax(gii, gjj)) {
+                close |= over;
+                t = over ? 2.0 + t : 0.0;
+            } else {
                 const float c = (float)(fabs(g) / size);
-                if (t > 0.1 || fabs(gjj - gii) <= kClose * fmax(gii, gjj)) {
-                    close |= over;
-                    t = wide && over && c > 1.5f * sqrtf(cos2[i] * cos2[j]) ? fmin(t, 0.6) : 0.0;
-                } else {
-                    csum = fmaf(c, c, csum);
-                }
+                csum = fmaf(c, c, csum);
+                sum = fmaf((float)t, (float)t, sum);
             }
             if (zeta < 0.0 || (zeta == 0.0 && i > j)) t = -t;
-            sum = fmaf((float)t, (float)t, sum);
         }
         Ej[i] = t;
     }
@@ -1613,7 +1610,55 @@ __global__ void k_polish_angles(const SvdSec* __restrict__ secs, const PolCol* _
     __syncthreads();
     if (threadIdx.x == 0) {
         atomicMax(&stat[4 * pc.sec + 2], __float_as_uint(ssum[0] + ssum[1] + ssum[2] + ssum[3]));
-        if (!wide) cos2[j] = scos[0] + scos[1] + scos[2] + scos[3];
+        cos2[s.s_off + j] = scos[0] + scos[1] + scos[2] + scos[3];
+    }
+}
+
+// What of E turns: no pair of two columns at or after cut[sector]; a close pair, by tan = 0.6 at most, where
+// its cosine is above 1.5 times what the others explain.  norms, two words per sector (float bits): largest
+// squared norm of a column of E without the close pairs and with them.
+__global__ void __launch_bounds__(128)
+    k_polish_take(const SvdSec* __restrict__ secs, const PolCol* __restrict__ cols, const double* __restrict__ G,
+                  double* __restrict__ E, const int* __restrict__ cut, const float* __restrict__ cos2,
+                  unsigned* __restrict__ norms) {
+    const PolCol pc = cols[blockIdx.x];
+    const SvdSec s = secs[pc.sec];
+    const int j = pc.j, n = s.n, from = cut[pc.sec];
+    const double* Gs = G + s.v_off;
+    double* Ej = E + s.v_off + (long long)j * n;
+    cos2 += s.s_off;
+    float narrow = 0.f, all = 0.f;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        const double e = Ej[i];
+        double t = e;
+        const int lo = min(i, j), hi = max(i, j);
+        if (lo >= from) {
+            t = 0.0;
+        } else if (fabs(e) > 1.0) {
+            const double c = fabs(Gs[hi + (long long)lo * n]) /
+                             (sqrt(Gs[lo + (long long)lo * n]) * sqrt(Gs[hi + (long long)hi * n]));
+            t = c > (double)(1.5f * sqrtf(cos2[i] * cos2[j])) ? copysign(fmin(fabs(e) - 2.0, 0.6), e) : 0.0;
+            all = fmaf((float)t, (float)t, all);
+        } else {
+            narrow = fmaf((float)t, (float)t, narrow);
+        }
+        if (t != e) Ej[i] = t;
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        narrow += __shfl_xor_sync(0xffffffffu, narrow, o);
+        all += __shfl_xor_sync(0xffffffffu, all, o);
+    }
+    __shared__ float sn[4], sa[4];
+    if ((threadIdx.x & 31) == 0) {
+        sn[threadIdx.x >> 5] = narrow;
+        sa[threadIdx.x >> 5] = all;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        narrow = (sn[0] + sn[1]) + (sn[2] + sn[3]);
+        all = narrow + ((sa[0] + sa[1]) + (sa[2] + sa[3]));
+        atomicMax(&norms[2 * pc.sec], __float_as_uint(narrow));
+        atomicMax(&norms[2 * pc.sec + 1], __float_as_uint(all));
     }
 }
 
@@ -1651,11 +1696,11 @@ bool polish64(const std::vector<SvdSec>& ss, const SvdSec* dsecs, DBuf& dW, DBuf
     Vn.ensure(voff * 8, st);
     norms.ensure(soff * 8, st);
     cos2.ensure(soff * 4, st);
-    stat.ensure((size_t)nsec * 16, st);
+    stat.ensure((size_t)nsec * 24, st);
     std::vector<unsigned> hs((size_t)nsec * 4);
     std::vector<double> hd(soff);
     const unsigned nc = (unsigned)cols.size();
-    std::vector<int> cut(nsec), sent;     // (sent: what dcut holds)
+    std::vector<int> cut(nsec);
     DBuf dcut;
     int maxn = 1;
     for (const SvdSec& x : ss) maxn = std::max(maxn, x.n);
@@ -1673,51 +1718,45 @@ bool polish64(const std::vector<SvdSec>& ss, const SvdSec* dsecs, DBuf& dW, DBuf
     };
     for (int pass = 0; pass < kPolishPasses; ++pass) {
         run_gemm64(gG, dW.as<double>(), dW.as<double>(), G.as<double>(), st);
-        auto angles = [&](bool wide) {
-            if (cut != sent) {
-                upload(dcut, cut, st);
-                sent = cut;
-            }
-            PD_CK(cudaMemsetAsync(stat.p, 0, (size_t)nsec * 16, st));
-            k_polish_angles<<<nc, 128, (size_t)nshared * 8, st>>>(dsecs, dcols.as<PolCol>(), G.as<double>(), E.as<double>(),
-                                                dcut.as<int>(), cos2.as<float>(), wide, stat.as<unsigned>(), nshared);
-            PD_LAUNCHED();
-            PD_CK(cudaMemcpyAsync(hs.data(), stat.p, (size_t)nsec * 16, cudaMemcpyDeviceToHost, st));
-            PD_CK(cudaStreamSynchronize(st));
-        };
-        for (int s = 0; s < nsec; ++s) cut[s] = ss[s].n;
-        angles(false);
-        bool unresolved = false, above = false;
+        PD_CK(cudaMemsetAsync(stat.p, 0, (size_t)nsec * 24, st));
+        k_polish_angles<<<nc, 128, (size_t)nshared * 8, st>>>(dsecs, dcols.as<PolCol>(), G.as<double>(), E.as<double>(),
+                                                              cos2.as<float>(), stat.as<unsigned>(), nshared);
+        PD_LAUNCHED();
+        PD_CK(cudaMemcpyAsync(hs.data(), stat.p, (size_t)nsec * 16, cudaMemcpyDeviceToHost, st));
+        PD_CK(cudaStreamSynchronize(st));
+        bool unresolved = false, above = false, close = false, finite = true;
         for (int s = 0; s < nsec; ++s) {
             above = above || hs[4 * s] > 0;
             unresolved = unresolved || (stages > 0 && hs[4 * s + 1] > 0);
+            close = close || hs[4 * s + 3] > 0;
         }
         if (!above) return true;
         *passes = pass + 1;
-        if (unresolved) {
-            // the unresolved columns turn against the others only
-            for (int s = 0; s < nsec; ++s) cut[s] = ss[s].n - (int)hs[4 * s + 1];
-            angles(false);
-        }
-        bool finite = true, close = false;
-        auto largest = [&]() {
+        auto largest = [&](int first, int step) {          // of squared norms
             float m = 0.f;
             for (int s = 0; s < nsec; ++s) {
                 float v;
-                std::memcpy(&v, &hs[4 * s + 2], 4);
+                std::memcpy(&v, &hs[first + step * s], 4);
                 finite = finite && std::isfinite(v);
                 m = std::max(m, std::sqrt(v));
-                close = close || hs[4 * s + 3];
             }
             return m;
         };
-        const float narrow = largest();
-        float norm = narrow;
-        if (finite && close) {
-            angles(true);
-            norm = largest();
+        float narrow = largest(2, 4), norm = narrow;       // of E without close pairs, and with them
+        if (unresolved || close) {
+            // the unresolved columns turn against the others only
+            for (int s = 0; s < nsec; ++s) cut[s] = ss[s].n - (unresolved ? (int)hs[4 * s + 1] : 0);
+            upload(dcut, cut, st);
+            unsigned* norms2 = stat.as<unsigned>() + 4 * nsec;
+            k_polish_take<<<nc, 128, 0, st>>>(dsecs, dcols.as<PolCol>(), G.as<double>(), E.as<double>(), dcut.as<int>(),
+                                              cos2.as<float>(), norms2);
+            PD_LAUNCHED();
+            PD_CK(cudaMemcpyAsync(hs.data(), norms2, (size_t)nsec * 8, cudaMemcpyDeviceToHost, st));
+            PD_CK(cudaStreamSynchronize(st));
+            narrow = largest(0, 2);
+            norm = largest(1, 2);
             // columns that all want large angles among themselves do not settle this way
-            if (norm > 0.6f && !unresolved && (norm > 1.2f || ++large > 2)) return false;
+            if (close && norm > 0.6f && !unresolved && (norm > 1.2f || ++large > 2)) return false;
         }
         if (!finite) return false;
         // E <- Q - I
