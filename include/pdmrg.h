@@ -103,9 +103,9 @@ typedef struct {
                                (dmrg_gemm64 mode 1); batches outside its K limit, and those too
                                small to gain from it, stay on the FP64 units: below 1 GFLOP
                                where a plan is run many times (a Davidson's matvec, the
-                               measurements of one state), below 6 GFLOP elsewhere.  2 = every
-                               batch inside the K limit, whatever its size.  0 = FP64 units
-                               throughout.                                                      */
+                               passes of an FP64 split, the measurements of one state),
+                               below 6 GFLOP elsewhere.  2 = every batch inside the K limit,
+                               whatever its size.  0 = FP64 units throughout.                   */
     int svd_plain_jacobi;   /* 1 = every split's one-sided Jacobi runs on the sector matrix W
                                itself; 0 (default) = on R^T from a Householder QR W = QR (a
                                few sweeps instead of many; sectors taller than the QR panel's

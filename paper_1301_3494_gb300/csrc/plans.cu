@@ -166,7 +166,7 @@ void GemmBatch::stage_f64(ListPack& pk) {
 // Whether a batch runs emulated.  Its plan is built on the host (one to several ms for the batches of a
 // bond) and a run is seven launches and two host waits around the slice products, so it only pays for
 // large batches, or for middling ones whose plan is run many times.  Size and that hint (a Davidson's
-// matvec, a kept measurement plan) decide, never the history of a batch: the two arithmetics round
+// matvec, a polish, a kept measurement plan) decide, never the history of a batch: the two arithmetics round
 // differently, and one operator must not change between its applications.  Measured, FP64 units against
 // a first emulated run / a repeated one:
 //   17 of 320 x 320 x 640 (2.2 GFLOP)        2.1 ms,  2.0 / 1.0 ms
@@ -1677,6 +1677,7 @@ bool polish64(const std::vector<SvdSec>& ss, const SvdSec* dsecs, DBuf& dW, DBuf
     const int nsec = (int)ss.size();
     std::vector<PolCol> cols;
     GemmBatch gG, gW, gV, gE;
+    gG.repeated = gW.repeated = gV.repeated = true;    // once a pass, five to ten passes
     for (int s = 0; s < nsec; ++s) {
         const SvdSec& x = ss[s];
         for (int j = 0; j < x.n; ++j) cols.push_back({s, j});
