@@ -1514,10 +1514,11 @@ void fp64_precondition(const std::vector<SvdSec>& ss, const SvdSec* dsecs, DBuf&
 // between exactly degenerate columns are not even wanted: their cosines are the products of those with the
 // other columns and vanish with them.  So a pair of nearly equal columns turns only where its cosine is
 // above the tolerance and above what the others explain (the root of the product of the two columns' sums of
-// squared cosines), and a cluster of five or more columns goes to the scalar Jacobi at once.  A 200 x 200 matrix of two values:
-// 13.2 ms with all angles taken together (and the scalar Jacobi after), 2.8 now, 14.6 by the scalar Jacobi
-// alone; 300 values 1e-9 apart, which only that one settles: 57.3, 55.1 and 55.7.  (Waiting for all small
-// angles instead costs passes where a few pairs are close: 7 to 15 for 5 or 6 at an FP64 m = 2000 bond.)
+// squared cosines), and a cluster of five or more columns goes to the scalar Jacobi at once.  A 200 x 200
+// matrix of two values: 13.2 ms with all angles taken together (and the scalar Jacobi after), 2.8 now, 14.6
+// by the scalar Jacobi alone; 300 values 1e-9 apart, which only that one settles: 57.3, 54.8 and 55.7.
+// (Waiting for all small angles instead costs passes where a few pairs are close: 7 to 15 for 5 or 6 at an
+// FP64 m = 2000 bond.)
 // Columns below kNull of the sector's largest are finished: W V was formed in FP64, so a column that is
 // not zero in exact arithmetic does not come out below rounding, 1e-16 of the largest, and one that is (an
 // exactly low-rank matrix: its columns are multiples of each other, bit for bit) falls by that factor in
